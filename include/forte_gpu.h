@@ -479,11 +479,11 @@ int forte_sci_set_stream(forte_sci *sci, void *cuda_stream);
  *         a word listed twice counts twice
  *   C, S  device [nvec][ndet] FP64; S overwritten, must not overlap C
  *   ndet >= 0 (<= 2^31), nvec >= 0; 0 is a no-op
- * Every pair (i, j) is screened by popcount(D_i ^ D_j) <= 4 (cost ndet^2 / 32
- * warp steps), so the call suits lists up to ~1e6 determinants.  Deterministic:
- * per-row sums are taken in list order within fixed splits, added in split order.
- * Asynchronous on the handle's stream; grows a scratch buffer (nvec <= 4 at a time
- * x splits x ndet doubles) on demand. */
+ * Every pair (i, j) is screened (32 pairs a logic operation and occupied orbital; cost
+ * ndet^2), so the call suits lists up to ~1e6 determinants.  Deterministic: the order
+ * of a row's sum follows from the list alone.
+ * Asynchronous on the handle's stream; grows a scratch buffer (65 bits a determinant)
+ * on demand. */
 int forte_sci_sigma(forte_sci *sci, long long ndet, const uint64_t *dets, const double *C, double *S, int nvec);
 
 #ifdef __cplusplus
