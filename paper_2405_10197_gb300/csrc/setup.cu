@@ -189,6 +189,49 @@ int build_spin_tables(forte_ctx *ctx) {
   return build_one_spin(ctx, ctx->sh[1], ctx->nb);
 }
 
+// off[I]: the replacements of string I that move an electron, dealt round-robin from 16
+// buckets of pair mod 16 (list order within a bucket).  One thread per string.
+__global__ void k_off_list(const Repl *__restrict__ list, int nk, int nko, int N, uint32_t *__restrict__ off) {
+  const int I = blockIdx.x * blockDim.x + threadIdx.x;
+  if (I >= N) return;
+  int cnt[16], seen[16];
+  for (int b = 0; b < 16; ++b) cnt[b] = seen[b] = 0;
+  const Repl *L = list + (long long)I * nk;
+  for (int e = 0; e < nk; ++e)
+    if (L[e].J != I) ++cnt[L[e].pair & 15];
+  for (int e = 0; e < nk; ++e) {
+    const Repl r = L[e];
+    if (r.J == I) continue;
+    const int b = r.pair & 15, k = seen[b]++;
+    int at = 0;
+    for (int c = 0; c < 16; ++c) at += min(cnt[c], k) + (c < b && cnt[c] > k ? 1 : 0);
+    off[(long long)I * nko + at] = (uint32_t)r.J | ((uint32_t)r.pair << 16) | (r.sgn < 0 ? 0x80000000u : 0u);
+  }
+}
+
+// W[pq][j] = sum of (pq|rr) over the orbitals r of string j.
+__global__ void k_occ_sums(const double *__restrict__ gpair, int np, const uint32_t *__restrict__ str, int N,
+                           double *__restrict__ W) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (long long)np * N) return;
+  const double *g = gpair + i / N * np;
+  double v = 0.0;
+  for (uint32_t m = str[i % N]; m; m &= m - 1) {
+    const int r = __ffs((int)m) - 1;
+    v += g[r * (r + 1) / 2 + r];
+  }
+  W[i] = v;
+}
+
+bool sigma_small(const forte_ctx *ctx) {
+  const SpinHost &A = ctx->sh[0], &B = ctx->sh[ctx->same_strings ? 0 : 1];
+  const long long k = A.nel * (ctx->n - A.nel) + 1;
+  if (8 * k * (B.N + ctx->npair) > 100 * 1024) return false;
+  for (long long j = 0; j < B.N; ++j)  // rows of one length (they are, for string Hamiltonians)
+    if (B.csr_ptr[j + 1] - B.csr_ptr[j] != B.csr_ptr[1]) return false;
+  return true;
+}
+
 template <typename T>
 static int upload(T **dst, const T *src, size_t count) {
   size_t bytes = sizeof(T) * (count ? count : 1);
@@ -223,14 +266,13 @@ int upload_tables(forte_ctx *ctx) {
         dense[(size_t)I * n2 + r.pq] = (r.J << 1) | (r.sgn < 0 ? 1 : 0);
       }
     if ((st = upload(&D.dense, dense.data(), dense.size()))) return st;
-    if (H.N <= 65536) {
-      std::vector<uint32_t> l4(H.list.size());
-      for (size_t i = 0; i < l4.size(); ++i) {
-        const Repl &r = H.list[i];
-        l4[i] = (uint32_t)r.J | ((uint32_t)r.pair << 16) | (r.sgn < 0 ? 0x80000000u : 0u);
-      }
-      if ((st = upload(&D.list4, l4.data(), l4.size()))) return st;
+    const int nko = H.nel * (n - H.nel);
+    if (cudaMalloc(&D.off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)H.N * nko)) != cudaSuccess) {
+      set_error("cudaMalloc of the replacement lists failed");
+      return FORTE_ERR_ALLOC;
     }
+    k_off_list<<<(unsigned)((H.N + 63) / 64), 64>>>(D.list, H.nk, nko, (int)H.N, D.off);
+    FORTE_LAUNCH_CHECK();
     if (H.N < 16384 && ctx->npair <= 128) {
       std::vector<uint16_t> tab((size_t)H.N * 128, 0xFFFFu);
       for (long long J = 0; J < H.N; ++J)
@@ -253,6 +295,29 @@ int upload_tables(forte_ctx *ctx) {
               ctx->eri[(((size_t)p * n + q) * n + r) * n + s];
   int st;
   if ((st = upload(&ctx->d_gpair, gp.data(), gp.size()))) return st;
+  {
+    const SpinHost &B = ctx->sh[ctx->same_strings ? 0 : 1];
+    if (cudaMalloc(&ctx->d_W, sizeof(double) * (size_t)np * B.N) != cudaSuccess) {
+      set_error("cudaMalloc of the occupation sums failed");
+      return FORTE_ERR_ALLOC;
+    }
+    k_occ_sums<<<(unsigned)(((long long)np * B.N + 255) / 256), 256>>>(ctx->d_gpair, np, ctx->sd[1].str, (int)B.N,
+                                                                      ctx->d_W);
+    FORTE_LAUNCH_CHECK();
+    // (default stream, like the copies here; hdiag_build waits for it before create returns)
+    if (sigma_small(ctx)) {
+      const long long nnz = B.csr_ptr[1];
+      std::vector<int> col((size_t)nnz * B.N);
+      std::vector<double> val((size_t)nnz * B.N);
+      for (long long j = 0; j < B.N; ++j)
+        for (long long e = 0; e < nnz; ++e) {
+          col[(size_t)e * B.N + j] = B.csr_col[B.csr_ptr[j] + e];
+          val[(size_t)e * B.N + j] = B.csr_val[B.csr_ptr[j] + e];
+        }
+      if ((st = upload(&ctx->sd[1].ell_col, col.data(), col.size()))) return st;
+      if ((st = upload(&ctx->sd[1].ell_val, val.data(), val.size()))) return st;
+    }
+  }
   std::vector<float> gp32(gp.begin(), gp.end());
   if ((st = upload(&ctx->d_gpair32, gp32.data(), gp32.size()))) return st;
   return FORTE_OK;

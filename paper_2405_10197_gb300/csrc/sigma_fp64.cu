@@ -90,64 +90,294 @@ __global__ void k_transpose(const T *__restrict__ X, T *__restrict__ Y, long lon
   }
 }
 
-constexpr int AB_THREADS = 256;
+// ---- alpha-beta term, FP64 and double-FP32 ------------------------------------
+//
+// sigma[Ia, E_rs Jb] += s F[rs][Jb], F[rs][Jb] = sum_e s_e (pq_e|rs) C[J_e, Jb].
+// The replacements that move no electron are taken together: all of Ia's read the row
+// C[Ia] and all of Jb's write Jb, so they make one row (integrals summed over the
+// orbitals of Ia) and one output (integrals summed over those of Jb, d_W).  At 7 of 14
+// orbitals 50 x 50 instead of 56 x 56 products a determinant.
+// One GB300 (kernel): FP64 CAS(12,12), 4 vectors 13.2 -> 8.9 ms; double-FP32 CAS(13; 7,5)
+// 4.06 -> 3.03 ms.
+//
+// Shared memory: G[nk][npair] signed integral rows (row 0: the unmoved ones), row[NB] the
+// output row, D[nk][TJ] gathered rows of C.  A thread takes one (string, replacement)
+// of the tile at a time; the entry order of SpinDev::off gives the lanes' integral
+// loads different banks.
+struct AbF64 {  // bound by the FP64 pipe (2 DFMA per clock and SM)
+  using E = double;
+  static constexpr int THREADS = 256, TJ = 64;
+  double a = 0.0;
+  __device__ __forceinline__ void fma(E x, E y) { a = ::fma(x, y, a); }
+  __device__ __forceinline__ double value() const { return a; }
+  static __device__ __forceinline__ E make(double x) { return x; }
+  static __device__ __forceinline__ E neg(E x) { return -x; }
+};
 
-// sigma_ab for one alpha string Ia (blockIdx.x) and one vector (blockIdx.y).
-// Shared memory: Gs[nkA][npair] signed integral rows, srow[NB] output row,
-// D[nkA][TJ] gathered C rows, Lb[TJ][nkB] beta replacement lists of the tile.
-__global__ void __launch_bounds__(AB_THREADS) k_ab_fp64(const Repl *__restrict__ listA, int nkA,
-                                                        const Repl *__restrict__ listB, int nkB,
-                                                        long long NB, const double *__restrict__ gpair,
-                                                        int npair, const double *__restrict__ C,
-                                                        double *__restrict__ S, long long vstride,
-                                                        int TJ) {
-  extern __shared__ double smem[];
-  double *Gs = smem;                                  // nkA * npair
-  double *srow = Gs + (size_t)nkA * npair;            // NB
-  double *D = srow + NB;                              // nkA * TJ
-  Repl *Lb = reinterpret_cast<Repl *>(D + (size_t)nkA * TJ);  // TJ * nkB
+template <class OP>
+__global__ void __launch_bounds__(OP::THREADS) k_ab(const Repl *__restrict__ listA, int nkA,
+                                                    const uint32_t *__restrict__ offA, int noA,
+                                                    const uint32_t *__restrict__ offB, int noB, long long NB,
+                                                    const double *__restrict__ gpair,
+                                                    const typename OP::E *__restrict__ gE,
+                                                    const typename OP::E *__restrict__ W, int npair,
+                                                    const typename OP::E *__restrict__ C, double *__restrict__ S,
+                                                    long long vstride, int TJ) {
+  using E = typename OP::E;
+  constexpr int NT = OP::THREADS;
+  extern __shared__ double ab_smem[];
+  const int nk = noA + 1;
+  double *row = ab_smem;                            // NB
+  E *G = reinterpret_cast<E *>(row + NB);           // nk * npair
+  E *D = G + (size_t)nk * npair;                    // nk * TJ
+  __shared__ int s_J[80], s_pp[16];                 // C rows; pair indices of Ia's unmoved replacements
+  __shared__ int s_np;
   const long long Ia = blockIdx.x;
-  const double *Cv = C + (long long)blockIdx.y * vstride;
+  const E *Cv = C + (long long)blockIdx.y * vstride;
   double *Sv = S + (long long)blockIdx.y * vstride;
-  const Repl *la = listA + Ia * nkA;
-  __shared__ int s_J[80];
-  for (int e = threadIdx.x; e < nkA; e += AB_THREADS) s_J[e] = la[e].J;
-  for (int i = threadIdx.x; i < nkA * npair; i += AB_THREADS) {
-    int e = i / npair, rs = i % npair;
-    Repl r = la[e];
-    Gs[i] = r.sgn * gpair[(size_t)r.pair * npair + rs];
+  const uint32_t *la = offA + Ia * noA;
+  for (int e = threadIdx.x; e < noA; e += NT) s_J[e + 1] = la[e] & 0xFFFFu;
+  if (threadIdx.x == 0) {
+    s_J[0] = (int)Ia;
+    int m = 0;
+    for (int e = 0; e < nkA; ++e)
+      if (listA[Ia * nkA + e].J == Ia) s_pp[m++] = listA[Ia * nkA + e].pair;
+    s_np = m;
   }
-  for (long long i = threadIdx.x; i < NB; i += AB_THREADS) srow[i] = 0.0;
+  for (int i = threadIdx.x; i < noA * npair; i += NT) {
+    const uint32_t w = la[i / npair];
+    const E g = gE[(size_t)((w >> 16) & 0xFFu) * npair + i % npair];
+    G[npair + i] = (w >> 31) ? OP::neg(g) : g;
+  }
+  for (long long i = threadIdx.x; i < NB; i += NT) row[i] = 0.0;
   __syncthreads();
+  const int npp = s_np;
+  for (int rs = threadIdx.x; rs < npair; rs += NT) {
+    double v = 0.0;
+    for (int m = 0; m < npp; ++m) v += gpair[(size_t)s_pp[m] * npair + rs];
+    G[rs] = OP::make(v);
+  }
   for (long long j0 = 0; j0 < NB; j0 += TJ) {
     const int tj = (int)min((long long)TJ, NB - j0);
-    for (int i = threadIdx.x; i < nkA * tj; i += AB_THREADS) {
-      int e = i / tj, j = i % tj;
+    for (int i = threadIdx.x; i < nk * tj; i += NT) {
+      const int e = i / tj, j = i - e * tj;
       D[e * TJ + j] = Cv[(long long)s_J[e] * NB + j0 + j];
     }
-    for (int i = threadIdx.x; i < tj * nkB; i += AB_THREADS) Lb[i] = listB[j0 * nkB + i];
     __syncthreads();
-    const int npairs_tile = tj * nkB;
-    for (int w = threadIdx.x; w < npairs_tile; w += AB_THREADS) {
-      const int j = w / nkB;
-      const Repl rf = Lb[w];
-      const double *g = Gs + rf.pair;
-      const double *d = D + j;
-      double acc = 0.0;
+    const uint32_t *lb = offB + j0 * noB;
+    for (int w = threadIdx.x; w < tj * noB; w += NT) {
+      const uint32_t f = lb[w];
+      const E *g = G + ((f >> 16) & 0xFFu), *d = D + w / noB;
+      OP acc;
 #pragma unroll 8
-      for (int e = 0; e < nkA; ++e) acc += g[e * npair] * d[e * TJ];
-      atomicAdd(&srow[rf.J], rf.sgn * acc);
+      for (int e = 0; e < nk; ++e) acc.fma(g[e * npair], d[e * TJ]);
+      const double v = acc.value();
+      atomicAdd(&row[f & 0xFFFFu], (f >> 31) ? -v : v);
+    }
+    // the unmoved replacements of the tile's strings: output j itself, rows split over
+    // the threads
+    const int parts = NT / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
+    if (part < parts && j < tj) {
+      OP acc;
+      for (int e = 1 + part; e < nk; e += parts) {
+        const uint32_t w = la[e - 1];
+        const E x = W[(size_t)((w >> 16) & 0xFFu) * NB + j0 + j];
+        acc.fma((w >> 31) ? OP::neg(x) : x, D[e * TJ + j]);
+      }
+      for (int m = part; m < npp; m += parts) acc.fma(W[(size_t)s_pp[m] * NB + j0 + j], D[j]);
+      atomicAdd(&row[j0 + j], acc.value());
     }
     __syncthreads();
   }
-  for (long long i = threadIdx.x; i < NB; i += AB_THREADS) Sv[Ia * NB + i] += srow[i];
+  for (long long i = threadIdx.x; i < NB; i += NT) Sv[Ia * NB + i] += row[i];
 }
 
-static size_t ab_smem_bytes(int nkA, int nkB, int npair, long long NB, int TJ) {
-  return sizeof(double) * ((size_t)nkA * npair + NB + (size_t)nkA * TJ) + sizeof(Repl) * (size_t)TJ * nkB;
+// Launch of k_ab; the tile narrows until the block fits.
+template <class OP>
+static int ab_launch(forte_ctx *ctx, const char *name, const typename OP::E *gE, const typename OP::E *W,
+                     const typename OP::E *C, double *S, int nvec) {
+  const int n = ctx->n, nkA = ctx->sh[0].nk, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
+  const long long NA = ctx->Na, NB = ctx->Nb;
+  auto bytes = [&](int TJ) {
+    return sizeof(double) * (size_t)NB + sizeof(typename OP::E) * ((size_t)(noA + 1) * (ctx->npair + TJ));
+  };
+  int TJ = OP::TJ;
+  while (bytes(TJ) > 220 * 1024 && TJ > 8) TJ /= 2;
+  if (bytes(TJ) > 220 * 1024) {
+    set_error("alpha-beta kernel %s needs %zu bytes of shared memory", name, bytes(TJ));
+    return FORTE_ERR_ARG;
+  }
+  FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab<OP>));
+  FORTE_PROF(ctx, name);
+  k_ab<OP><<<dim3((unsigned)NA, (unsigned)nvec), OP::THREADS, bytes(TJ), ctx->stream>>>(
+      ctx->sd[0].list, nkA, ctx->sd[0].off, noA, ctx->sd[1].off, noB, NB, ctx->d_gpair, gE, W, ctx->npair, C, S,
+      ctx->Ndet, TJ);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+
+// ---- small spaces (sigma_small) ------------------------------------------------
+//
+// Up to about 10 orbitals a sigma is a few microseconds of FP64 work, so the launches,
+// the idle SMs and the latency of their chains count.  Every output is gathered by a few
+// threads that split its sum and add their parts in a fixed order: no transposes, no
+// atomics, and enough blocks for every SM.  One GB300, CAS(8,8), one vector: 53 -> 25 us
+// (the general kernels: a 70-block grid, 21 us for the alpha-beta term alone).
+
+constexpr int SM_THREADS = 256;
+
+// Sum over the `parts` thread groups of a block of their values for column i of CH.
+__device__ __forceinline__ double sm_sum(double v, double *red, int CH, int parts) {
+  red[threadIdx.x] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x < CH)
+    for (int p = 0; p < parts; ++p) t += red[p * CH + threadIdx.x];
+  return t;
+}
+
+// Alpha-alpha (ALPHA: S = H_aa C) or beta-beta (S += C H_bb) part of row blockIdx.y,
+// columns blockIdx.x * CH .., vector blockIdx.z.
+template <bool ALPHA>
+__global__ void __launch_bounds__(SM_THREADS) k_ss_small(const int *__restrict__ ptr, const int *__restrict__ col,
+                                                         const double *__restrict__ val, int nnz,
+                                                         const double *__restrict__ C, double *__restrict__ S,
+                                                         long long NB, long long vstride, int CH) {
+  __shared__ double red[SM_THREADS];
+  const int parts = SM_THREADS / CH, part = threadIdx.x / CH;
+  const long long Ia = blockIdx.y, Ib = (long long)blockIdx.x * CH + threadIdx.x % CH;
+  const double *Cv = C + (long long)blockIdx.z * vstride;
+  double a = 0.0;
+  if (Ib < NB) {
+    if (ALPHA) {
+      const int b = ptr[Ia], e = ptr[Ia + 1];
+#pragma unroll 4
+      for (int k = b + part; k < e; k += parts) a = fma(val[k], Cv[(long long)col[k] * NB + Ib], a);
+    } else {
+      const double *Cr = Cv + Ia * NB;
+#pragma unroll 4
+      for (int k = part; k < nnz; k += parts) a = fma(val[k * NB + Ib], Cr[col[k * NB + Ib]], a);
+    }
+  }
+  a = sm_sum(a, red, CH, parts);
+  if (threadIdx.x < CH && Ib < NB) {
+    double *s = S + (long long)blockIdx.z * vstride + Ia * NB + Ib;
+    *s = ALPHA ? a : *s + a;
+  }
+}
+
+// Alpha-beta part of row blockIdx.y: D holds the rows C[J_e] whole, G the signed
+// integrals, so that output Ib gathers F[rs][J] from every replacement J of Ib.
+__global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict__ listA, int nkA,
+                                                         const uint32_t *__restrict__ offA, int noA,
+                                                         const uint32_t *__restrict__ offB, int noB, int NB,
+                                                         const double *__restrict__ gpair, const double *__restrict__ W,
+                                                         int npair, const double *__restrict__ C,
+                                                         double *__restrict__ S, long long vstride, int CH) {
+  extern __shared__ double ab_smem[];
+  __shared__ double red[SM_THREADS];
+  __shared__ int s_pp[16], s_np;
+  const int nk = noA + 1;
+  double *G = ab_smem, *D = G + nk * npair;  // [nk][npair], [nk][NB]
+  const int Ia = blockIdx.y;
+  const double *Cv = C + (long long)blockIdx.z * vstride;
+  const uint32_t *la = offA + (long long)Ia * noA;
+  if (threadIdx.x == 0) {
+    int m = 0;
+    for (int e = 0; e < nkA; ++e) {
+      const Repl r = listA[(long long)Ia * nkA + e];
+      if (r.J == Ia) s_pp[m++] = r.pair;
+    }
+    s_np = m;
+  }
+  for (int i = threadIdx.x; i < noA * npair; i += SM_THREADS) {
+    const uint32_t w = la[i / npair];
+    const double g = gpair[((w >> 16) & 0xFFu) * npair + i % npair];
+    G[npair + i] = (w >> 31) ? -g : g;
+  }
+  for (int i = threadIdx.x; i < nk * NB; i += SM_THREADS) {
+    const int e = i / NB;
+    D[i] = Cv[(long long)(e ? (int)(la[e - 1] & 0xFFFFu) : Ia) * NB + (i - e * NB)];
+  }
+  __syncthreads();
+  const int npp = s_np;
+  for (int rs = threadIdx.x; rs < npair; rs += SM_THREADS) {
+    double v = 0.0;
+    for (int m = 0; m < npp; ++m) v += gpair[s_pp[m] * npair + rs];
+    G[rs] = v;
+  }
+  __syncthreads();
+  const int parts = SM_THREADS / CH, part = threadIdx.x / CH;
+  const int Ib = blockIdx.x * CH + threadIdx.x % CH;
+  double out = 0.0;
+  if (Ib < NB) {
+    const uint32_t *lb = offB + (long long)Ib * noB;
+    for (int f = part; f < noB; f += parts) {  // <Ib|E|J> = <J|E|Ib>, same pair and sign
+      const uint32_t w = lb[f];
+      const double *g = G + ((w >> 16) & 0xFFu), *d = D + (w & 0xFFFFu);
+      double a = 0.0, b = 0.0;
+      int e = 0;
+#pragma unroll 4
+      for (; e + 1 < nk; e += 2) {
+        a = fma(g[e * npair], d[e * NB], a);
+        b = fma(g[(e + 1) * npair], d[(e + 1) * NB], b);
+      }
+      if (e < nk) a = fma(g[e * npair], d[e * NB], a);
+      out += (w >> 31) ? -(a + b) : a + b;
+    }
+    // the unmoved replacements of Ib
+    for (int e = 1 + part; e < nk; e += parts) {
+      const uint32_t w = la[e - 1];
+      const double x = W[(long long)((w >> 16) & 0xFFu) * NB + Ib];
+      out = fma((w >> 31) ? -x : x, D[e * NB + Ib], out);
+    }
+    for (int m = part; m < npp; m += parts) out = fma(W[(long long)s_pp[m] * NB + Ib], D[Ib], out);
+  }
+  out = sm_sum(out, red, CH, parts);
+  if (threadIdx.x < CH && Ib < NB) S[(long long)blockIdx.z * vstride + (long long)Ia * NB + Ib] += out;
+}
+
+// Columns per block: as many threads share an output as leave two blocks an SM busy, and
+// 32 columns once the grid is larger than that.
+static int sm_columns(long long NA, long long NB, int nvec) {
+  int CH = 32;
+  while (CH > 8 && NA * ((NB + CH - 1) / CH) * nvec < 2 * 152) CH /= 2;
+  return CH;
+}
+
+static bool sd_small(const forte_ctx *ctx) { return ctx->sd[1].ell_col != nullptr; }
+
+static int sigma_fp64_small(forte_ctx *ctx, const double *C, double *S, int nvec) {
+  cudaStream_t st = ctx->stream;
+  const int n = ctx->n, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
+  const long long NA = ctx->Na, NB = ctx->Nb, ND = ctx->Ndet;
+  const int CH = sm_columns(NA, NB, nvec);
+  const SpinDev &A = ctx->sd[0], &B = ctx->sd[1];
+  const dim3 grid((unsigned)((NB + CH - 1) / CH), (unsigned)NA, (unsigned)nvec);
+  {
+    FORTE_PROF(ctx, "ss_spmm");
+    k_ss_small<true><<<grid, SM_THREADS, 0, st>>>(A.csr_ptr, A.csr_col, A.csr_val, 0, C, S, NB, ND, CH);
+    FORTE_LAUNCH_CHECK();
+  }
+  {
+    FORTE_PROF(ctx, "ss_spmm");
+    k_ss_small<false><<<grid, SM_THREADS, 0, st>>>(nullptr, B.ell_col, B.ell_val,
+                                                  ctx->sh[ctx->same_strings ? 0 : 1].csr_ptr[1], C, S, NB, ND, CH);
+    FORTE_LAUNCH_CHECK();
+  }
+  if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0) {
+    const size_t smem = sizeof(double) * (size_t)(noA + 1) * (NB + ctx->npair);
+    if (smem > 44 * 1024) FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_small));
+    FORTE_PROF(ctx, "ab_fp64");
+    k_ab_small<<<grid, SM_THREADS, smem, st>>>(A.list, ctx->sh[0].nk, A.off, noA, B.off, noB, (int)NB, ctx->d_gpair,
+                                              ctx->d_W, ctx->npair, C, S, ND, CH);
+    FORTE_LAUNCH_CHECK();
+  }
+  return FORTE_OK;
 }
 
 int sigma_fp64(forte_ctx *ctx, const double *C, double *S, int nvec) {
+  if (sd_small(ctx)) return sigma_fp64_small(ctx, C, S, nvec);
   // beta-beta scratch: T1 = C^T, T2 = H_bb T1 (grown on demand)
   const long long ND = ctx->Ndet;
   int rc = ctx->sc_t1.ensure(sizeof(double) * ND * nvec);
@@ -161,6 +391,7 @@ int sigma_fp64(forte_ctx *ctx, const double *C, double *S, int nvec) {
 // doubles); allocates nothing.  Shared by forte_sigma (context scratch) and
 // forte_sigma_fp64_noalloc (the library's fixed array).
 int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, double *T1, double *T2) {
+  if (sd_small(ctx)) return sigma_fp64_small(ctx, C, S, nvec);
   cudaStream_t st = ctx->stream;
   const long long NA = ctx->Na, NB = ctx->Nb, ND = ctx->Ndet;
   // alpha-alpha: S = H_aa C
@@ -197,29 +428,8 @@ int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, dou
     }
   }
   // alpha-beta
-  const int nkA = ctx->sh[0].nk, nkB = ctx->sh[ctx->same_strings ? 0 : 1].nk;
-  if (nkA > 0 && nkB > 0) {
-    if (nkA > 80) {
-      set_error("alpha replacement list too long (%d)", nkA);
-      return FORTE_ERR_ARG;
-    }
-    int TJ = 64;
-    size_t smem = ab_smem_bytes(nkA, nkB, ctx->npair, NB, TJ);
-    while (smem > 220 * 1024 && TJ > 8) {
-      TJ /= 2;
-      smem = ab_smem_bytes(nkA, nkB, ctx->npair, NB, TJ);
-    }
-    if (smem > 220 * 1024) {
-      set_error("alpha-beta FP64 kernel needs %zu bytes of shared memory", smem);
-      return FORTE_ERR_ARG;
-    }
-    FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_fp64));
-    dim3 grid((unsigned)NA, nvec);
-    FORTE_PROF(ctx, "ab_fp64");
-    k_ab_fp64<<<grid, AB_THREADS, smem, st>>>(ctx->sd[0].list, nkA, ctx->sd[1].list, nkB, NB, ctx->d_gpair,
-                                              ctx->npair, C, S, ND, TJ);
-    FORTE_LAUNCH_CHECK();
-  }
+  if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0)
+    return ab_launch<AbF64>(ctx, "ab_fp64", ctx->d_gpair, ctx->d_W, C, S, nvec);
   return FORTE_OK;
 }
 
@@ -413,60 +623,21 @@ __global__ void __launch_bounds__(SS_THREADS) k_ss_spmm_df(const int *__restrict
   }
 }
 
-// sigma_ab in double-FP32 for one alpha string Ia (blockIdx.x) and one vector
-// (blockIdx.y): k_ab_fp64 with (hi, lo) operands; the output row stays FP64.
-// 16 warps and 32-string tiles: two CTAs fit on an SM, so the tile gathers of one
-// overlap the shared-memory-bound inner products of the other.
-constexpr int AB_DF_THREADS = 512;
-constexpr int AB_DF_TJ = 32;
-__global__ void __launch_bounds__(AB_DF_THREADS) k_ab_df(const Repl *__restrict__ listA, int nkA,
-                                                      const Repl *__restrict__ listB, int nkB, long long NB,
-                                                      const float2 *__restrict__ gpair2, int npair,
-                                                      const float2 *__restrict__ C2, double *__restrict__ S,
-                                                      long long vstride, int TJ) {
-  extern __shared__ double smem[];
-  float2 *Gs = reinterpret_cast<float2 *>(smem);                 // nkA * npair
-  double *srow = smem + (size_t)nkA * npair;                     // NB
-  float2 *D = reinterpret_cast<float2 *>(srow + NB);              // nkA * TJ
-  Repl *Lb = reinterpret_cast<Repl *>(D + (size_t)nkA * TJ);      // TJ * nkB
-  const long long Ia = blockIdx.x;
-  const float2 *Cv = C2 + (long long)blockIdx.y * vstride;
-  double *Sv = S + (long long)blockIdx.y * vstride;
-  const Repl *la = listA + Ia * nkA;
-  __shared__ int s_J[80];
-  for (int e = threadIdx.x; e < nkA; e += AB_DF_THREADS) s_J[e] = la[e].J;
-  for (int i = threadIdx.x; i < nkA * npair; i += AB_DF_THREADS) {
-    const int e = i / npair, rs = i % npair;
-    const Repl r = la[e];
-    float2 g = gpair2[(size_t)r.pair * npair + rs];
-    if (r.sgn < 0) g = make_float2(-g.x, -g.y);
-    Gs[i] = g;
+// The alpha-beta term in double-FP32 (k_ab): bound by the 13 FP32 instructions of a term
+// and its two 8-byte shared-memory loads.  16 warps and 32-string tiles: two blocks fit
+// on an SM, so the tile gathers of one overlap the products of the other.
+struct AbDf {
+  using E = float2;
+  static constexpr int THREADS = 512, TJ = 32;
+  float h = 0.f, l = 0.f;
+  __device__ __forceinline__ void fma(E x, E y) { df_fma(h, l, x, y); }
+  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
+  static __device__ __forceinline__ E make(double x) {
+    const float f = (float)x;
+    return make_float2(f, (float)(x - (double)f));
   }
-  for (long long i = threadIdx.x; i < NB; i += AB_DF_THREADS) srow[i] = 0.0;
-  __syncthreads();
-  for (long long j0 = 0; j0 < NB; j0 += TJ) {
-    const int tj = (int)min((long long)TJ, NB - j0);
-    for (int i = threadIdx.x; i < nkA * tj; i += AB_DF_THREADS) {
-      const int e = i / tj, j = i % tj;
-      D[e * TJ + j] = Cv[(long long)s_J[e] * NB + j0 + j];
-    }
-    for (int i = threadIdx.x; i < tj * nkB; i += AB_DF_THREADS) Lb[i] = listB[j0 * nkB + i];
-    __syncthreads();
-    const int npairs_tile = tj * nkB;
-    for (int w = threadIdx.x; w < npairs_tile; w += AB_DF_THREADS) {
-      const int j = w / nkB;
-      const Repl rf = Lb[w];
-      const float2 *g = Gs + rf.pair;
-      const float2 *d = D + j;
-      float ah = 0.f, al = 0.f;
-#pragma unroll 8
-      for (int e = 0; e < nkA; ++e) df_fma(ah, al, g[e * npair], d[e * TJ]);
-      atomicAdd(&srow[rf.J], rf.sgn * ((double)ah + (double)al));
-    }
-    __syncthreads();
-  }
-  for (long long i = threadIdx.x; i < NB; i += AB_DF_THREADS) Sv[Ia * NB + i] += srow[i];
-}
+  static __device__ __forceinline__ E neg(E x) { return make_float2(-x.x, -x.y); }
+};
 
 static int df_setup(forte_ctx *ctx) {
   if (ctx->d_gpair2) return FORTE_OK;
@@ -474,6 +645,11 @@ static int df_setup(forte_ctx *ctx) {
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gpair2, sizeof(float2) * (size_t)np * np));
   k_df_split<<<(unsigned)std::min<long long>(((long long)np * np + 255) / 256, 1024), 256, 0, ctx->stream>>>(
       ctx->d_gpair, (float2 *)ctx->d_gpair2, (long long)np * np);
+  FORTE_LAUNCH_CHECK();
+  const long long nw = (long long)np * ctx->Nb;
+  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_W2, sizeof(float2) * (size_t)nw));
+  k_df_split<<<(unsigned)std::min<long long>((nw + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
+      ctx->d_W, (float2 *)ctx->d_W2, nw);
   FORTE_LAUNCH_CHECK();
   const int nsp = ctx->same_strings ? 1 : 2;
   for (int s = 0; s < nsp; ++s) {
@@ -536,29 +712,8 @@ int sigma_df(forte_ctx *ctx, const double *C, double *S, int nvec, bool with_ab)
       FORTE_LAUNCH_CHECK();
     }
   }
-  const int nkA = ctx->sh[0].nk, nkB = ctx->sh[ctx->same_strings ? 0 : 1].nk;
-  if (with_ab && nkA > 0 && nkB > 0) {
-    if (nkA > 80) {
-      set_error("alpha replacement list too long (%d)", nkA);
-      return FORTE_ERR_ARG;
-    }
-    int TJ = AB_DF_TJ;
-    size_t smem = ab_smem_bytes(nkA, nkB, ctx->npair, NB, TJ);
-    while (smem > 220 * 1024 && TJ > 8) {
-      TJ /= 2;
-      smem = ab_smem_bytes(nkA, nkB, ctx->npair, NB, TJ);
-    }
-    if (smem > 220 * 1024) {
-      set_error("alpha-beta double-FP32 kernel needs %zu bytes of shared memory", smem);
-      return FORTE_ERR_ARG;
-    }
-    FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_df));
-    dim3 grid((unsigned)NA, nvec);
-    FORTE_PROF(ctx, "ab_df");
-    k_ab_df<<<grid, AB_DF_THREADS, smem, st>>>(ctx->sd[0].list, nkA, ctx->sd[1].list, nkB, NB,
-                                            (const float2 *)ctx->d_gpair2, ctx->npair, C2, S, ND, TJ);
-    FORTE_LAUNCH_CHECK();
-  }
+  if (with_ab && ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0)
+    return ab_launch<AbDf>(ctx, "ab_df", (const float2 *)ctx->d_gpair2, (const float2 *)ctx->d_W2, C2, S, nvec);
   return FORTE_OK;
 }
 
