@@ -53,11 +53,13 @@ __device__ __forceinline__ double block_sum_t(T v, double *red) {
 
 // Second pass of a reduction, fused into the kernel that writes the partials: every
 // block publishes its partials part[block][0..m) and counts itself in; the last block
-// to arrive sums part[b][c] over b (strided by thread, then block_sum: the order of
-// a separate 256-thread pass) into out[c] and resets the counter for the next
-// launch on the stream.  No block waits for another.
+// to arrive sums part[b][c] over b into out[c] and resets the counter for the next
+// launch on the stream.  A group of `g` lanes (a power of two, m groups if they fit)
+// takes a column: the FP64 pipe issues a warp's addition in 16 clocks, so a block-wide
+// sum per column, most of whose lanes add zeros, took longer than the rest of a short
+// kernel.  No block waits for another.
 __device__ __forceinline__ void last_block_sums(const double *part, int m, double *__restrict__ out,
-                                                unsigned *counter, double *red) {
+                                                unsigned *counter) {
   __shared__ bool s_last;
   __threadfence();
   __syncthreads();
@@ -66,11 +68,18 @@ __device__ __forceinline__ void last_block_sums(const double *part, int m, doubl
   if (!s_last) return;
   __threadfence();
   const int nblk = (int)gridDim.x;
-  for (int c = 0; c < m; ++c) {
+  int g = 32;
+  while (g > 4 && m * g > (int)blockDim.x) g >>= 1;
+  const int groups = blockDim.x / g, lane = threadIdx.x % g;
+  for (int c0 = 0; c0 < m; c0 += groups) {
+    const int c = c0 + threadIdx.x / g;
     double s = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += __ldcg(part + (long long)b * m + c);
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) out[c] = s;
+    if (c < m) {
+#pragma unroll 4
+      for (int b = lane; b < nblk; b += g) s += __ldcg(part + (long long)b * m + c);
+    }
+    for (int o = g >> 1; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (c < m && lane == 0) out[c] = s;
   }
   if (threadIdx.x == 0) *counter = 0u;
 }
@@ -100,7 +109,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_multidot(const T *__restrict__ V
     const double at = block_sum_t<T>(a, red);
     if (threadIdx.x == 0) part[(long long)blockIdx.x * nv + i] = at;
   }
-  last_block_sums(part, nv, out, counter, red);
+  last_block_sums(part, nv, out, counter);
 }
 
 // out_{c0+c} = sum_i coef[i*ncomb + c0 + c] V_i  for c < NC.  NC is a template
@@ -160,7 +169,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_residual_precond(
   }
   const double rt = block_sum_t<T>(rr, red);
   if (threadIdx.x == 0) part[blockIdx.x] = rt;
-  last_block_sums(part, 1, out, counter, red);
+  last_block_sums(part, 1, out, counter);
 }
 
 // t_out = t_in - sum_i c_i B_i ; part[block][i] = B_i . t_out (i < k), part[block][k] = |t_out|^2.
@@ -219,7 +228,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_orth_update(const T *__restrict_
   }
   const double nt = block_sum_t<T>(nn, red);
   if (threadIdx.x == 0) part[(long long)blockIdx.x * (k + 1) + k] = nt;
-  last_block_sums(part, k + 1, out, counter, red);
+  last_block_sums(part, k + 1, out, counter);
 }
 
 // y = a x + b y
@@ -253,7 +262,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_precond_dot(const double *__rest
     part[2 * blockIdx.x] = acc;
     part[2 * blockIdx.x + 1] = rr;
   }
-  last_block_sums(part, 2, out, counter, red);
+  last_block_sums(part, 2, out, counter);
 }
 
 // rinv = 1 / |theta - hdiag| with the magnitude clamped below at guard: the FP64
@@ -319,6 +328,178 @@ __global__ void k_nonfinite(const double *__restrict__ x, long long n, int *flag
   for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n;
        j += (long long)gridDim.x * blockDim.x)
     if (!isfinite(x[j])) *flag = 1;
+}
+
+// ------------------------------------------------------------------ short vectors
+// Up to VS_MAX_N elements the kernels above and below leave most SMs idle (a block takes
+// 4096 or 2048 elements), and the FP64 work of a block is then the time: 5 blocks of a
+// 4900-element residual pass took 31 us.  Here a block of 64 threads takes 128 elements,
+// one chunk, so that the vectors spread over the SMs; the per-thread sums of a column
+// meet in shared memory, where 4 threads add one column (64 values), instead of a
+// five-step warp reduction per column.  Elements are loaded singly, so any count and
+// alignment will do.  One GB300, CAS(8,8) FP64 solve (133 iterations): residual pass 31 ->
+// 14 us, 11-vector dots 22 -> 9 us, whole solve 21.5 -> 14.0 ms.
+constexpr int VS_T = 64;
+constexpr int VS_E = 2;
+constexpr long long VS_CHUNK = VS_T * VS_E;
+constexpr int VS_COLS = 16;  // columns reduced at a time
+constexpr long long VS_MAX_N = VS_CHUNK * 608;
+
+struct VsRed {
+  double v[VS_COLS][VS_T + 1];
+};
+// Publish the block's sums of columns c0 .. c0 + nc (r.v filled by every thread).
+__device__ __forceinline__ void vs_columns(VsRed &r, int c0, int nc, int m, double *part) {
+  __syncthreads();
+  const int c = threadIdx.x >> 2, q = threadIdx.x & 3;
+  double a = 0.0, b = 0.0;
+  if (c < nc) {
+#pragma unroll
+    for (int k = 0; k < VS_T / 4; k += 2) {
+      a += r.v[c][q + 4 * k];
+      b += r.v[c][q + 4 * k + 4];
+    }
+  }
+  a += b;
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  if (c < nc && q == 0) part[(long long)blockIdx.x * m + c0 + c] = a;
+  __syncthreads();
+}
+
+// part[block][col0 + i] = sum over the chunk of V_i . x, i < nv (m columns in all).
+template <typename T>
+__device__ __forceinline__ void vs_dots(VsRed &r, const T *__restrict__ V, int nv, long long ld, const T (&x)[VS_E],
+                                        long long j0, long long n, int col0, int m, double *part) {
+  for (int i0 = 0; i0 < nv; i0 += VS_COLS) {
+    const int nc = min(VS_COLS, nv - i0);
+#pragma unroll 4
+    for (int i = 0; i < nc; ++i) {
+      const T *v = V + (long long)(i0 + i) * ld;
+      T a = 0;
+#pragma unroll
+      for (int e = 0; e < VS_E; ++e)
+        if (j0 + e * VS_T < n) a += v[j0 + e * VS_T] * x[e];
+      r.v[i][threadIdx.x] = (double)a;
+    }
+    vs_columns(r, col0 + i0, nc, m, part);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(VS_T) k_multidot_s(const T *__restrict__ V, int nv, long long ld,
+                                                     const T *__restrict__ x, long long n, double *__restrict__ part,
+                                                     double *__restrict__ out, unsigned *counter) {
+  __shared__ VsRed r;
+  const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
+  T xr[VS_E];
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e) xr[e] = j0 + e * VS_T < n ? x[j0 + e * VS_T] : T(0);
+  vs_dots(r, V, nv, ld, xr, j0, n, 0, nv, part);
+  last_block_sums(part, nv, out, counter);
+}
+
+// As k_orth_update_p: t_out = scale (t_in - B c), out = [B^T t_out (zeros unless DOTS), |t_out|^2].
+template <typename T, bool DOTS>
+__global__ void __launch_bounds__(VS_T) k_orth_update_s(const T *__restrict__ B, int k, long long ld,
+                                                        const double *__restrict__ c, const T *t_in, T *t_out,
+                                                        long long n, double scale, double *__restrict__ part,
+                                                        double *__restrict__ out, unsigned *counter) {
+  __shared__ VsRed r;
+  __shared__ T sc[VK_MAXV];
+  const int ku = c ? k : 0;
+  for (int i = threadIdx.x; i < ku; i += VS_T) sc[i] = (T)c[i];
+  __syncthreads();
+  const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
+  T t[VS_E], nn = 0;
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e) t[e] = j0 + e * VS_T < n ? t_in[j0 + e * VS_T] : T(0);
+#pragma unroll 4
+  for (int i = 0; i < ku; ++i)
+#pragma unroll
+    for (int e = 0; e < VS_E; ++e)
+      if (j0 + e * VS_T < n) t[e] -= sc[i] * B[(long long)i * ld + j0 + e * VS_T];
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e)
+    if (j0 + e * VS_T < n) {
+      if (scale != 1.0) t[e] *= (T)scale;
+      t_out[j0 + e * VS_T] = t[e];
+      nn += t[e] * t[e];
+    }
+  r.v[0][threadIdx.x] = (double)nn;
+  vs_columns(r, k, 1, k + 1, part);
+  if (DOTS) {
+    vs_dots(r, B, k, ld, t, j0, n, 0, k + 1, part);
+  } else {
+    for (int i = threadIdx.x; i < k; i += VS_T) part[(long long)blockIdx.x * (k + 1) + i] = 0.0;
+  }
+  last_block_sums(part, k + 1, out, counter);
+}
+
+// As k_residual_precond_p: t = r / (theta - H_II), out = [|r|^2 (, B^T t, |t|^2)].
+template <typename T, bool DOTS>
+__global__ void __launch_bounds__(VS_T) k_residual_precond_s(const T *__restrict__ B, const T *__restrict__ S, int k,
+                                                             long long ld, const double *__restrict__ u, double theta,
+                                                             const double *__restrict__ hd, double guard,
+                                                             T *__restrict__ t, long long n, double *__restrict__ part,
+                                                             double *__restrict__ out, unsigned *counter) {
+  __shared__ VsRed r;
+  __shared__ T su[VK_MAXV];
+  const int m = DOTS ? k + 2 : 1;
+  for (int i = threadIdx.x; i < k; i += VS_T) su[i] = (T)u[i];
+  __syncthreads();
+  const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
+  T hx[VS_E], xv[VS_E], rr = 0, tt = 0;
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e) hx[e] = xv[e] = 0;
+#pragma unroll 4
+  for (int i = 0; i < k; ++i)
+#pragma unroll
+    for (int e = 0; e < VS_E; ++e)
+      if (j0 + e * VS_T < n) {
+        hx[e] += su[i] * S[(long long)i * ld + j0 + e * VS_T];
+        xv[e] += su[i] * B[(long long)i * ld + j0 + e * VS_T];
+      }
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e)
+    if (j0 + e * VS_T < n) {
+      const T res = hx[e] - (T)theta * xv[e];
+      rr += res * res;
+      double den = theta - hd[j0 + e * VS_T];
+      if (fabs(den) < guard) den = (den >= 0.0) ? guard : -guard;
+      hx[e] = res / (T)den;  // hx now holds t
+      tt += hx[e] * hx[e];
+      t[j0 + e * VS_T] = hx[e];
+    }
+  r.v[0][threadIdx.x] = (double)rr;
+  vs_columns(r, 0, 1, m, part);
+  if (DOTS) {
+    r.v[0][threadIdx.x] = (double)tt;
+    vs_columns(r, k + 1, 1, m, part);
+    vs_dots(r, B, k, ld, hx, j0, n, 1, m, part);
+  }
+  last_block_sums(part, m, out, counter);
+}
+
+// z = r * rinv; out = [r . z, r . r]
+__global__ void __launch_bounds__(VS_T) k_precond_dot_s(const double *__restrict__ rv, const double *__restrict__ rinv,
+                                                        double *__restrict__ z, long long n, double *__restrict__ part,
+                                                        double *__restrict__ out, unsigned *counter) {
+  __shared__ VsRed r;
+  const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
+  double rz = 0.0, rr = 0.0;
+#pragma unroll
+  for (int e = 0; e < VS_E; ++e)
+    if (j0 + e * VS_T < n) {
+      const double x = rv[j0 + e * VS_T], y = x * rinv[j0 + e * VS_T];
+      z[j0 + e * VS_T] = y;
+      rz = fma(x, y, rz);
+      rr = fma(x, x, rr);
+    }
+  r.v[0][threadIdx.x] = rz;
+  r.v[1][threadIdx.x] = rr;
+  vs_columns(r, 0, 2, 2, part);
+  last_block_sums(part, 2, out, counter);
 }
 
 // ------------------------------------------------------------------ packet kernels
@@ -407,7 +588,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_p(const T *__re
                                                            double *__restrict__ part, double *__restrict__ out,
                                                            unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[VK_MAXV * VP_WARPS];
   for (int i = threadIdx.x; i < nv * VP_WARPS; i += blockDim.x) sw[i] = 0.0;
   __syncthreads();
@@ -442,7 +622,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_p(const T *__re
     }
   }
   block_partials(sw, nv, part);
-  last_block_sums(part, nv, out, counter, red);
+  last_block_sums(part, nv, out, counter);
 }
 
 // The same for nv <= KMAX: loop over the vectors unrolled, partial sums of the
@@ -453,7 +633,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_u(const T *__re
                                                                    double *__restrict__ part,
                                                                    double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[KMAX * VP_WARPS];
   for (int i = threadIdx.x; i < nv * VP_WARPS; i += blockDim.x) sw[i] = 0.0;
   __syncthreads();
@@ -495,7 +674,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_u(const T *__re
   for (int i = 0; i < KMAX; ++i)
     if (i < nv) warp_add(acc[i], sw + i * VP_WARPS);
   block_partials(sw, nv, part);
-  last_block_sums(part, nv, out, counter, red);
+  last_block_sums(part, nv, out, counter);
 }
 
 // t_out = scale (t_in - sum_i c_i B_i); out = [B_i . t_out (i < k, zeros unless DOTS),
@@ -507,7 +686,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_p(const T *_
                                                               double *__restrict__ part, double *__restrict__ out,
                                                               unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[(VK_MAXV + 1) * VP_WARPS];
   __shared__ T sc[VK_MAXV];
   const int ku = c ? k : 0;
@@ -577,7 +755,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_p(const T *_
     }
   }
   block_partials(sw, k + 1, part);
-  last_block_sums(part, k + 1, out, counter, red);
+  last_block_sums(part, k + 1, out, counter);
 }
 
 // The same for k <= KMAX: loops over the basis unrolled, partial sums in registers.
@@ -588,7 +766,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_u(const T *_
                                                                       double *__restrict__ part,
                                                                       double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[(KMAX + 1) * VP_WARPS];
   __shared__ T sc[KMAX];
   const int ku = c ? k : 0;
@@ -669,7 +846,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_u(const T *_
       if (i < k) warp_add(acc[i], sw + i * VP_WARPS);
   }
   block_partials(sw, k + 1, part);
-  last_block_sums(part, k + 1, out, counter, red);
+  last_block_sums(part, k + 1, out, counter);
 }
 
 // r = sum_i u_i S_i - theta sum_i u_i B_i ;  t = r / (theta - hdiag) (guarded).
@@ -684,7 +861,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_p(
     double theta, const double *__restrict__ hd, double guard, T *__restrict__ t, long long np,
     double *__restrict__ part, double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[(VK_MAXV + 2) * VP_WARPS];
   __shared__ T su[VK_MAXV];
   const int m = DOTS ? k + 2 : 1;
@@ -758,7 +934,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_p(
     }
   }
   block_partials(sw, m, part);
-  last_block_sums(part, m, out, counter, red);
+  last_block_sums(part, m, out, counter);
 }
 
 // The same for k <= KMAX with the loops over the basis unrolled (the loads of all k
@@ -770,7 +946,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_u(
     double theta, const double *__restrict__ hd, double guard, T *__restrict__ t, long long np,
     double *__restrict__ part, double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
-  __shared__ double red[32];
   __shared__ double sw[(KMAX + 2) * VP_WARPS];
   __shared__ T su[KMAX];
   const int m = DOTS ? k + 2 : 1;
@@ -858,7 +1033,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_u(
       if (i < k) warp_add(acc[i], sw + (1 + i) * VP_WARPS);
   }
   block_partials(sw, m, part);
-  last_block_sums(part, m, out, counter, red);
+  last_block_sums(part, m, out, counter);
 }
 
 // z = r * rinv; out[0] = r . z, out[1] = r . r
@@ -867,7 +1042,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_precond_dot_p(const doub
                                                                       double *__restrict__ z, long long np,
                                                                       double *__restrict__ part, double *__restrict__ out,
                                                                       unsigned *counter) {
-  __shared__ double red[32];
   __shared__ double sw[2 * VP_WARPS];
   if (threadIdx.x < 2 * VP_WARPS) sw[threadIdx.x] = 0.0;
   __syncthreads();
@@ -895,7 +1069,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_precond_dot_p(const doub
     warp_add(rr, sw + VP_WARPS);
   }
   block_partials(sw, 2, part);
-  last_block_sums(part, 2, out, counter, red);
+  last_block_sums(part, 2, out, counter);
 }
 
 // y = a x + b y and x = alpha src over packets (grid-stride).  With a or b equal to 1
@@ -952,6 +1126,7 @@ static bool vp_ok(long long n, long long ld, std::initializer_list<const void *>
     if (q && ((uintptr_t)q & 15u) != 0) return false;
   return true;
 }
+static unsigned vs_blocks(long long n) { return (unsigned)std::max<long long>(1, (n + VS_CHUNK - 1) / VS_CHUNK); }
 // persistent grid: VP_BPS resident blocks of VK_THREADS per SM, at least one block
 static unsigned vp_grid(const forte_ctx *ctx, long long np) {
   int nsm = 0;
@@ -967,14 +1142,16 @@ template <typename T>
 static int vk_multidot_t(forte_ctx *ctx, const T *V, int nv, long long ld, const T *x, long long n, double *out) {
   if (nv <= 0) return FORTE_OK;
   if (nv > VK_MAXV) { set_error("multidot: too many vectors (%d)", nv); return FORTE_ERR_ARG; }
-  const bool pk = vp_ok<T>(n, ld, {V, x});
-  const unsigned nb = pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
+  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {V, x});
+  const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
   double *part;
   unsigned *cnt;
   int rc = part_buffer(ctx, (size_t)nb * nv, &part, &cnt);
   if (rc) return rc;
   FORTE_PROF(ctx, "multidot");
-  if (pk && nv <= 4)
+  if (vs)
+    k_multidot_s<T><<<nb, VS_T, 0, ctx->stream>>>(V, nv, ld, x, n, part, out, cnt);
+  else if (pk && nv <= 4)
     k_multidot_u<T, 4><<<nb, VK_THREADS, 0, ctx->stream>>>(V, nv, ld, x, n / Pk<T>::P, part, out, cnt);
   else if (pk && nv <= 8)
     k_multidot_u<T, 8><<<nb, VK_THREADS, 0, ctx->stream>>>(V, nv, ld, x, n / Pk<T>::P, part, out, cnt);
@@ -1015,9 +1192,9 @@ template <typename T>
 static int vk_residual_precond_t(forte_ctx *ctx, const T *B, const T *S, int k, long long ld, const double *u,
                                  double theta, double guard, T *t, double *rnorm2, long long n, double *dots) {
   if (k > VK_MAXV) { set_error("residual: subspace too large (%d)", k); return FORTE_ERR_ARG; }
-  const bool pk = vp_ok<T>(n, ld, {B, S, t, ctx->d_hdiag});
-  if (dots && !pk) return -1;  // no fused dots: the caller forms them with vk_orth_update
-  const unsigned nb = pk ? vp_grid(ctx, 2 * (n / Pk<T>::P)) : vk_blocks(n);  // chunks of half the packets
+  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, S, t, ctx->d_hdiag});
+  if (dots && !pk && !vs) return -1;  // no fused dots: the caller forms them with vk_orth_update
+  const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, 2 * (n / Pk<T>::P)) : vk_blocks(n);  // chunks of half the packets
   const int m = dots ? k + 2 : 1;
   double *part;
   unsigned *cnt;
@@ -1035,7 +1212,12 @@ static int vk_residual_precond_t(forte_ctx *ctx, const T *B, const T *S, int k, 
       k_residual_precond_u<T, false, 2, KM><<<nb, VK_THREADS, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, \
                                                                                 npk, part, rnorm2, cnt);             \
   } while (0)
-  if (pk && k <= 4)
+  if (vs && dots)
+    k_residual_precond_s<T, true><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, dots, cnt);
+  else if (vs)
+    k_residual_precond_s<T, false><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, rnorm2,
+                                                                 cnt);
+  else if (pk && k <= 4)
     FORTE_RESID_U(4);
   else if (pk && k <= 8)
     FORTE_RESID_U(8);
@@ -1070,13 +1252,13 @@ template <typename T>
 static int vk_orth_update_t(forte_ctx *ctx, const T *B, int k, long long ld, const double *c, const T *t_in,
                             T *t_out, double *dots_out, long long n, bool dots, double scale) {
   if (k + 1 > VK_MAXV) { set_error("orth: subspace too large (%d)", k); return FORTE_ERR_ARG; }
-  const bool pk = vp_ok<T>(n, ld, {B, t_in, t_out});
-  const unsigned nb = pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
+  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, t_in, t_out});
+  const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
   double *part;
   unsigned *cnt;
   int rc = part_buffer(ctx, (size_t)nb * (k + 1), &part, &cnt);
   if (rc) return rc;
-  if (!pk && scale != 1.0) {  // element path: the scale is a separate pass
+  if (!pk && !vs && scale != 1.0) {  // element path: the scale is a separate pass
     if ((rc = vk_orth_update_t(ctx, B, k, ld, c, t_in, t_out, dots_out, n, dots, 1.0))) return rc;
     if ((rc = vk_scale(ctx, t_out, t_out, scale, n))) return rc;
     // |t_out|^2 and the dots scale with scale^2 and scale
@@ -1093,7 +1275,11 @@ static int vk_orth_update_t(forte_ctx *ctx, const T *B, int k, long long ld, con
       k_orth_update_u<T, false, KM><<<nb, VK_THREADS, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, npk,      \
                                                                         scale, part, dots_out, cnt);        \
   } while (0)
-  if (pk && k <= 4)
+  if (vs && dots)
+    k_orth_update_s<T, true><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
+  else if (vs)
+    k_orth_update_s<T, false><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
+  else if (pk && k <= 4)
     FORTE_ORTH_U(4);
   else if (pk && k <= 8)
     FORTE_ORTH_U(8);
@@ -1196,14 +1382,16 @@ int vk_precond_inv(forte_ctx *ctx, double theta, double guard, double *rinv, lon
 }
 
 int vk_precond_dot(forte_ctx *ctx, const double *r, const double *rinv, double *z, double *dot_out, long long n) {
-  const bool pk = vp_ok<double>(n, n, {r, z, rinv});
-  const unsigned nb = pk ? vp_grid(ctx, n / 2) : vk_blocks(n);
+  const bool vs = n <= VS_MAX_N, pk = vp_ok<double>(n, n, {r, z, rinv});
+  const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / 2) : vk_blocks(n);
   double *part;
   unsigned *cnt;
   int rc = part_buffer(ctx, (size_t)2 * nb, &part, &cnt);
   if (rc) return rc;
   FORTE_PROF(ctx, "precond_dot");
-  if (pk)
+  if (vs)
+    k_precond_dot_s<<<nb, VS_T, 0, ctx->stream>>>(r, rinv, z, n, part, dot_out, cnt);
+  else if (pk)
     k_precond_dot_p<<<nb, VK_THREADS, 0, ctx->stream>>>(r, rinv, z, n / 2, part, dot_out, cnt);
   else
     k_precond_dot<<<nb, VK_THREADS, 0, ctx->stream>>>(r, rinv, z, n, part, dot_out, cnt);
