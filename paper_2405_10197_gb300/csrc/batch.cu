@@ -1160,6 +1160,7 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
   double *dwork = (double *)(dbuf + ((table_bytes + 255) & ~(size_t)255));
   if (!classes.empty()) {
     FORTE_CUDA_TRY(cudaMemcpy(dbuf, pool.host.data(), table_bytes, cudaMemcpyHostToDevice));
+    FORTE_CUDA_TRY(cudaStreamSynchronize(nullptr));  // the class streams do not wait for the default one
     for (int s = 0; s < (int)classes.size(); ++s) {
       cudaStream_t x = nullptr;
       FORTE_CUDA_TRY(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));

@@ -230,6 +230,10 @@ namespace forte {
 // Always the same value, so concurrent callers (batched solves) cannot undercut
 // one another's launches.
 cudaError_t set_smem_optin_max(const void *func);
+// Copy host data to the device on the context's stream, so that the kernels queued there
+// afterwards see it.  (cudaMemcpy from pageable memory may return before its last chunk
+// has reached the device, and work on a non-blocking stream does not wait for it.)
+cudaError_t copy_in(const forte_ctx *ctx, void *dst, const void *src, size_t bytes);
 int build_spin_tables(forte_ctx *ctx);
 // Spaces whose gathered alpha rows fit in shared memory next to a second block: the FP64
 // sigma runs without transposes or atomics there (sigma_fp64.cu).

@@ -333,14 +333,14 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
       set_error("cudaMalloc of the string classes failed");
       return FORTE_ERR_ALLOC;
     }
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_cls[s], cls[s].data(), sizeof(int) * cls[s].size(), cudaMemcpyHostToDevice));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cls[s], cls[s].data(), sizeof(int) * cls[s].size()));
   }
   if (cudaMalloc(&ctx->d_gas_ok, ok.size()) != cudaSuccess) {
     gas_release(ctx);
     set_error("cudaMalloc of the class table failed");
     return FORTE_ERR_ALLOC;
   }
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_ok, ok.data(), ok.size(), cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_ok, ok.data(), ok.size()));
   // lists of the restricted sigma: kept alpha rows; per alpha class the beta strings
   // of its allowed classes (ascending)
   {
@@ -364,9 +364,9 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
       return FORTE_ERR_ALLOC;
     }
     if (!rowsv.empty())
-      FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_rows, rowsv.data(), sizeof(int) * rowsv.size(), cudaMemcpyHostToDevice));
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_boff, boff.data(), sizeof(int) * boff.size(), cudaMemcpyHostToDevice));
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_blist, blist.data(), sizeof(int) * blist.size(), cudaMemcpyHostToDevice));
+      FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_rows, rowsv.data(), sizeof(int) * rowsv.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_boff, boff.data(), sizeof(int) * boff.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_blist, blist.data(), sizeof(int) * blist.size()));
     ctx->gas_nrows = (long long)rowsv.size();
     ctx->gas_maxnnz = maxnnz;
   }
@@ -390,10 +390,9 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
       set_error("cudaMalloc of the restricted-sigma class lists failed");
       return FORTE_ERR_ALLOC;
     }
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size(), cudaMemcpyHostToDevice));
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size(), cudaMemcpyHostToDevice));
-    FORTE_CUDA_TRY(cudaMemcpy(ctx->d_gas_reach, reach.data(), sizeof(unsigned long long) * reach.size(),
-                              cudaMemcpyHostToDevice));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_reach, reach.data(), sizeof(unsigned long long) * reach.size()));
   }
   ctx->gas_nc[0] = ncA;
   ctx->gas_nc[1] = ncB;

@@ -298,7 +298,8 @@ forte_sci *forte_sci_create(int norb, const double *h, const double *eri) {
   if (cudaGetDevice(&s->device) != cudaSuccess || cudaMalloc(&s->d_h, sizeof(double) * n * n) != cudaSuccess ||
       cudaMalloc(&s->d_eri, sizeof(double) * n4) != cudaSuccess ||
       cudaMemcpy(s->d_h, h, sizeof(double) * n * n, cudaMemcpyHostToDevice) != cudaSuccess ||
-      cudaMemcpy(s->d_eri, eri, sizeof(double) * n4, cudaMemcpyHostToDevice) != cudaSuccess) {
+      cudaMemcpy(s->d_eri, eri, sizeof(double) * n4, cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaStreamSynchronize(nullptr) != cudaSuccess) {  // (the handle's stream may not wait for the default one)
     set_error("forte_sci_create: device allocation or copy failed");
     cudaFree(s->d_h);
     cudaFree(s->d_eri);

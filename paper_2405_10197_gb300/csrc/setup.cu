@@ -161,6 +161,11 @@ static int build_one_spin(forte_ctx *ctx, SpinHost &S, int nel) {
   return FORTE_OK;
 }
 
+cudaError_t copy_in(const forte_ctx *ctx, void *dst, const void *src, size_t bytes) {
+  const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->stream);  // src may go out of scope
+}
+
 cudaError_t set_smem_optin_max(const void *func) {
   int dev = 0, mx = 0;
   cudaError_t e = cudaGetDevice(&dev);

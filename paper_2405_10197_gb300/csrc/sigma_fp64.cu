@@ -503,7 +503,7 @@ int hdiag_build(forte_ctx *ctx) {
     }
   double *dW = nullptr;
   FORTE_CUDA_TRY(cudaMalloc(&dW, sizeof(double) * W.size()));
-  FORTE_CUDA_TRY(cudaMemcpy(dW, W.data(), sizeof(double) * W.size(), cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, dW, W.data(), sizeof(double) * W.size()));
   if (!ctx->d_hdiag) {
     cudaError_t e = cudaMalloc(&ctx->d_hdiag, sizeof(double) * ctx->Ndet);
     if (e != cudaSuccess) {

@@ -828,16 +828,16 @@ static int ab_positions(forte_ctx *ctx) {
       dcnt[r.J] = (int8_t)(dcnt[r.J] + (r.sgn < 0 ? -1 : 1));
     }
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abDcnt, dcnt.size()));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_abDcnt, dcnt.data(), dcnt.size(), cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abDcnt, dcnt.data(), dcnt.size()));
   ctx->ab_split = split;
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abTabL, sizeof(uint16_t) * tabL.size()));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_abTabL, tabL.data(), sizeof(uint16_t) * tabL.size(), cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abTabL, tabL.data(), sizeof(uint16_t) * tabL.size()));
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abPosOf, sizeof(uint16_t) * posOf.size()));
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abStrOf, sizeof(int) * strOf.size()));
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abTab, sizeof(uint16_t) * tab.size()));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_abPosOf, posOf.data(), sizeof(uint16_t) * posOf.size(), cudaMemcpyHostToDevice));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_abStrOf, strOf.data(), sizeof(int) * strOf.size(), cudaMemcpyHostToDevice));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_abTab, tab.data(), sizeof(uint16_t) * tab.size(), cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abPosOf, posOf.data(), sizeof(uint16_t) * posOf.size()));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abStrOf, strOf.data(), sizeof(int) * strOf.size()));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abTab, tab.data(), sizeof(uint16_t) * tab.size()));
   ctx->ab_NBpos = NBpos;
   return FORTE_OK;
 }

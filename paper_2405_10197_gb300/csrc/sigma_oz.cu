@@ -532,8 +532,8 @@ static int oz_ab_setup(forte_ctx *ctx) {
   FORTE_LAUNCH_CHECK();
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozG, sizeof(uint16_t) * gd.size()));
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozGa, sizeof(int) * 128));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_ozG, gd.data(), sizeof(uint16_t) * gd.size(), cudaMemcpyHostToDevice));
-  FORTE_CUDA_TRY(cudaMemcpy(ctx->d_ozGa, ga.data(), sizeof(int) * 128, cudaMemcpyHostToDevice));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_ozG, gd.data(), sizeof(uint16_t) * gd.size()));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_ozGa, ga.data(), sizeof(int) * 128));
   if (!ctx->d_err) {
     const int rc_err = err_word_setup(ctx);
     if (rc_err) return rc_err;
@@ -545,8 +545,7 @@ static int oz_ab_setup(forte_ctx *ctx) {
 static int sigma_ab_oz(forte_ctx *ctx, const double *C, double *S, int nvec) {
   const int nkA = ctx->sh[0].nk, nkB = ctx->sh[ctx->same_strings ? 0 : 1].nk;
   if (nkA <= 0 || nkB <= 0) return FORTE_OK;
-  int rc = oz_ab_setup(ctx);
-  if (rc) return rc;
+  int rc = FORTE_OK;
   cudaStream_t st = ctx->stream;
   const long long NA = ctx->Na, NB = ctx->Nb;
   const long long NBp = (NB + ZB_TN - 1) / ZB_TN * ZB_TN;
@@ -602,8 +601,10 @@ static int sigma_ab_oz(forte_ctx *ctx, const double *C, double *S, int nvec) {
 // tensor-core one does not apply (more than 15 orbitals, n_kl > 64).
 int sigma_oz64(forte_ctx *ctx, const double *C, double *S, int nvec) {
   if (!oz_ab_supported(ctx)) return sigma_df(ctx, C, S, nvec, true);
-  int rc = sigma_df(ctx, C, S, nvec, false);
+  const bool ab = ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0;
+  int rc = ab ? oz_ab_setup(ctx) : FORTE_OK;  // (waits for its uploads: before anything is queued)
   if (rc) return rc;
+  if ((rc = sigma_df(ctx, C, S, nvec, false))) return rc;
   return sigma_ab_oz(ctx, C, S, nvec);
 }
 
