@@ -193,6 +193,29 @@ static int sigma_dispatch(forte_ctx *ctx, const float *C, float *S, int nvec, in
 
 // ----------------------------------------------------------------- Davidson
 
+// Areas of the page-locked memory that the copies of an iteration go through:
+// coefficients of the residual passes (64 a root), their results (66 a root), columns of
+// the subspace matrix (64 a new vector), scalars.
+struct PinArea {
+  double *u, *rd, *g, *s;
+};
+static int pin_area(forte_ctx *ctx, PinArea &p) {
+  constexpr size_t NU = 64 * 64, NRD = 64 * 66, NG = 64 * 64, NS = 80;
+  if (!ctx->h_pin &&
+      cudaHostAlloc(&ctx->h_pin, sizeof(double) * (NU + NRD + NG + NS), cudaHostAllocPortable) !=
+          cudaSuccess) {
+    ctx->h_pin = nullptr;
+    cudaGetLastError();
+    set_error("cudaHostAlloc of the solver's exchange area failed");
+    return FORTE_ERR_ALLOC;
+  }
+  p.u = ctx->h_pin;
+  p.rd = p.u + NU;
+  p.g = p.rd + NRD;
+  p.s = p.g + NG;
+  return FORTE_OK;
+}
+
 struct DvResult {
   std::vector<double> E, rn;
   int iters = 0;
@@ -319,8 +342,8 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
   // device layout: B[maxsub], S[maxsub], T[nroots], W[keep] vectors; then small arrays
   size_t nvecs = (size_t)maxsub * 2 + nroots + keep;
   size_t small_off = ((sizeof(T) * nvecs * N + 255) / 256) * 256;
-  // coef, u, d0, d1, d2 (4416 doubles), then per root [|r|^2, B^T t, |t|^2] (66 each)
-  size_t small_bytes = sizeof(double) * (64 * 64 + 4 * 64 + 64 + 64 * 66);
+  // coef, d0, d1, d2 (4416 doubles), then u, the residual passes' results, G columns
+  size_t small_bytes = sizeof(double) * (64 * 64 + 4 * 64 + 64 + 64 * 64 + 64 * 66 + 64 * 64);
   int rc = ctx->sc_dv.ensure(small_off + small_bytes + 256);
   if (rc) return rc;
   T *B = (T *)ctx->sc_dv.ptr;
@@ -328,11 +351,14 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
   T *Tv = S + (size_t)maxsub * N;
   T *W = Tv + (size_t)nroots * N;
   double *d_coef = (double *)((char *)ctx->sc_dv.ptr + small_off);  // [64*64]
-  double *d_u = d_coef + 64 * 64;                                    // [64]
-  double *d_d0 = d_u + 64;                                           // [65]
+  double *d_d0 = d_coef + 64 * 64 + 64;                              // [65]
   double *d_d1 = d_d0 + 65;                                          // [65]
   double *d_d2 = d_d1 + 65;                                          // [65]
-  double *d_rd = d_coef + 64 * 64 + 4 * 64 + 64;                     // [64][66]
+  double *d_u = d_coef + 64 * 64 + 4 * 64 + 64;                      // [64][64]
+  double *d_rd = d_u + 64 * 64;                                      // [64][66]
+  double *d_g = d_rd + 64 * 66;                                      // [64][64]
+  PinArea pin;
+  if ((rc = pin_area(ctx, pin))) return rc;
 
   int k = 0;
   if (ng > 0) {
@@ -406,13 +432,12 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
   std::vector<double> G((size_t)64 * 64, 0.0);
   auto Gat = [&](int i, int j) -> double & { return G[(size_t)i * 64 + j]; };
   if ((rc = sigma_dispatch(ctx, B, S, k, mode))) return rc;
-  std::vector<double> h_dots(65);
-  for (int j = 0; j < k; ++j) {
-    if ((rc = vk_multidot(ctx, B, k, N, S + (size_t)j * N, N, d_d0))) return rc;
-    FORTE_CUDA_TRY(cudaMemcpyAsync(h_dots.data(), d_d0, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-    FORTE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int i = 0; i < k; ++i) Gat(i, j) = h_dots[i];
-  }
+  for (int j = 0; j < k; ++j)
+    if ((rc = vk_multidot(ctx, B, k, N, S + (size_t)j * N, N, d_g + 64 * j))) return rc;
+  FORTE_CUDA_TRY(cudaMemcpyAsync(pin.g, d_g, sizeof(double) * 64 * k, cudaMemcpyDeviceToHost, st));
+  FORTE_CUDA_TRY(cudaStreamSynchronize(st));
+  for (int j = 0; j < k; ++j)
+    for (int i = 0; i < k; ++i) Gat(i, j) = pin.g[64 * j + i];
   std::vector<double> Gk, w, U, coef;
   res.E.assign(nroots, 0.0);
   res.rn.assign(nroots, INFINITY);
@@ -431,31 +456,26 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
     // residuals and preconditioned corrections; where the packet kernel applies, the
     // same pass forms B^T t and |t|^2 for the Gram-Schmidt step of the new direction
     // (not in a spin-parity sector, where t is projected before that step)
-    std::vector<double> rn2(nroots), hrd((size_t)nroots * 66);
+    std::vector<double> rn2(nroots);
     std::vector<char> fused(nroots, 0);
-    bool any_fused = false;
+    for (int r = 0; r < nroots; ++r)
+      for (int i = 0; i < k; ++i) pin.u[64 * r + i] = U[(size_t)i * k + r];
+    FORTE_CUDA_TRY(cudaMemcpyAsync(d_u, pin.u, sizeof(double) * 64 * nroots, cudaMemcpyHostToDevice, st));
     for (int r = 0; r < nroots; ++r) {
-      std::vector<double> u(k);
-      for (int i = 0; i < k; ++i) u[i] = U[(size_t)i * k + r];
-      FORTE_CUDA_TRY(cudaMemcpyAsync(d_u, u.data(), sizeof(double) * k, cudaMemcpyHostToDevice, st));
       T *t = Tv + (size_t)r * N;
       int rr = -1;
       if (ctx->spin_parity == 0)
-        rr = vk_residual_precond(ctx, B, S, k, N, d_u, w[r], ctx->dv_guard, t, nullptr, N, d_rd + (size_t)r * 66);
+        rr = vk_residual_precond(ctx, B, S, k, N, d_u + 64 * r, w[r], ctx->dv_guard, t, nullptr, N, d_rd + 66 * r);
       if (rr == -1) {
-        rr = vk_residual_precond(ctx, B, S, k, N, d_u, w[r], ctx->dv_guard, t, d_d0 + r, N);
+        rr = vk_residual_precond(ctx, B, S, k, N, d_u + 64 * r, w[r], ctx->dv_guard, t, d_rd + 66 * r, N);
       } else if (rr == FORTE_OK) {
         fused[r] = 1;
-        any_fused = true;
       }
       if (rr) return rr;
     }
-    FORTE_CUDA_TRY(cudaMemcpyAsync(rn2.data(), d_d0, sizeof(double) * nroots, cudaMemcpyDeviceToHost, st));
-    if (any_fused)
-      FORTE_CUDA_TRY(cudaMemcpyAsync(hrd.data(), d_rd, sizeof(double) * hrd.size(), cudaMemcpyDeviceToHost, st));
+    FORTE_CUDA_TRY(cudaMemcpyAsync(pin.rd, d_rd, sizeof(double) * 66 * nroots, cudaMemcpyDeviceToHost, st));
     FORTE_CUDA_TRY(cudaStreamSynchronize(st));
-    for (int r = 0; r < nroots; ++r)
-      if (fused[r]) rn2[r] = hrd[(size_t)r * 66];
+    for (int r = 0; r < nroots; ++r) rn2[r] = pin.rd[66 * r];
     const int k_res = k;  // B[0..k_res) as the fused dots saw it
     bool all = true, bad = false;
     for (int r = 0; r < nroots; ++r) {
@@ -513,8 +533,8 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
       const T *src = b;         // vector pass 1 reads
       if (fused[r] && !collapsed && k == k_res) {
         // B^T t and |t|^2 from the residual pass: no copy pass, no host wait
-        for (int i = 0; i <= k; ++i) h0[i] = hrd[(size_t)r * 66 + 1 + i];
-        c0 = d_rd + (size_t)r * 66 + 1;
+        for (int i = 0; i <= k; ++i) h0[i] = pin.rd[66 * r + 1 + i];
+        c0 = d_rd + 66 * r + 1;
         src = t;
       } else {
         if ((rc = vk_orth_update(ctx, B, k, N, nullptr, t, b, d_d0, N))) return rc;  // copy + B^T t + |t|^2
@@ -561,12 +581,12 @@ static int davidson_run(forte_ctx *ctx, int nroots, double tol, int mode, const 
       return FORTE_OK;
     }
     if ((rc = sigma_dispatch(ctx, B + (size_t)k_old * N, S + (size_t)k_old * N, k - k_old, mode))) return rc;
-    for (int j = k_old; j < k; ++j) {
-      if ((rc = vk_multidot(ctx, B, k, N, S + (size_t)j * N, N, d_d0))) return rc;
-      FORTE_CUDA_TRY(cudaMemcpyAsync(h_dots.data(), d_d0, sizeof(double) * k, cudaMemcpyDeviceToHost, st));
-      FORTE_CUDA_TRY(cudaStreamSynchronize(st));
-      for (int i = 0; i < k; ++i) { Gat(i, j) = h_dots[i]; Gat(j, i) = h_dots[i]; }
-    }
+    for (int j = k_old; j < k; ++j)
+      if ((rc = vk_multidot(ctx, B, k, N, S + (size_t)j * N, N, d_g + 64 * (j - k_old)))) return rc;
+    FORTE_CUDA_TRY(cudaMemcpyAsync(pin.g, d_g, sizeof(double) * 64 * (k - k_old), cudaMemcpyDeviceToHost, st));
+    FORTE_CUDA_TRY(cudaStreamSynchronize(st));
+    for (int j = k_old; j < k; ++j)
+      for (int i = 0; i < k; ++i) Gat(i, j) = Gat(j, i) = pin.g[64 * (j - k_old) + i];
   }
 }
 
@@ -593,17 +613,20 @@ static int refine_jd(forte_ctx *ctx, int nroots, double tol, int inner_mode, int
   // and the inverse preconditioner diagonal
   size_t nvec = (size_t)2 * kmax + nkeep + 6;
   size_t small_off = sizeof(double) * nvec * N;
-  int rc = ctx->sc_dv.ensure(small_off + sizeof(double) * (64 * 64 + 4 * 66) + 256);
+  int rc = ctx->sc_dv.ensure(small_off + sizeof(double) * (64 * 64 + 4 * 66 + 64 * 64) + 256);
   if (rc) return rc;
   double *V = (double *)ctx->sc_dv.ptr;
   double *HV = V + (size_t)kmax * N;
   double *W = HV + (size_t)kmax * N;
   double *px = W + (size_t)nkeep * N, *pr = px + N, *pz = pr + N, *pp = pz + N, *pq = pp + N, *pinv = pq + N;
   double *d_coef = (double *)((char *)ctx->sc_dv.ptr + small_off);
-  double *d_a = d_coef + 64 * 64, *d_b = d_a + 66, *d_s = d_b + 66;
+  double *d_a = d_coef + 64 * 64, *d_b = d_a + 66, *d_s = d_b + 66, *d_g = d_s + 2 * 66;
+  PinArea pin;
+  if ((rc = pin_area(ctx, pin))) return rc;
   auto fetch = [&](const double *src, int cnt, double *dst) -> int {
-    FORTE_CUDA_TRY(cudaMemcpyAsync(dst, src, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
+    FORTE_CUDA_TRY(cudaMemcpyAsync(pin.s, src, sizeof(double) * cnt, cudaMemcpyDeviceToHost, st));
     FORTE_CUDA_TRY(cudaStreamSynchronize(st));
+    std::copy(pin.s, pin.s + cnt, dst);
     return FORTE_OK;
   };
   // project v onto the complement of V[0..nk): two classical Gram-Schmidt passes
@@ -637,11 +660,12 @@ static int refine_jd(forte_ctx *ctx, int nroots, double tol, int inner_mode, int
   for (int outer = 0;; ++outer) {
     // Rayleigh-Ritz over V[0..k)
     G.assign((size_t)k * k, 0.0);
-    for (int j = 0; j < k; ++j) {
-      if ((rc = vk_multidot(ctx, V, k, N, HV + (size_t)j * N, N, d_a))) return rc;
-      if ((rc = fetch(d_a, k, h.data()))) return rc;
-      for (int i = 0; i < k; ++i) G[(size_t)i * k + j] = h[i];
-    }
+    for (int j = 0; j < k; ++j)
+      if ((rc = vk_multidot(ctx, V, k, N, HV + (size_t)j * N, N, d_g + 64 * j))) return rc;
+    FORTE_CUDA_TRY(cudaMemcpyAsync(pin.g, d_g, sizeof(double) * 64 * k, cudaMemcpyDeviceToHost, st));
+    FORTE_CUDA_TRY(cudaStreamSynchronize(st));
+    for (int j = 0; j < k; ++j)
+      for (int i = 0; i < k; ++i) G[(size_t)i * k + j] = pin.g[64 * j + i];
     Gk.assign((size_t)k * k, 0.0);
     for (int i = 0; i < k; ++i)
       for (int j = 0; j < k; ++j) Gk[(size_t)i * k + j] = 0.5 * (G[(size_t)i * k + j] + G[(size_t)j * k + i]);
@@ -664,8 +688,8 @@ static int refine_jd(forte_ctx *ctx, int nroots, double tol, int inner_mode, int
       double *R = W + (size_t)r * N;
       FORTE_CUDA_TRY(cudaMemcpyAsync(R, HV + (size_t)r * N, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
       if ((rc = vk_axpby(ctx, -w[r], V + (size_t)r * N, 1.0, R, N))) return rc;
-      if ((rc = vk_multidot(ctx, R, 1, N, R, N, d_a))) return rc;
-      if ((rc = fetch(d_a, 1, h.data()))) return rc;
+      if ((rc = vk_multidot(ctx, R, 1, N, R, N, d_s))) return rc;
+      if ((rc = fetch(d_s, 1, h.data()))) return rc;
       res.E[r] = w[r];
       res.rn[r] = sqrt(std::max(0.0, h[0]));
       if (!isfinite(h[0]) || !isfinite(w[r])) { set_error("non-finite residual in refinement"); return FORTE_ERR_NUMERIC; }
@@ -848,6 +872,7 @@ void forte_destroy(forte_ctx *ctx) {
   for (int s = 0; s < (ctx->same_strings ? 1 : 2); ++s) {
     cudaFree(ctx->d_hd_hi[s]); cudaFree(ctx->d_hd_lo[s]); cudaFree(ctx->d_hd_t32[s]);
   }
+  if (ctx->h_pin) cudaFreeHost(ctx->h_pin);
   ctx->sc_t1.release(); ctx->sc_t2.release(); ctx->sc_dv.release();
   ctx->sc_small.release(); ctx->sc_rdm.release(); ctx->sc_mixed.release(); ctx->sc_grad.release(); ctx->sc_df.release();
   ctx->sc_rdm3.release(); ctx->sc_gas.release(); ctx->sc_spin.release(); ctx->sc_aci.release();
@@ -976,8 +1001,16 @@ int forte_davidson(forte_ctx *ctx, int nroots, double tol) {
   if (rc) return rc;
   DvResult res;
   ctx->nroots_done = 0;
-  if (ctx->precision == FORTE_FP64 || ctx->precision == FORTE_DF32 || ctx->precision == FORTE_OZ64) {
-    rc = davidson_run<double>(ctx, nroots, tol, ctx->precision, ctx->d_guess, ctx->nguess, ctx->dv_max_iter,
+  // Tiny spaces: a reduced-precision sigma saves nothing there, and the refinement's many
+  // short passes cost more than the FP64 iterations (one GB300, one root, FP64 against
+  // BF16x2: 7 orbitals with 4 + 3 electrons, 0.3 M products a sigma, 8.8 against
+  // 11.6 ms; 8 with 4 + 4, 1.9 M, 26.9 against 27.9 ms, and twice that for three roots
+  // either way).
+  const bool reduced = ctx->precision == FORTE_TF32 || ctx->precision == FORTE_BF16X2;
+  const int mode = reduced && !ctx->wait_budget && fp64_small(ctx, 1) && fp64_products(ctx) <= 1e6 ? FORTE_FP64
+                                                                                                  : ctx->precision;
+  if (mode == FORTE_FP64 || mode == FORTE_DF32 || mode == FORTE_OZ64) {
+    rc = davidson_run<double>(ctx, nroots, tol, mode, ctx->d_guess, ctx->nguess, ctx->dv_max_iter,
                               ctx->d_roots, res);
     if (rc) return mixed_status(ctx) ? FORTE_ERR_TIMEOUT : rc;  // an expired wait explains the failure
     if ((rc = mixed_status(ctx))) return rc;
@@ -991,7 +1024,7 @@ int forte_davidson(forte_ctx *ctx, int nroots, double tol) {
     if (res.converged || res.stalled) {
       // Jacobi-Davidson from the Ritz vectors, inner solves in the same arithmetic
       const int it_dl = res.iters;
-      rc = refine_jd(ctx, nroots, tol, ctx->precision, ctx->precision, ctx->d_roots, ctx->d_roots,
+      rc = refine_jd(ctx, nroots, tol, mode, mode, ctx->d_roots, ctx->d_roots,
                      std::max(1, std::min(60, ctx->dv_max_iter - it_dl)), res);
       if (rc) return mixed_status(ctx) ? FORTE_ERR_TIMEOUT : rc;
       if ((rc = mixed_status(ctx))) return rc;

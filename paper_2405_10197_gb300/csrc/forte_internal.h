@@ -163,6 +163,8 @@ struct forte_ctx {
   forte::Scratch sc_t1, sc_t2;     // sigma: transposes for the beta-beta term
   forte::Scratch sc_dv;            // Davidson subspace and work vectors
   forte::Scratch sc_small;         // small device arrays (dots, norms)
+  // page-locked host memory of the solvers' small copies (pin_area in api.cu)
+  double *h_pin = nullptr;
   unsigned *d_vk_count = nullptr;  // arrival counter of the fused reductions (zero between launches)
   forte::Scratch sc_rdm;           // RDM intermediates
   forte::Scratch sc_mixed;         // reduced-precision copies of vectors
@@ -244,6 +246,10 @@ int upload_tables(forte_ctx *ctx);
 int sigma_fp64(forte_ctx *ctx, const double *C, double *S, int nvec);
 // the same with caller-provided beta-beta scratch T1, T2 (nvec * Ndet doubles each)
 int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, double *T1, double *T2);
+// FP64 multiply-adds of one sigma vector, and whether the FP64 kernels are the better
+// choice for nvec vectors in a mode that only asks for FP64-class results
+double fp64_products(const forte_ctx *ctx);
+bool fp64_small(const forte_ctx *ctx, int nvec);
 int hdiag_build(forte_ctx *ctx);
 // FP64-class sigma in double-FP32 arithmetic (relative error ~2^-46 per term);
 // with_ab = false leaves out the alpha-beta term (same-spin terms only)

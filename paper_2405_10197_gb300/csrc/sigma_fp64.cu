@@ -337,6 +337,20 @@ __global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict_
   if (threadIdx.x < CH && Ib < NB) S[(long long)blockIdx.z * vstride + (long long)Ia * NB + Ib] += out;
 }
 
+double fp64_products(const forte_ctx *ctx) {
+  const SpinHost &A = ctx->sh[0], &B = ctx->sh[ctx->same_strings ? 0 : 1];
+  const double ka = A.nel * (ctx->n - A.nel) + 1, kb = B.nel * (ctx->n - B.nel) + 1;
+  return (double)ctx->Ndet * (ka * kb + (double)A.csr_ptr[1] + (double)B.csr_ptr[1]);
+}
+
+// The small-space FP64 kernels against the double-FP32 / digit-slice ones (one GB300, one
+// vector): 9.4 M products (9 orbitals, 5 + 4) 46 us against 75 / 110 us, 59 M (10, 5 + 5)
+// 184 against 140 / 187 us; four vectors 108 against 135 / 227 and 627 against 351 /
+// 486 us.  The line lies at 40 M in all.
+bool fp64_small(const forte_ctx *ctx, int nvec) {
+  return ctx->sd[1].ell_col && fp64_products(ctx) * nvec <= 40e6;
+}
+
 // Columns per block: as many threads share an output as leave two blocks an SM busy, and
 // 32 columns once the grid is larger than that.
 static int sm_columns(long long NA, long long NB, int nvec) {
@@ -666,6 +680,7 @@ static int df_setup(forte_ctx *ctx) {
 }
 
 int sigma_df(forte_ctx *ctx, const double *C, double *S, int nvec, bool with_ab) {
+  if (with_ab && fp64_small(ctx, nvec)) return sigma_fp64(ctx, C, S, nvec);  // faster and more exact there
   int rc = df_setup(ctx);
   if (rc) return rc;
   cudaStream_t st = ctx->stream;

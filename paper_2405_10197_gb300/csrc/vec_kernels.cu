@@ -338,7 +338,7 @@ __global__ void k_nonfinite(const double *__restrict__ x, long long n, int *flag
 // meet in shared memory, where 4 threads add one column (64 values), instead of a
 // five-step warp reduction per column.  Elements are loaded singly, so any count and
 // alignment will do.  One GB300, CAS(8,8) FP64 solve (133 iterations): residual pass 31 ->
-// 14 us, 11-vector dots 22 -> 9 us, whole solve 21.5 -> 14.0 ms.
+// 14 us, 11-vector dots 22 -> 9 us, whole solve 18.9 -> 14.0 ms.
 constexpr int VS_T = 64;
 constexpr int VS_E = 2;
 constexpr long long VS_CHUNK = VS_T * VS_E;
