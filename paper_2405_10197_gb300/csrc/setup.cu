@@ -194,22 +194,22 @@ int build_spin_tables(forte_ctx *ctx) {
   return build_one_spin(ctx, ctx->sh[1], ctx->nb);
 }
 
-// off[I]: the replacements of string I that move an electron, dealt round-robin from 16
-// buckets of pair mod 16 (list order within a bucket).  One thread per string.
+// off[I]: the replacements of string I that move an electron, dealt round-robin from 8
+// buckets of pair mod 8 (list order within a bucket).  One thread per string.
 __global__ void k_off_list(const Repl *__restrict__ list, int nk, int nko, int N, uint32_t *__restrict__ off) {
   const int I = blockIdx.x * blockDim.x + threadIdx.x;
   if (I >= N) return;
-  int cnt[16], seen[16];
-  for (int b = 0; b < 16; ++b) cnt[b] = seen[b] = 0;
+  int cnt[8], seen[8];
+  for (int b = 0; b < 8; ++b) cnt[b] = seen[b] = 0;
   const Repl *L = list + (long long)I * nk;
   for (int e = 0; e < nk; ++e)
-    if (L[e].J != I) ++cnt[L[e].pair & 15];
+    if (L[e].J != I) ++cnt[L[e].pair & 7];
   for (int e = 0; e < nk; ++e) {
     const Repl r = L[e];
     if (r.J == I) continue;
-    const int b = r.pair & 15, k = seen[b]++;
+    const int b = r.pair & 7, k = seen[b]++;
     int at = 0;
-    for (int c = 0; c < 16; ++c) at += min(cnt[c], k) + (c < b && cnt[c] > k ? 1 : 0);
+    for (int c = 0; c < 8; ++c) at += min(cnt[c], k) + (c < b && cnt[c] > k ? 1 : 0);
     off[(long long)I * nko + at] = (uint32_t)r.J | ((uint32_t)r.pair << 16) | (r.sgn < 0 ? 0x80000000u : 0u);
   }
 }

@@ -90,127 +90,104 @@ __global__ void k_transpose(const T *__restrict__ X, T *__restrict__ Y, long lon
   }
 }
 
-// ---- alpha-beta term, FP64 and double-FP32 ------------------------------------
+// ---- FP64 alpha-beta term ------------------------------------------------------
 //
 // sigma[Ia, E_rs Jb] += s F[rs][Jb], F[rs][Jb] = sum_e s_e (pq_e|rs) C[J_e, Jb].
 // The replacements that move no electron are taken together: all of Ia's read the row
 // C[Ia] and all of Jb's write Jb, so they make one row (integrals summed over the
 // orbitals of Ia) and one output (integrals summed over those of Jb, d_W).  At 7 of 14
-// orbitals 50 x 50 instead of 56 x 56 products a determinant.
-// One GB300 (kernel): FP64 CAS(12,12), 4 vectors 13.2 -> 8.9 ms; double-FP32 CAS(13; 7,5)
-// 4.06 -> 3.03 ms.
+// orbitals 50 x 50 instead of 56 x 56 products a determinant; the FP64 pipe (2 DFMA per
+// clock and SM) bounds the rest.  One GB300, CAS(12,12), 4 vectors: 13.2 -> 8.9 ms.
+// (Two replacements a thread, for two independent sums, measured 9.1 ms.)
 //
 // Shared memory: G[nk][npair] signed integral rows (row 0: the unmoved ones), row[NB] the
 // output row, D[nk][TJ] gathered rows of C.  A thread takes one (string, replacement)
 // of the tile at a time; the entry order of SpinDev::off gives the lanes' integral
 // loads different banks.
-struct AbF64 {  // bound by the FP64 pipe (2 DFMA per clock and SM)
-  using E = double;
-  static constexpr int THREADS = 256, TJ = 64;
-  double a = 0.0;
-  __device__ __forceinline__ void fma(E x, E y) { a = ::fma(x, y, a); }
-  __device__ __forceinline__ double value() const { return a; }
-  static __device__ __forceinline__ E make(double x) { return x; }
-  static __device__ __forceinline__ E neg(E x) { return -x; }
-};
+constexpr int AB_THREADS = 256;
 
-template <class OP>
-__global__ void __launch_bounds__(OP::THREADS) k_ab(const Repl *__restrict__ listA, int nkA,
-                                                    const uint32_t *__restrict__ offA, int noA,
-                                                    const uint32_t *__restrict__ offB, int noB, long long NB,
-                                                    const double *__restrict__ gpair,
-                                                    const typename OP::E *__restrict__ gE,
-                                                    const typename OP::E *__restrict__ W, int npair,
-                                                    const typename OP::E *__restrict__ C, double *__restrict__ S,
-                                                    long long vstride, int TJ) {
-  using E = typename OP::E;
-  constexpr int NT = OP::THREADS;
+__global__ void __launch_bounds__(AB_THREADS) k_ab_fp64(const uint32_t *__restrict__ strA,
+                                                        const uint32_t *__restrict__ offA, int noA,
+                                                        const uint32_t *__restrict__ offB, int noB, long long NB,
+                                                        const double *__restrict__ gpair, const double *__restrict__ W,
+                                                        int npair, const double *__restrict__ C,
+                                                        double *__restrict__ S, long long vstride, int TJ) {
   extern __shared__ double ab_smem[];
   const int nk = noA + 1;
-  double *row = ab_smem;                            // NB
-  E *G = reinterpret_cast<E *>(row + NB);           // nk * npair
-  E *D = G + (size_t)nk * npair;                    // nk * TJ
-  __shared__ int s_J[80], s_pp[16];                 // C rows; pair indices of Ia's unmoved replacements
-  __shared__ int s_np;
+  double *row = ab_smem;                   // NB
+  double *G = row + NB;                    // nk * npair
+  double *D = G + (size_t)nk * npair;      // nk * TJ
+  __shared__ int s_J[80], s_pp[16];        // C rows; pair indices of Ia's unmoved replacements
   const long long Ia = blockIdx.x;
-  const E *Cv = C + (long long)blockIdx.y * vstride;
+  const double *Cv = C + (long long)blockIdx.y * vstride;
   double *Sv = S + (long long)blockIdx.y * vstride;
   const uint32_t *la = offA + Ia * noA;
-  for (int e = threadIdx.x; e < noA; e += NT) s_J[e + 1] = la[e] & 0xFFFFu;
-  if (threadIdx.x == 0) {
-    s_J[0] = (int)Ia;
-    int m = 0;
-    for (int e = 0; e < nkA; ++e)
-      if (listA[Ia * nkA + e].J == Ia) s_pp[m++] = listA[Ia * nkA + e].pair;
-    s_np = m;
-  }
-  for (int i = threadIdx.x; i < noA * npair; i += NT) {
+  for (int e = threadIdx.x; e < noA; e += AB_THREADS) s_J[e + 1] = la[e] & 0xFFFFu;
+  const uint32_t occ = strA[Ia];
+  const int npp = __popc(occ);
+  if (threadIdx.x == 0) s_J[0] = (int)Ia;
+  if (threadIdx.x < 32 && ((occ >> threadIdx.x) & 1u))
+    s_pp[__popc(occ & ((1u << threadIdx.x) - 1u))] = threadIdx.x * (threadIdx.x + 3) / 2;  // pair (r, r)
+  for (int i = threadIdx.x; i < noA * npair; i += AB_THREADS) {
     const uint32_t w = la[i / npair];
-    const E g = gE[(size_t)((w >> 16) & 0xFFu) * npair + i % npair];
-    G[npair + i] = (w >> 31) ? OP::neg(g) : g;
+    const double g = gpair[(size_t)((w >> 16) & 0xFFu) * npair + i % npair];
+    G[npair + i] = (w >> 31) ? -g : g;
   }
-  for (long long i = threadIdx.x; i < NB; i += NT) row[i] = 0.0;
+  for (long long i = threadIdx.x; i < NB; i += AB_THREADS) row[i] = 0.0;
   __syncthreads();
-  const int npp = s_np;
-  for (int rs = threadIdx.x; rs < npair; rs += NT) {
+  for (int rs = threadIdx.x; rs < npair; rs += AB_THREADS) {
     double v = 0.0;
     for (int m = 0; m < npp; ++m) v += gpair[(size_t)s_pp[m] * npair + rs];
-    G[rs] = OP::make(v);
+    G[rs] = v;
   }
   for (long long j0 = 0; j0 < NB; j0 += TJ) {
     const int tj = (int)min((long long)TJ, NB - j0);
-    for (int i = threadIdx.x; i < nk * tj; i += NT) {
+    for (int i = threadIdx.x; i < nk * tj; i += AB_THREADS) {
       const int e = i / tj, j = i - e * tj;
       D[e * TJ + j] = Cv[(long long)s_J[e] * NB + j0 + j];
     }
     __syncthreads();
     const uint32_t *lb = offB + j0 * noB;
-    for (int w = threadIdx.x; w < tj * noB; w += NT) {
+    for (int w = threadIdx.x; w < tj * noB; w += AB_THREADS) {
       const uint32_t f = lb[w];
-      const E *g = G + ((f >> 16) & 0xFFu), *d = D + w / noB;
-      OP acc;
+      const double *g = G + ((f >> 16) & 0xFFu), *d = D + w / noB;
+      double v = 0.0;
 #pragma unroll 8
-      for (int e = 0; e < nk; ++e) acc.fma(g[e * npair], d[e * TJ]);
-      const double v = acc.value();
+      for (int e = 0; e < nk; ++e) v = fma(g[e * npair], d[e * TJ], v);
       atomicAdd(&row[f & 0xFFFFu], (f >> 31) ? -v : v);
     }
     // the unmoved replacements of the tile's strings: output j itself, rows split over
     // the threads
-    const int parts = NT / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
+    const int parts = AB_THREADS / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
     if (part < parts && j < tj) {
-      OP acc;
+      double v = 0.0;
       for (int e = 1 + part; e < nk; e += parts) {
         const uint32_t w = la[e - 1];
-        const E x = W[(size_t)((w >> 16) & 0xFFu) * NB + j0 + j];
-        acc.fma((w >> 31) ? OP::neg(x) : x, D[e * TJ + j]);
+        const double x = W[(size_t)((w >> 16) & 0xFFu) * NB + j0 + j];
+        v = fma((w >> 31) ? -x : x, D[e * TJ + j], v);
       }
-      for (int m = part; m < npp; m += parts) acc.fma(W[(size_t)s_pp[m] * NB + j0 + j], D[j]);
-      atomicAdd(&row[j0 + j], acc.value());
+      for (int m = part; m < npp; m += parts) v = fma(W[(size_t)s_pp[m] * NB + j0 + j], D[j], v);
+      atomicAdd(&row[j0 + j], v);
     }
     __syncthreads();
   }
-  for (long long i = threadIdx.x; i < NB; i += NT) Sv[Ia * NB + i] += row[i];
+  for (long long i = threadIdx.x; i < NB; i += AB_THREADS) Sv[Ia * NB + i] += row[i];
 }
 
-// Launch of k_ab; the tile narrows until the block fits.
-template <class OP>
-static int ab_launch(forte_ctx *ctx, const char *name, const typename OP::E *gE, const typename OP::E *W,
-                     const typename OP::E *C, double *S, int nvec) {
-  const int n = ctx->n, nkA = ctx->sh[0].nk, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
+static int ab_fp64(forte_ctx *ctx, const double *C, double *S, int nvec) {
+  const int n = ctx->n, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
   const long long NA = ctx->Na, NB = ctx->Nb;
-  auto bytes = [&](int TJ) {
-    return sizeof(double) * (size_t)NB + sizeof(typename OP::E) * ((size_t)(noA + 1) * (ctx->npair + TJ));
-  };
-  int TJ = OP::TJ;
+  auto bytes = [&](int TJ) { return sizeof(double) * ((size_t)NB + (size_t)(noA + 1) * (ctx->npair + TJ)); };
+  int TJ = 64;
   while (bytes(TJ) > 220 * 1024 && TJ > 8) TJ /= 2;
   if (bytes(TJ) > 220 * 1024) {
-    set_error("alpha-beta kernel %s needs %zu bytes of shared memory", name, bytes(TJ));
+    set_error("alpha-beta FP64 kernel needs %zu bytes of shared memory", bytes(TJ));
     return FORTE_ERR_ARG;
   }
-  FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab<OP>));
-  FORTE_PROF(ctx, name);
-  k_ab<OP><<<dim3((unsigned)NA, (unsigned)nvec), OP::THREADS, bytes(TJ), ctx->stream>>>(
-      ctx->sd[0].list, nkA, ctx->sd[0].off, noA, ctx->sd[1].off, noB, NB, ctx->d_gpair, gE, W, ctx->npair, C, S,
+  FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_fp64));
+  FORTE_PROF(ctx, "ab_fp64");
+  k_ab_fp64<<<dim3((unsigned)NA, (unsigned)nvec), AB_THREADS, bytes(TJ), ctx->stream>>>(
+      ctx->sd[0].str, ctx->sd[0].off, noA, ctx->sd[1].off, noB, NB, ctx->d_gpair, ctx->d_W, ctx->npair, C, S,
       ctx->Ndet, TJ);
   FORTE_LAUNCH_CHECK();
   return FORTE_OK;
@@ -221,7 +198,7 @@ static int ab_launch(forte_ctx *ctx, const char *name, const typename OP::E *gE,
 // Up to about 10 orbitals a sigma is a few microseconds of FP64 work, so the launches,
 // the idle SMs and the latency of their chains count.  Every output is gathered by a few
 // threads that split its sum and add their parts in a fixed order: no transposes, no
-// atomics, and enough blocks for every SM.  One GB300, CAS(8,8), one vector: 53 -> 25 us
+// atomics, and enough blocks for every SM.  One GB300, CAS(8,8), one vector: 53 -> 22 us
 // (the general kernels: a 70-block grid, 21 us for the alpha-beta term alone).
 
 constexpr int SM_THREADS = 256;
@@ -247,6 +224,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_ss_small(const int *__restrict__
   const int parts = SM_THREADS / CH, part = threadIdx.x / CH;
   const long long Ia = blockIdx.y, Ib = (long long)blockIdx.x * CH + threadIdx.x % CH;
   const double *Cv = C + (long long)blockIdx.z * vstride;
+  cudaTriggerProgrammaticLaunchCompletion();
   double a = 0.0;
   if (Ib < NB) {
     if (ALPHA) {
@@ -260,6 +238,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_ss_small(const int *__restrict__
     }
   }
   a = sm_sum(a, red, CH, parts);
+  if (!ALPHA) cudaGridDependencySynchronize();  // S of the kernel before
   if (threadIdx.x < CH && Ib < NB) {
     double *s = S + (long long)blockIdx.z * vstride + Ia * NB + Ib;
     *s = ALPHA ? a : *s + a;
@@ -268,7 +247,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_ss_small(const int *__restrict__
 
 // Alpha-beta part of row blockIdx.y: D holds the rows C[J_e] whole, G the signed
 // integrals, so that output Ib gathers F[rs][J] from every replacement J of Ib.
-__global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict__ listA, int nkA,
+__global__ void __launch_bounds__(SM_THREADS) k_ab_small(const uint32_t *__restrict__ strA,
                                                          const uint32_t *__restrict__ offA, int noA,
                                                          const uint32_t *__restrict__ offB, int noB, int NB,
                                                          const double *__restrict__ gpair, const double *__restrict__ W,
@@ -276,20 +255,16 @@ __global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict_
                                                          double *__restrict__ S, long long vstride, int CH) {
   extern __shared__ double ab_smem[];
   __shared__ double red[SM_THREADS];
-  __shared__ int s_pp[16], s_np;
+  __shared__ int s_pp[16];
   const int nk = noA + 1;
   double *G = ab_smem, *D = G + nk * npair;  // [nk][npair], [nk][NB]
   const int Ia = blockIdx.y;
   const double *Cv = C + (long long)blockIdx.z * vstride;
   const uint32_t *la = offA + (long long)Ia * noA;
-  if (threadIdx.x == 0) {
-    int m = 0;
-    for (int e = 0; e < nkA; ++e) {
-      const Repl r = listA[(long long)Ia * nkA + e];
-      if (r.J == Ia) s_pp[m++] = r.pair;
-    }
-    s_np = m;
-  }
+  const uint32_t occ = strA[Ia];
+  const int npp = __popc(occ);
+  if (threadIdx.x < 32 && ((occ >> threadIdx.x) & 1u))
+    s_pp[__popc(occ & ((1u << threadIdx.x) - 1u))] = threadIdx.x * (threadIdx.x + 3) / 2;  // pair (r, r)
   for (int i = threadIdx.x; i < noA * npair; i += SM_THREADS) {
     const uint32_t w = la[i / npair];
     const double g = gpair[((w >> 16) & 0xFFu) * npair + i % npair];
@@ -300,7 +275,6 @@ __global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict_
     D[i] = Cv[(long long)(e ? (int)(la[e - 1] & 0xFFFFu) : Ia) * NB + (i - e * NB)];
   }
   __syncthreads();
-  const int npp = s_np;
   for (int rs = threadIdx.x; rs < npair; rs += SM_THREADS) {
     double v = 0.0;
     for (int m = 0; m < npp; ++m) v += gpair[s_pp[m] * npair + rs];
@@ -334,6 +308,7 @@ __global__ void __launch_bounds__(SM_THREADS) k_ab_small(const Repl *__restrict_
     for (int m = part; m < npp; m += parts) out = fma(W[(long long)s_pp[m] * NB + Ib], D[Ib], out);
   }
   out = sm_sum(out, red, CH, parts);
+  cudaGridDependencySynchronize();  // S of the kernels before
   if (threadIdx.x < CH && Ib < NB) S[(long long)blockIdx.z * vstride + (long long)Ia * NB + Ib] += out;
 }
 
@@ -368,24 +343,37 @@ static int sigma_fp64_small(forte_ctx *ctx, const double *C, double *S, int nvec
   const int CH = sm_columns(NA, NB, nvec);
   const SpinDev &A = ctx->sd[0], &B = ctx->sd[1];
   const dim3 grid((unsigned)((NB + CH - 1) / CH), (unsigned)NA, (unsigned)nvec);
+  // The second and third kernel may start while the one before runs (they read C and the
+  // tables) and wait for it only where they add to S: their launch and first loads
+  // overlap its tail.
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(SM_THREADS);
+  cfg.stream = st;
   {
     FORTE_PROF(ctx, "ss_spmm");
     k_ss_small<true><<<grid, SM_THREADS, 0, st>>>(A.csr_ptr, A.csr_col, A.csr_val, 0, C, S, NB, ND, CH);
     FORTE_LAUNCH_CHECK();
   }
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
   {
     FORTE_PROF(ctx, "ss_spmm");
-    k_ss_small<false><<<grid, SM_THREADS, 0, st>>>(nullptr, B.ell_col, B.ell_val,
-                                                  ctx->sh[ctx->same_strings ? 0 : 1].csr_ptr[1], C, S, NB, ND, CH);
-    FORTE_LAUNCH_CHECK();
+    FORTE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_ss_small<false>, (const int *)nullptr, (const int *)B.ell_col,
+                                      (const double *)B.ell_val, (int)ctx->sh[ctx->same_strings ? 0 : 1].csr_ptr[1], C, S,
+                                      NB, ND, CH));
   }
   if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0) {
     const size_t smem = sizeof(double) * (size_t)(noA + 1) * (NB + ctx->npair);
     if (smem > 44 * 1024) FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_small));
+    cfg.dynamicSmemBytes = smem;
     FORTE_PROF(ctx, "ab_fp64");
-    k_ab_small<<<grid, SM_THREADS, smem, st>>>(A.list, ctx->sh[0].nk, A.off, noA, B.off, noB, (int)NB, ctx->d_gpair,
-                                              ctx->d_W, ctx->npair, C, S, ND, CH);
-    FORTE_LAUNCH_CHECK();
+    FORTE_CUDA_TRY(cudaLaunchKernelEx(&cfg, k_ab_small, (const uint32_t *)A.str, (const uint32_t *)A.off, noA,
+                                      (const uint32_t *)B.off, noB, (int)NB, (const double *)ctx->d_gpair,
+                                      (const double *)ctx->d_W, ctx->npair, C, S, ND, CH));
   }
   return FORTE_OK;
 }
@@ -443,7 +431,7 @@ int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, dou
   }
   // alpha-beta
   if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0)
-    return ab_launch<AbF64>(ctx, "ab_fp64", ctx->d_gpair, ctx->d_W, C, S, nvec);
+    return ab_fp64(ctx, C, S, nvec);
   return FORTE_OK;
 }
 
@@ -552,117 +540,316 @@ int hdiag_build(forte_ctx *ctx) {
 // times the FP64 pipe's operations, so ~12 FP32 operations per term beat one DFMA.
 // ============================================================================
 
-__device__ __forceinline__ void df_fma(float &ah, float &al, float2 a, float2 b) {
-  const float p = a.x * b.x;
-  const float pe = fmaf(a.x, b.x, -p);
-  const float c = fmaf(a.x, b.y, a.y * b.x);
-  const float s = ah + p;
-  const float bb = s - ah;
-  const float e = (ah - (s - bb)) + (p - bb);
+// Two such sums side by side in the packed FP32 instructions (add / mul / fma .f32x2), which
+// issue twice the operations of the single ones: measured on one GB300, the same-spin
+// product of one spin at CAS(14,14) takes 2.5 ms with them, 3.64 ms without.  The
+// operations and their rounding are those of a TwoSum with FMA product residual.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pk2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpk2(f32x2 v, float &a, float &b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+constexpr f32x2 F32X2_M1 = 0xBF800000BF800000ull;  // (-1, -1)
+constexpr f32x2 F32X2_SIGN = 0x8000000080000000ull;
+
+// (ah, al) += (gh + gl)(xh + xl)
+__device__ __forceinline__ void df_fma2(f32x2 &ah, f32x2 &al, f32x2 gh, f32x2 gl, f32x2 xh, f32x2 xl) {
+  const f32x2 p = mul2(gh, xh);
+  const f32x2 npe = fma2(gh ^ F32X2_SIGN, xh, p);  // p - gh xh: minus the product's residual
+  const f32x2 c = fma2(gh, xl, mul2(gl, xh));
+  const f32x2 s = add2(ah, p);
+  const f32x2 bb = fma2(ah, F32X2_M1, s);
+  const f32x2 e = add2(fma2(fma2(bb, F32X2_M1, s), F32X2_M1, ah), fma2(bb, F32X2_M1, p));
   ah = s;
-  al += e + (pe + c);
+  al = add2(al, add2(e, fma2(npe, F32X2_M1, c)));
 }
 
-// Y[c][r] = X[r][c] for an R x Cc matrix of (hi, lo) pairs per vector.
-__global__ void k_transpose_df(const float2 *__restrict__ X, float2 *__restrict__ Y, long long R, long long Cc,
-                               long long vstride) {
-  __shared__ float2 tile[32][33];
-  const float2 *Xv = X + (long long)blockIdx.z * vstride;
-  float2 *Yv = Y + (long long)blockIdx.z * vstride;
-  const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32;
+// The operands are planar: hi [rows][ld] and lo behind it, rows padded with zeros to a
+// multiple of four, so that two neighbours are one packed operand.
+__device__ __forceinline__ void df_split(double v, float &h, float &l) {
+  h = (float)v;
+  l = (float)(v - (double)h);
+}
+// FP32 to FP64 with integer operations for normal numbers (the conversion instruction
+// shares the narrow FP64 pipe).
+__device__ __forceinline__ double to_double(float x) {
+  const uint32_t b = __float_as_uint(x), e = (b >> 23) & 255u;
+  if (e == 0u || e == 255u) return (double)x;  // zero, subnormal, infinity, NaN
+  return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7FFFFFFFu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+static long long df_ld(long long ncol) { return (ncol + 3) & ~3LL; }
+
+// hi, lo [vector][R][ld] of X [vector][R][Cc].
+__global__ void k_df_split(const double *__restrict__ X, float *__restrict__ hi, float *__restrict__ lo, long long rows,
+                           long long Cc, long long ld) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < rows * ld; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / ld, c = i - r * ld;
+    float h = 0.f, l = 0.f;
+    if (c < Cc) df_split(X[r * Cc + c], h, l);
+    hi[i] = h;
+    lo[i] = l;
+  }
+}
+
+// hi, lo [vector][Cc][ld] of the transpose of X [vector][R][Cc].
+__global__ void k_df_split_t(const double *__restrict__ X, float *__restrict__ hi, float *__restrict__ lo, long long R,
+                             long long Cc, long long ld) {
+  __shared__ double tile[32][33];
+  const double *Xv = X + (long long)blockIdx.z * R * Cc;
+  const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32, o = (long long)blockIdx.z * Cc * ld;
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const long long r = r0 + i, c = c0 + threadIdx.x;
-    if (r < R && c < Cc) tile[i][threadIdx.x] = Xv[r * Cc + c];
+    tile[i][threadIdx.x] = (r < R && c < Cc) ? Xv[r * Cc + c] : 0.0;
   }
   __syncthreads();
   for (int i = threadIdx.y; i < 32; i += blockDim.y) {
     const long long c = c0 + i, r = r0 + threadIdx.x;
-    if (r < R && c < Cc) Yv[c * R + r] = tile[threadIdx.x][i];
+    if (r < ld && c < Cc) {
+      float h, l;
+      df_split(tile[threadIdx.x][i], h, l);
+      hi[o + c * ld + r] = h;
+      lo[o + c * ld + r] = l;
+    }
   }
 }
 
-// x -> (hi, lo)
-__global__ void k_df_split(const double *__restrict__ x, float2 *__restrict__ y, long long n) {
+// (hi, lo) pairs of a table
+__global__ void k_df_pairs(const double *__restrict__ x, float2 *__restrict__ y, long long n) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const double v = x[i];
-    const float h = (float)v;
-    y[i] = make_float2(h, (float)(v - (double)h));
+    float h, l;
+    df_split(x[i], h, l);
+    y[i] = make_float2(h, l);
   }
 }
 
-// Same-spin CSR product in double-FP32: Y[row, c] (+)= sum_nz val * X[col, c],
-// X and val as (hi, lo) pairs, Y FP64.  grid.x = nrow * nchunk, grid.y = vector.
-__global__ void __launch_bounds__(SS_THREADS) k_ss_spmm_df(const int *__restrict__ ptr, const int *__restrict__ col,
-                                                           const float2 *__restrict__ val, const float2 *__restrict__ X,
-                                                           double *__restrict__ Y, long long nrow, long long ncol,
-                                                           int nchunk, long long vstride, int accumulate) {
-  __shared__ int s_col[SS_SEG];
-  __shared__ float2 s_val[SS_SEG];
+// Same-spin CSR product in double-FP32: Y[row, c] = sum_nz val * X[col, c], Y FP64 [nrow][ncol].
+// grid.x = nrow * nchunk, grid.y = vector.  A thread takes four neighbouring columns (two
+// 16-byte loads a term); blockDim and nchunk are chosen so that few lanes lie beyond the
+// last column.
+constexpr int SSD_SEG = 256;  // CSR entries staged per pass
+__global__ void __launch_bounds__(256) k_ss_spmm_df(const int *__restrict__ ptr, const int *__restrict__ col,
+                                                    const float2 *__restrict__ val, const float *__restrict__ Xhi,
+                                                    const float *__restrict__ Xlo, double *__restrict__ Y,
+                                                    long long nrow, long long ncol, long long ld, int nchunk) {
+  __shared__ float2 sv[SSD_SEG];
+  __shared__ unsigned srow[SSD_SEG];  // row start in units of four columns
   const long long row = blockIdx.x / nchunk;
-  const int chunk = blockIdx.x % nchunk;
-  const float2 *Xv = X + (long long)blockIdx.y * vstride;
-  double *Yv = Y + (long long)blockIdx.y * vstride;
-  const long long c0 = (long long)chunk * SS_THREADS * SS_CPT + threadIdx.x;
-  float ah[SS_CPT], al[SS_CPT];
-#pragma unroll
-  for (int k = 0; k < SS_CPT; ++k) ah[k] = al[k] = 0.f;
+  const int chunk = blockIdx.x % nchunk, nt = blockDim.x;
+  const long long q = (long long)chunk * nt + threadIdx.x;          // columns 4q .. 4q + 3
+  const long long vo = (long long)blockIdx.y * nrow * (ld / 4), qs = min(q, ld / 4 - 1);  // (past the end: the last)
+  const ulonglong2 *hp = reinterpret_cast<const ulonglong2 *>(Xhi) + vo + qs;
+  const ulonglong2 *lp = reinterpret_cast<const ulonglong2 *>(Xlo) + vo + qs;
+  f32x2 ah0 = 0, ah1 = 0, al0 = 0, al1 = 0;
   const int b = ptr[row], e = ptr[row + 1];
-  for (int s0 = b; s0 < e; s0 += SS_SEG) {
-    const int cnt = min(SS_SEG, e - s0);
+  for (int s0 = b; s0 < e; s0 += SSD_SEG) {
+    const int cnt = min(SSD_SEG, e - s0);
     __syncthreads();
-    for (int i = threadIdx.x; i < cnt; i += SS_THREADS) {
-      s_col[i] = col[s0 + i];
-      s_val[i] = val[s0 + i];
+    for (int i = threadIdx.x; i < cnt; i += nt) {
+      sv[i] = val[s0 + i];
+      srow[i] = (unsigned)(col[s0 + i] * (ld / 4));
     }
     __syncthreads();
 #pragma unroll 4
     for (int i = 0; i < cnt; ++i) {
-      const float2 v = s_val[i];
-      const float2 *xr = Xv + (long long)s_col[i] * ncol;
-#pragma unroll
-      for (int k = 0; k < SS_CPT; ++k) {
-        const long long c = c0 + (long long)k * SS_THREADS;
-        if (c < ncol) df_fma(ah[k], al[k], v, xr[c]);
-      }
+      const float2 v = sv[i];
+      const f32x2 gh = pk2(v.x, v.x), gl = pk2(v.y, v.y);
+      const ulonglong2 h = __ldg(hp + srow[i]), l = __ldg(lp + srow[i]);
+      df_fma2(ah0, al0, gh, gl, h.x, l.x);
+      df_fma2(ah1, al1, gh, gl, h.y, l.y);
     }
   }
+  if (4 * q >= ncol) return;
+  float h[4], l[4];
+  unpk2(ah0, h[0], h[1]);
+  unpk2(ah1, h[2], h[3]);
+  unpk2(al0, l[0], l[1]);
+  unpk2(al1, l[2], l[3]);
+  double *y = Y + ((long long)blockIdx.y * nrow + row) * ncol + 4 * q;
 #pragma unroll
-  for (int k = 0; k < SS_CPT; ++k) {
-    const long long c = c0 + (long long)k * SS_THREADS;
-    if (c < ncol) {
-      double *y = Yv + row * ncol + c;
-      const double r = (double)ah[k] + (double)al[k];
-      *y = accumulate ? *y + r : r;
-    }
-  }
+  for (int k = 0; k < 4; ++k)
+    if (4 * q + k < ncol) y[k] = (double)h[k] + (double)l[k];
 }
 
-// The alpha-beta term in double-FP32 (k_ab): bound by the 13 FP32 instructions of a term
-// and its two 8-byte shared-memory loads.  16 warps and 32-string tiles: two blocks fit
-// on an SM, so the tile gathers of one overlap the products of the other.
-struct AbDf {
-  using E = float2;
-  static constexpr int THREADS = 512, TJ = 32;
-  float h = 0.f, l = 0.f;
-  __device__ __forceinline__ void fma(E x, E y) { df_fma(h, l, x, y); }
-  __device__ __forceinline__ double value() const { return (double)h + (double)l; }
-  static __device__ __forceinline__ E make(double x) {
-    const float f = (float)x;
-    return make_float2(f, (float)(x - (double)f));
+static int ss_spmm_df(forte_ctx *ctx, const SpinDev &sp, const float2 *val, const float *Xhi, const float *Xlo, double *Y,
+                      long long nrow, long long ncol, int nvec) {
+  // the block size (whole warps, 64 .. 256) with the fewest idle lanes
+  const long long ld = df_ld(ncol);
+  int nt = 256, nchunk = 1;
+  long long best = 1LL << 62;
+  for (int t = 256; t >= 64; t -= 32) {
+    const long long n = (ld / 4 + t - 1) / t;
+    if (n * t < best) {
+      best = n * t;
+      nt = t;
+      nchunk = (int)n;
+    }
   }
-  static __device__ __forceinline__ E neg(E x) { return make_float2(-x.x, -x.y); }
-};
+  FORTE_PROF(ctx, "ss_spmm_df");
+  k_ss_spmm_df<<<dim3((unsigned)(nrow * nchunk), (unsigned)nvec), nt, 0, ctx->stream>>>(sp.csr_ptr, sp.csr_col, val, Xhi,
+                                                                                        Xlo, Y, nrow, ncol, ld, nchunk);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+
+// The alpha-beta term in double-FP32 (the sums of k_ab_fp64).  A thread's sum over the rows e
+// runs as two packed ones over even and odd e, so G[pair] and D[string] hold 16-byte quads
+// (hi_e, hi_e+1, lo_e, lo_e+1), e padded with zeros to nkp, nkp / 2 odd: quads of different
+// pair mod 8 lie in different banks, the order SpinDev::off deals the replacements in.
+// Bound by those shared-memory loads and the 13 packed operations of two terms.  One
+// GB300, CAS(13; 7,5): 4.06 -> 2.69 ms.
+constexpr int AB_DF_THREADS = 512;
+__global__ void __launch_bounds__(AB_DF_THREADS) k_ab_df(const uint32_t *__restrict__ strA,
+                                                         const uint32_t *__restrict__ offA, int noA,
+                                                         const uint32_t *__restrict__ offB, int noB, long long NB,
+                                                         const double *__restrict__ gpair,
+                                                         const float2 *__restrict__ gpair2,
+                                                         const float2 *__restrict__ W2, int npair, int nkp,
+                                                         const float *__restrict__ Chi, const float *__restrict__ Clo,
+                                                         long long ld, double *__restrict__ S, long long vstride,
+                                                         int TJ) {
+  constexpr int NT = AB_DF_THREADS;
+  extern __shared__ double ab_smem[];
+  const int nk = noA + 1;
+  double *row = ab_smem;                                    // NB
+  float *G = reinterpret_cast<float *>(row + ((NB + 1) & ~1LL));  // [npair][nkp / 2] quads
+  float *D = G + 2 * (size_t)npair * nkp;                         // [TJ][nkp / 2] quads
+  // element e of row r: hi at quad(r, e), lo two floats further
+  auto quad = [nkp](int r, int e) { return (r * (nkp >> 1) + (e >> 1)) * 4 + (e & 1); };
+  __shared__ int s_J[80], s_pp[16];
+  const long long Ia = blockIdx.x;
+  const float *Ch = Chi + (long long)blockIdx.y * gridDim.x * ld, *Cl = Clo + (long long)blockIdx.y * gridDim.x * ld;
+  double *Sv = S + (long long)blockIdx.y * vstride;
+  const uint32_t *la = offA + Ia * noA;
+  for (int e = threadIdx.x; e < noA; e += NT) s_J[e + 1] = la[e] & 0xFFFFu;
+  const uint32_t occ = strA[Ia];
+  const int npp = __popc(occ);
+  if (threadIdx.x == 0) s_J[0] = (int)Ia;
+  if (threadIdx.x < 32 && ((occ >> threadIdx.x) & 1u))
+    s_pp[__popc(occ & ((1u << threadIdx.x) - 1u))] = threadIdx.x * (threadIdx.x + 3) / 2;  // pair (r, r)
+  for (int i = threadIdx.x; i < npair * (nkp - 1); i += NT) {
+    const int e = 1 + i / npair, rs = i % npair;  // (the padding rows e >= nk are zero)
+    float2 g = make_float2(0.f, 0.f);
+    if (e < nk) {
+      const uint32_t w = la[e - 1];
+      g = gpair2[(size_t)((w >> 16) & 0xFFu) * npair + rs];
+      if (w >> 31) g = make_float2(-g.x, -g.y);
+    }
+    G[quad(rs, e)] = g.x;
+    G[quad(rs, e) + 2] = g.y;
+  }
+  for (long long i = threadIdx.x; i < NB; i += NT) row[i] = 0.0;
+  for (int i = threadIdx.x; i < TJ * (nkp - nk); i += NT) {
+    const int j = i / (nkp - nk), e = nk + i % (nkp - nk);
+    D[quad(j, e)] = D[quad(j, e) + 2] = 0.f;
+  }
+  __syncthreads();
+  for (int rs = threadIdx.x; rs < npair; rs += NT) {
+    double v = 0.0;
+    for (int m = 0; m < npp; ++m) v += gpair[(size_t)s_pp[m] * npair + rs];
+    df_split(v, G[quad(rs, 0)], G[quad(rs, 0) + 2]);
+  }
+  for (long long j0 = 0; j0 < NB; j0 += TJ) {
+    const int tj = (int)min((long long)TJ, NB - j0);
+    for (int i = threadIdx.x; i < nk * tj; i += NT) {
+      const int e = i / tj, j = i - e * tj;
+      const long long at = (long long)s_J[e] * ld + j0 + j;
+      D[quad(j, e)] = Ch[at];
+      D[quad(j, e) + 2] = Cl[at];
+    }
+    __syncthreads();
+    const uint32_t *lb = offB + j0 * noB;
+    for (int w = threadIdx.x; w < tj * noB; w += NT) {
+      const uint32_t f = lb[w];
+      const ulonglong2 *g = reinterpret_cast<const ulonglong2 *>(G) + (int)((f >> 16) & 0xFFu) * (nkp / 2);
+      const ulonglong2 *d = reinterpret_cast<const ulonglong2 *>(D) + w / noB * (nkp / 2);
+      f32x2 ah = 0, al = 0;
+#pragma unroll 4
+      for (int e = 0; e < nkp / 2; ++e) {
+        const ulonglong2 x = g[e], y = d[e];
+        df_fma2(ah, al, x.x, x.y, y.x, y.y);
+      }
+      // the two sums joined in FP32 (TwoSum), one FP64 addition: a conversion or addition
+      // on the FP64 pipe takes a warp 16 clocks, as long as four terms
+      float h0, h1, l0, l1;
+      unpk2(ah, h0, h1);
+      unpk2(al, l0, l1);
+      const float h = h0 + h1, b = h - h0;
+      const double v = to_double(h) + to_double(((h0 - (h - b)) + (h1 - b)) + (l0 + l1));
+      atomicAdd(&row[f & 0xFFFFu], (f >> 31) ? -v : v);
+    }
+    // the unmoved replacements of the tile's strings: output j itself, rows split over
+    // the threads
+    const int parts = NT / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
+    if (part < parts && j < tj) {
+      f32x2 ah = 0, al = 0;
+      auto term = [&](float2 x, int e) { df_fma2(ah, al, pk2(x.x, 0.f), pk2(x.y, 0.f), pk2(D[quad(j, e)], 0.f), pk2(D[quad(j, e) + 2], 0.f)); };
+      for (int e = 1 + part; e < nk; e += parts) {
+        const uint32_t w = la[e - 1];
+        const float2 x = W2[(size_t)((w >> 16) & 0xFFu) * NB + j0 + j];
+        term((w >> 31) ? make_float2(-x.x, -x.y) : x, e);
+      }
+      for (int m = part; m < npp; m += parts) term(W2[(size_t)s_pp[m] * NB + j0 + j], 0);
+      float h, l, z;
+      unpk2(ah, h, z);
+      unpk2(al, l, z);
+      atomicAdd(&row[j0 + j], (double)h + (double)l);
+    }
+    __syncthreads();
+  }
+  for (long long i = threadIdx.x; i < NB; i += NT) Sv[Ia * NB + i] += row[i];
+}
+
+static int ab_df(forte_ctx *ctx, const float *Chi, const float *Clo, double *S, int nvec) {
+  const int n = ctx->n, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
+  const long long NA = ctx->Na, NB = ctx->Nb;
+  int nkp = (noA + 2) & ~1;
+  if ((nkp / 2) % 2 == 0) nkp += 2;
+  auto bytes = [&](int TJ) { return sizeof(double) * (((size_t)NB + 1) / 2 * 2 + (size_t)nkp * (ctx->npair + TJ)); };
+  int TJ = 64;  // (narrower where that lets a second block onto the SM)
+  if (bytes(64) > 112 * 1024 && bytes(32) <= 112 * 1024) TJ = 32;
+  while (bytes(TJ) > 220 * 1024 && TJ > 8) TJ /= 2;
+  if (bytes(TJ) > 220 * 1024) {
+    set_error("alpha-beta double-FP32 kernel needs %zu bytes of shared memory", bytes(TJ));
+    return FORTE_ERR_ARG;
+  }
+  FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_ab_df));
+  FORTE_PROF(ctx, "ab_df");
+  k_ab_df<<<dim3((unsigned)NA, (unsigned)nvec), AB_DF_THREADS, bytes(TJ), ctx->stream>>>(
+      ctx->sd[0].str, ctx->sd[0].off, noA, ctx->sd[1].off, noB, NB, ctx->d_gpair, (const float2 *)ctx->d_gpair2,
+      (const float2 *)ctx->d_W2, ctx->npair, nkp, Chi, Clo, df_ld(NB), S, ctx->Ndet, TJ);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
 
 static int df_setup(forte_ctx *ctx) {
   if (ctx->d_gpair2) return FORTE_OK;
   const int np = ctx->npair;
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gpair2, sizeof(float2) * (size_t)np * np));
-  k_df_split<<<(unsigned)std::min<long long>(((long long)np * np + 255) / 256, 1024), 256, 0, ctx->stream>>>(
+  k_df_pairs<<<(unsigned)std::min<long long>(((long long)np * np + 255) / 256, 1024), 256, 0, ctx->stream>>>(
       ctx->d_gpair, (float2 *)ctx->d_gpair2, (long long)np * np);
   FORTE_LAUNCH_CHECK();
   const long long nw = (long long)np * ctx->Nb;
   FORTE_CUDA_TRY(cudaMalloc(&ctx->d_W2, sizeof(float2) * (size_t)nw));
-  k_df_split<<<(unsigned)std::min<long long>((nw + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
+  k_df_pairs<<<(unsigned)std::min<long long>((nw + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
       ctx->d_W, (float2 *)ctx->d_W2, nw);
   FORTE_LAUNCH_CHECK();
   const int nsp = ctx->same_strings ? 1 : 2;
@@ -670,7 +857,7 @@ static int df_setup(forte_ctx *ctx) {
     const long long nnz = (long long)ctx->sh[s].csr_col.size();
     FORTE_CUDA_TRY(cudaMalloc(&ctx->d_csr_val2[s], sizeof(float2) * (size_t)std::max(1LL, nnz)));
     if (nnz > 0) {
-      k_df_split<<<(unsigned)std::min<long long>((nnz + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
+      k_df_pairs<<<(unsigned)std::min<long long>((nnz + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
           ctx->sd[s].csr_val, (float2 *)ctx->d_csr_val2[s], nnz);
       FORTE_LAUNCH_CHECK();
     }
@@ -685,50 +872,37 @@ int sigma_df(forte_ctx *ctx, const double *C, double *S, int nvec, bool with_ab)
   if (rc) return rc;
   cudaStream_t st = ctx->stream;
   const long long NA = ctx->Na, NB = ctx->Nb, ND = ctx->Ndet;
-  const size_t nf = (size_t)nvec * ND;
-  if ((rc = ctx->sc_df.ensure(sizeof(float2) * nf + 256))) return rc;
-  if ((rc = ctx->sc_t1.ensure(sizeof(float2) * nf + 256))) return rc;
-  if ((rc = ctx->sc_t2.ensure(sizeof(double) * nf + 256))) return rc;
-  float2 *C2 = (float2 *)ctx->sc_df.ptr, *T1 = (float2 *)ctx->sc_t1.ptr;
+  const long long ldb = df_ld(NB), lda = df_ld(NA);
+  const size_t nc = (size_t)nvec * NA * ldb, nt = (size_t)nvec * NB * lda;
+  if ((rc = ctx->sc_df.ensure(2 * sizeof(float) * nc + 256))) return rc;
+  if ((rc = ctx->sc_t1.ensure(2 * sizeof(float) * nt + 256))) return rc;
+  if ((rc = ctx->sc_t2.ensure(sizeof(double) * (size_t)nvec * ND + 256))) return rc;
+  float *Chi = (float *)ctx->sc_df.ptr, *Clo = Chi + nc, *Thi = (float *)ctx->sc_t1.ptr, *Tlo = Thi + nt;
   double *T2 = (double *)ctx->sc_t2.ptr;
-  const float2 *v2a = (const float2 *)ctx->d_csr_val2[0], *v2b = (const float2 *)ctx->d_csr_val2[1];
   {
     FORTE_PROF(ctx, "df_split");
-    k_df_split<<<(unsigned)std::min<size_t>((nf + 255) / 256, 152 * 16), 256, 0, st>>>(C, C2, (long long)nf);
+    k_df_split<<<(unsigned)std::min<size_t>((nc + 255) / 256, 152 * 16), 256, 0, st>>>(C, Chi, Clo, (long long)nvec * NA,
+                                                                                      NB, ldb);
     FORTE_LAUNCH_CHECK();
   }
+  if ((rc = ss_spmm_df(ctx, ctx->sd[0], (const float2 *)ctx->d_csr_val2[0], Chi, Clo, S, NA, NB, nvec))) return rc;
   {
-    const int nchunk = (int)((NB + SS_THREADS * SS_CPT - 1) / (SS_THREADS * SS_CPT));
-    dim3 grid((unsigned)(NA * nchunk), nvec);
-    FORTE_PROF(ctx, "ss_spmm_df");
-    k_ss_spmm_df<<<grid, SS_THREADS, 0, st>>>(ctx->sd[0].csr_ptr, ctx->sd[0].csr_col, v2a, C2, S, NA, NB, nchunk, ND, 0);
-    FORTE_LAUNCH_CHECK();
-  }
-  {
-    dim3 tb(32, 8);
-    dim3 g1((unsigned)((NB + 31) / 32), (unsigned)((NA + 31) / 32), nvec);
+    const dim3 tb(32, 8);
+    const dim3 g1((unsigned)((NB + 31) / 32), (unsigned)((lda + 31) / 32), nvec);
     {
       FORTE_PROF(ctx, "transpose");
-      k_transpose_df<<<g1, tb, 0, st>>>(C2, T1, NA, NB, ND);
+      k_df_split_t<<<g1, tb, 0, st>>>(C, Thi, Tlo, NA, NB, lda);
       FORTE_LAUNCH_CHECK();
     }
-    const int nchunk = (int)((NA + SS_THREADS * SS_CPT - 1) / (SS_THREADS * SS_CPT));
-    dim3 grid((unsigned)(NB * nchunk), nvec);
-    {
-      FORTE_PROF(ctx, "ss_spmm_df");
-      k_ss_spmm_df<<<grid, SS_THREADS, 0, st>>>(ctx->sd[1].csr_ptr, ctx->sd[1].csr_col, v2b, T1, T2, NB, NA, nchunk, ND,
-                                                0);
-      FORTE_LAUNCH_CHECK();
-    }
-    dim3 g2((unsigned)((NA + 31) / 32), (unsigned)((NB + 31) / 32), nvec);
+    if ((rc = ss_spmm_df(ctx, ctx->sd[1], (const float2 *)ctx->d_csr_val2[1], Thi, Tlo, T2, NB, NA, nvec))) return rc;
+    const dim3 g2((unsigned)((NA + 31) / 32), (unsigned)((NB + 31) / 32), nvec);
     {
       FORTE_PROF(ctx, "transpose");
       k_transpose<double><<<g2, tb, 0, st>>>(T2, S, NB, NA, ND, 1);
       FORTE_LAUNCH_CHECK();
     }
   }
-  if (with_ab && ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0)
-    return ab_launch<AbDf>(ctx, "ab_df", (const float2 *)ctx->d_gpair2, (const float2 *)ctx->d_W2, C2, S, nvec);
+  if (with_ab && ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0) return ab_df(ctx, Chi, Clo, S, nvec);
   return FORTE_OK;
 }
 
