@@ -1102,7 +1102,7 @@ int forte_set_gas_route(forte_ctx *ctx, int route) {
 
 int forte_get_gas_route(const forte_ctx *ctx, int *route_fp64, int *route_fp32, double *ms) {
   if (!ctx) { set_error("NULL context"); return FORTE_ERR_ARG; }
-  const bool cand = ctx->gas_on && !ctx->detmask_on && ctx->d_gas_reach;
+  const bool cand = ctx->gas_on && !ctx->detmask_on && ctx->d_gas_off;
   for (int t = 0; t < 2; ++t) {
     int r = -1;
     if (!ctx->gas_on) r = -1;

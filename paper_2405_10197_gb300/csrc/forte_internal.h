@@ -70,8 +70,8 @@ struct SpinDev {
   double *diag = nullptr;
   int *dense = nullptr;   // [N][n*n]: (J << 1) | (sgn < 0), or -1 when E_pq|I> = 0
   // the replacements that move an electron, [N][nel (n - nel)]: J | pair << 16 |
-  // (sgn < 0) << 31, ordered so that neighbouring entries have different pair mod 16
-  // (shared-memory banks of 8-byte words)
+  // (sgn < 0) << 31, ordered so that neighbouring entries have different pair mod 8
+  // (shared-memory banks of 16-byte words)
   uint32_t *off = nullptr;
   // CSR rows entry-major, [nnz][N] (small spaces only: see sigma_small)
   int *ell_col = nullptr;
@@ -182,14 +182,18 @@ struct forte_ctx {
   int *d_gas_cls[2] = {nullptr, nullptr};  // [N_alpha], [N_beta]
   int gas_nc[2] = {0, 0};
   uint8_t *d_gas_ok = nullptr;             // [gas_nc[0]][gas_nc[1]]
-  // the restricted sigma over the kept determinants only: kept alpha rows, and per
-  // alpha class the beta strings of its allowed classes (offsets [nc_alpha + 1])
+  // the restricted sigma over the kept determinants only (gas.cu): kept alpha rows, beta
+  // strings by class, their replacement lists and H_bb rows by target class
   int *d_gas_rows = nullptr;               // [gas_nrows]
   long long gas_nrows = 0;
-  int *d_gas_boff = nullptr, *d_gas_blist = nullptr;
   int gas_maxnnz = 0;                      // longest same-spin CSR row (alpha)
-  int *d_gas_coff = nullptr, *d_gas_cstr = nullptr;  // beta strings by class: [ncB + 1], [N_beta]
-  unsigned long long *d_gas_reach = nullptr;         // [ncB]: classes reached by one beta replacement
+  int *d_gas_coff = nullptr, *d_gas_cstr = nullptr;  // [ncB + 1], [N_beta]
+  uint32_t *d_gas_off = nullptr;
+  unsigned long long *d_gas_okm = nullptr;  // [alpha classes]: mask of the allowed beta classes
+  uint8_t *d_gas_tcls = nullptr, *d_gas_ccls = nullptr;
+  int *d_gas_ellc = nullptr;
+  double *d_gas_ellv = nullptr;
+  float *d_gas_ellv32 = nullptr;
   int gas_route = -1;                      // restricted sigma: -1 timed choice, 0 full grid, 1 kept only
   long long gas_ndiag = 0;                 // kept determinants with I_alpha == I_beta (n_alpha == n_beta)
   // restricted sigma path per vector type [FP64, FP32]: -1 not yet timed, 0 full

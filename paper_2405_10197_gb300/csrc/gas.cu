@@ -46,119 +46,243 @@ __global__ void k_det_fill(T *__restrict__ x, long long total, long long nd, con
     if (!mask[i % nd]) x[i] = value;
 }
 
+// ---- the restricted sigma over the kept determinants ----------------------------
+//
+// All strings of one class (per-space occupations) have the same number of single
+// replacements into every class, and the same number of same-spin Hamiltonian entries
+// from every class.  With each string's lists ordered by target class, the entries that
+// a restriction allows are therefore the same positions for every string of a class:
+// one short position list per block and class compacts the work, and every lane of a warp
+// has an allowed product to form.
+//   gas_off   [N_beta][no]: moving replacements of a beta string, by target class
+//   gas_tcls  [class][no]: target class of each position
+//   gas_ellc / gas_ellv (and FP32 values): H_bb rows by column class, entry-major within a
+//             class (base nnz coff[class], then [nnz][strings of the class])
+//   gas_ccls  [class][nnz]: column class of each position
+// Built on the device; one thread per beta string (in class order).
+constexpr int GAS_MAXCLS = 64;
+
+__global__ void k_gas_order(const uint32_t *__restrict__ off, int no, const int *__restrict__ ptr,
+                            const int *__restrict__ col, const double *__restrict__ val, int nnz,
+                            const int *__restrict__ cls, int nc, const int *__restrict__ coff,
+                            const int *__restrict__ cstr, int N, uint32_t *__restrict__ goff,
+                            uint8_t *__restrict__ tcls, int *__restrict__ ellc, double *__restrict__ ellv,
+                            float *__restrict__ ellv32, uint8_t *__restrict__ ccls, int *__restrict__ flag) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int J = cstr[i], b = cls[J], i0 = coff[b], nb = coff[b + 1] - i0, ii = i - i0;
+  int at[GAS_MAXCLS + 1];
+  auto starts = [&](auto target, int cnt) {  // counting sort: at[c] = first position of class c
+    for (int c = 0; c <= nc; ++c) at[c] = 0;
+    for (int e = 0; e < cnt; ++e) ++at[target(e) + 1];
+    for (int c = 0; c < nc; ++c) at[c + 1] += at[c];
+  };
+  auto ot = [&](int e) { return cls[off[(long long)J * no + e] & 0xFFFFu]; };
+  starts(ot, no);
+  for (int e = 0; e < no; ++e) {
+    const int c = ot(e), p = at[c]++;
+    goff[(long long)J * no + p] = off[(long long)J * no + e];
+    if (ii == 0) tcls[b * no + p] = (uint8_t)c;
+  }
+  if (ptr[J + 1] - ptr[J] != nnz) {
+    *flag = 1;
+    return;
+  }
+  auto ct = [&](int e) { return cls[col[ptr[J] + e]]; };
+  starts(ct, nnz);
+  for (int e = 0; e < nnz; ++e) {
+    const int c = ct(e), p = at[c]++;
+    const long long w = (long long)nnz * i0 + (long long)p * nb + ii;
+    ellc[w] = col[ptr[J] + e];
+    ellv[w] = val[ptr[J] + e];
+    ellv32[w] = (float)val[ptr[J] + e];
+    if (ii == 0) ccls[b * nnz + p] = (uint8_t)c;
+  }
+}
+// Every string of a class has its class's position lists (the counting argument above).
+__global__ void k_gas_check(const uint32_t *__restrict__ goff, int no, const uint8_t *__restrict__ tcls,
+                            const int *__restrict__ ellc, int nnz, const uint8_t *__restrict__ ccls,
+                            const int *__restrict__ cls, const int *__restrict__ coff, const int *__restrict__ cstr, int N,
+                            int *__restrict__ flag) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= N) return;
+  const int J = cstr[i], b = cls[J], i0 = coff[b], nb = coff[b + 1] - i0, ii = i - i0;
+  bool bad = false;
+  for (int p = 0; p < no; ++p) bad |= cls[goff[(long long)J * no + p] & 0xFFFFu] != tcls[b * no + p];
+  for (int p = 0; p < nnz; ++p) bad |= cls[ellc[(long long)nnz * i0 + (long long)p * nb + ii]] != ccls[b * nnz + p];
+  if (bad) *flag = 1;
+}
+
 constexpr int GAS_THREADS = 256;
+
+// list = the p < cnt with ok(p), ascending, compacted by warp `w` of the block; the count
+// goes to *n.  The caller synchronises before the list is read.
+template <typename F>
+__device__ __forceinline__ void gas_compact(int w, int cnt, F ok, uint16_t *list, int *n) {
+  if ((int)(threadIdx.x >> 5) != w) return;
+  const int lane = threadIdx.x & 31;
+  int m = 0;
+  for (int p0 = 0; p0 < cnt; p0 += 32) {
+    const int p = p0 + lane;
+    const bool k = p < cnt && ok(p);
+    const unsigned bal = __ballot_sync(0xffffffffu, k);
+    if (k) list[m + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)p;
+    m += __popc(bal);
+  }
+  if (lane == 0) *n = m;
+}
 
 // P H P C for the kept determinants of the kept alpha row Ia = rows[blockIdx.x]
 // (vector blockIdx.y), every other entry of S left as it is (zero).
-//  (1) alpha-beta, driven by the source beta strings: for each beta class cb whose
-//      strings carry weight (some J_k of the row, k in L(Ia), has an allowed
-//      (class(J_k), cb) pair: elsewhere C is zero) and reach an allowed output
-//      class, tiles of TJ strings Jb of that class are gathered as
-//      D[k][j] = C[J_k][Jb_j] for the allowed k only, and every replacement
-//      E_rs Jb = s I_b with an allowed output adds
-//      s * sum_k s_k (pq_k|rs) D[k][j] to the row accumulator (shared memory);
-//  (2) per kept output: the accumulator plus the same-spin CSR terms
-//      sum_Ja H_aa[Ia][Ja] C[Ja][Ib] + sum_Jb H_bb[Ib][Jb] C[Ia][Jb].
-// Each (output, replacement pair) of Eq. 1's two-body alpha-beta part is formed
-// once, and only where both its source and its output are kept.  T: FP64, or FP32
-// for the FP32 vectors of the reduced-precision phase.
+//  (1) alpha-beta, driven by the source beta strings, class by class: tiles of TJ strings Jb
+//      of class cb are gathered as D[k][j] = C[J_k][Jb_j] for the rows J_k that carry
+//      weight there (k in L(Ia) with an allowed (class(J_k), cb) pair; k = 0 stands for
+//      all replacements that move no electron, as in k_ab_fp64), and every replacement
+//      E_rs Jb = s I_b with an allowed output adds s sum_k s_k (pq_k|rs) D[k][j] to the row
+//      accumulator (shared memory); the unmoved replacements of Jb go to Jb itself
+//      with the integral sums W;
+//  (2) per kept output: the accumulator plus the same-spin terms
+//      sum_Ja H_aa[Ia][Ja] C[Ja][Ib] + sum_Jb H_bb[Ib][Jb] C[Ia][Jb] over allowed sources.
+// The FP64 pipe bounds it.  One GB300, CAS(14,14) with at most 2 holes in orbitals 0-3
+// and 2 particles in 10-13 (369,712 of 11.8 M determinants): 4.73 -> 2.80 ms (before, a lane
+// whose replacement was not allowed idled, and the same-spin sums ran over all entries).
+// T: FP64, or FP32 for the FP32 vectors of the reduced-precision phase.
 template <typename T>
 __global__ void __launch_bounds__(GAS_THREADS) k_gas_sigma(
-    const T *__restrict__ C, T *__restrict__ S, long long NB, long long vstride,
-    const Repl *__restrict__ listA, int nkA, const Repl *__restrict__ listB, int nkB,
-    const int *__restrict__ ptrA, const int *__restrict__ colA, const T *__restrict__ valA,
-    const int *__restrict__ ptrB, const int *__restrict__ colB, const T *__restrict__ valB,
-    const T *__restrict__ gpair, int npair, const int *__restrict__ clsA, const int *__restrict__ clsB,
-    const uint8_t *__restrict__ ok, int ncB, const unsigned long long *__restrict__ reachB,
-    const int *__restrict__ rows, const int *__restrict__ boff, const int *__restrict__ blist,
+    const T *__restrict__ C, T *__restrict__ S, long long NB, long long vstride, const uint32_t *__restrict__ strA,
+    const uint32_t *__restrict__ offA, int noA, const int *__restrict__ ptrA, const int *__restrict__ colA,
+    const T *__restrict__ valA, int maxnnzA, const uint32_t *__restrict__ goffB, int noB,
+    const uint8_t *__restrict__ tcls, const int *__restrict__ ellc, const T *__restrict__ ellv, int nnzB,
+    const uint8_t *__restrict__ ccls, const T *__restrict__ gpair, const double *__restrict__ W, int npair,
+    const int *__restrict__ clsA, const unsigned long long *__restrict__ okm, int ncB, const int *__restrict__ rows,
     const int *__restrict__ coff, const int *__restrict__ cstr, int TJ) {
   extern __shared__ __align__(16) uint8_t gsm[];
-  const int Ia = rows[blockIdx.x];
+  const int Ia = rows[blockIdx.x], nk = noA + 1;
   const int rb = ptrA[Ia], nnz = ptrA[Ia + 1] - rb;
-  T *Gs = (T *)gsm;                                         // [nkA][npair] signed integral rows
-  T *srow = Gs + (size_t)nkA * npair;                       // [NB] alpha-beta accumulator
-  T *D = srow + NB;                                         // [nkA][TJ] gathered C rows
-  T *sval = D + (size_t)nkA * TJ;                           // [nnz] CSR row Ia of H_aa
-  Repl *Lb = (Repl *)(((uintptr_t)(sval + nnz) + 7) & ~(uintptr_t)7);  // [TJ][nkB]
-  int *scol = (int *)(Lb + (size_t)TJ * nkB);               // [nnz]
-  int *sJ = scol + nnz;                                     // [nkA]
-  int *kcnt = sJ + nkA;                                     // [ncB]
-  uint16_t *klist = (uint16_t *)(kcnt + ncB);               // [ncB][nkA]: k * npair of the allowed k
-  uint8_t *sclsB = (uint8_t *)(klist + (size_t)ncB * nkA);  // [NB] beta classes
-  const Repl *la = listA + (long long)Ia * nkA;
-  const int ca = clsA[Ia];
-  const uint8_t *okA = ok + (size_t)ca * ncB;
-  for (int i = threadIdx.x; i < nkA * npair; i += GAS_THREADS) {
-    const int e = i / npair, rs = i % npair;
-    const Repl r = la[e];
-    const T g = gpair[(size_t)r.pair * npair + rs];
-    Gs[i] = r.sgn < 0 ? -g : g;
+  T *G = (T *)gsm;                                // [nk][npair] signed integral rows
+  T *srow = G + (size_t)nk * npair;               // [NB] alpha-beta accumulator
+  T *D = srow + NB;                               // [nk][TJ] gathered C rows
+  T *sval = D + (size_t)nk * TJ;                  // [maxnnzA] CSR row Ia of H_aa
+  int *scol = (int *)(sval + maxnnzA);            // [maxnnzA]
+  int *sJ = scol + maxnnzA;                       // [nk] rows of C
+  int *sj = sJ + nk;                              // [TJ] strings of the tile
+  // class masks (bit b: beta class b is allowed) of the rows that k and the H_aa entries read
+  unsigned long long *kmask = (unsigned long long *)(((uintptr_t)(sj + TJ) + 7) & ~(uintptr_t)7);  // [nk]
+  unsigned long long *emask = kmask + nk;         // [maxnnzA]
+  uint16_t *klist = (uint16_t *)(emask + maxnnzA);  // [nk]: allowed k
+  uint16_t *plist = klist + nk;                   // [max(noB, 1)]: allowed positions of the sources' lists
+  uint16_t *elist = plist + noB + 1;              // [maxnnzA]: allowed entries of H_aa[Ia]
+  uint16_t *flist = elist + maxnnzA;              // [nnzB]: allowed positions of H_bb rows
+  __shared__ int s_pp[16], s_n[2];
+  const uint32_t *la = offA + (long long)Ia * noA;
+  const uint32_t occ = strA[Ia];
+  const int npp = __popc(occ);
+  const unsigned long long okA = okm[clsA[Ia]];
+  if (threadIdx.x < 32 && ((occ >> threadIdx.x) & 1u))
+    s_pp[__popc(occ & ((1u << threadIdx.x) - 1u))] = threadIdx.x * (threadIdx.x + 3) / 2;  // pair (r, r)
+  for (int e = threadIdx.x; e < nk; e += GAS_THREADS) {
+    sJ[e] = e ? (int)(la[e - 1] & 0xFFFFu) : Ia;
+    kmask[e] = okm[clsA[sJ[e]]];
   }
-  for (long long i = threadIdx.x; i < NB; i += GAS_THREADS) {
-    srow[i] = T(0);
-    sclsB[i] = (uint8_t)clsB[i];
+  for (int i = threadIdx.x; i < noA * npair; i += GAS_THREADS) {
+    const uint32_t w = la[i / npair];
+    const T g = gpair[(size_t)((w >> 16) & 0xFFu) * npair + i % npair];
+    G[npair + i] = (w >> 31) ? -g : g;
   }
+  for (long long i = threadIdx.x; i < NB; i += GAS_THREADS) srow[i] = T(0);
   for (int i = threadIdx.x; i < nnz; i += GAS_THREADS) {
     sval[i] = valA[rb + i];
     scol[i] = colA[rb + i];
+    emask[i] = okm[clsA[scol[i]]];
   }
-  for (int e = threadIdx.x; e < nkA; e += GAS_THREADS) sJ[e] = la[e].J;
-  // allowed k per source beta class (ascending k: deterministic sums)
-  for (int cb = threadIdx.x; cb < ncB; cb += GAS_THREADS) {
-    int m = 0;
-    for (int e = 0; e < nkA; ++e)
-      if (ok[(size_t)clsA[la[e].J] * ncB + cb]) klist[(size_t)cb * nkA + m++] = (uint16_t)(e * npair);
-    kcnt[cb] = m;
-  }
-  unsigned long long okmask = 0ull;
-  for (int b = 0; b < ncB; ++b)
-    if (okA[b]) okmask |= 1ull << b;
   __syncthreads();
+  for (int rs = threadIdx.x; rs < npair; rs += GAS_THREADS) {
+    T v = T(0);
+    for (int m = 0; m < npp; ++m) v += gpair[(size_t)s_pp[m] * npair + rs];
+    G[rs] = v;
+  }
   const T *Cv = C + (long long)blockIdx.y * vstride;
-  T *Sv = S + (long long)blockIdx.y * vstride;
+  T *Sv = S + (long long)blockIdx.y * vstride + (long long)Ia * NB;
   for (int cb = 0; cb < ncB; ++cb) {
-    const int kc = kcnt[cb];
-    if (kc == 0 || !(reachB[cb] & okmask)) continue;
-    const uint16_t *kl = klist + (size_t)cb * nkA;
+    if (coff[cb] == coff[cb + 1]) continue;
+    __syncthreads();
+    gas_compact(0, nk, [&](int e) { return (kmask[e] >> cb) & 1ull; }, klist, &s_n[0]);
+    gas_compact(1, noB, [&](int p) { return (okA >> tcls[cb * noB + p]) & 1ull; }, plist, &s_n[1]);
+    __syncthreads();
+    const int kc = s_n[0], pc = s_n[1];
+    const bool self = (okA >> cb) & 1ull;
+    if (kc == 0 || (pc == 0 && !self)) continue;
     for (int s0 = coff[cb]; s0 < coff[cb + 1]; s0 += TJ) {
       const int tj = min(TJ, coff[cb + 1] - s0);
       __syncthreads();
       for (int i = threadIdx.x; i < kc * tj; i += GAS_THREADS) {
-        const int kk = i / tj, j = i % tj;
-        D[kk * TJ + j] = Cv[(long long)sJ[kl[kk] / npair] * NB + cstr[s0 + j]];
+        const int kk = i / tj, j = i - kk * tj;
+        D[kk * TJ + j] = Cv[(long long)sJ[klist[kk]] * NB + cstr[s0 + j]];
       }
-      for (int i = threadIdx.x; i < tj * nkB; i += GAS_THREADS)
-        Lb[i] = listB[(long long)cstr[s0 + i / nkB] * nkB + i % nkB];
+      for (int j = threadIdx.x; j < tj; j += GAS_THREADS) sj[j] = cstr[s0 + j];
       __syncthreads();
-      for (int w = threadIdx.x; w < tj * nkB; w += GAS_THREADS) {
-        const Repl rf = Lb[w];
-        if (!((okmask >> sclsB[rf.J]) & 1ull)) continue;
-        const int j = w / nkB;
-        const T *g = Gs + rf.pair;
-        const T *d = D + j;
+      for (int w = threadIdx.x; w < tj * pc; w += GAS_THREADS) {
+        const int j = w / pc;
+        const uint32_t f = goffB[(long long)sj[j] * noB + plist[w - j * pc]];
+        const T *g = G + ((f >> 16) & 0xFFu), *d = D + j;
         T acc = T(0);
-        for (int kk = 0; kk < kc; ++kk) acc += g[kl[kk]] * d[kk * TJ];
-        atomicAdd(&srow[rf.J], rf.sgn < 0 ? -acc : acc);
+#pragma unroll 4
+        for (int kk = 0; kk < kc; ++kk) acc += g[klist[kk] * npair] * d[kk * TJ];
+        atomicAdd(&srow[f & 0xFFFFu], (f >> 31) ? -acc : acc);
+      }
+      if (self) {
+        // the unmoved replacements of Jb, the rows split over the threads
+        const int parts = GAS_THREADS / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
+        if (part < parts && j < tj) {
+          T acc = T(0);
+          for (int kk = part; kk < kc; kk += parts) {
+            const int e = klist[kk];
+            const T d = D[kk * TJ + j];
+            if (e == 0) {
+              for (int m = 0; m < npp; ++m) acc += (T)W[(size_t)s_pp[m] * NB + sj[j]] * d;
+            } else {
+              const uint32_t w = la[e - 1];
+              const T x = (T)W[(size_t)((w >> 16) & 0xFFu) * NB + sj[j]];
+              acc += ((w >> 31) ? -x : x) * d;
+            }
+          }
+          atomicAdd(&srow[sj[j]], acc);
+        }
       }
     }
   }
-  __syncthreads();
-  for (int b = boff[ca] + threadIdx.x; b < boff[ca + 1]; b += GAS_THREADS) {
-    const long long Ib = blist[b];
-    T acc = srow[Ib];
-    for (int e = 0; e < nnz; ++e) acc += sval[e] * Cv[(long long)scol[e] * NB + Ib];
-    for (int f = ptrB[Ib]; f < ptrB[Ib + 1]; ++f) acc += valB[f] * Cv[(long long)Ia * NB + colB[f]];
-    Sv[(long long)Ia * NB + Ib] = acc;
+  for (int b = 0; b < ncB; ++b) {
+    const int i0 = coff[b], nb = coff[b + 1] - i0;
+    if (!((okA >> b) & 1ull) || nb == 0) continue;
+    __syncthreads();
+    gas_compact(0, nnz, [&](int e) { return (emask[e] >> b) & 1ull; }, elist, &s_n[0]);
+    gas_compact(1, nnzB, [&](int p) { return (okA >> ccls[b * nnzB + p]) & 1ull; }, flist, &s_n[1]);
+    __syncthreads();
+    const int ne = s_n[0], nf = s_n[1];
+    for (int i = threadIdx.x; i < nb; i += GAS_THREADS) {
+      const int Ib = cstr[i0 + i];
+      T acc = srow[Ib], acc2 = T(0);
+#pragma unroll 4
+      for (int e = 0; e < ne; ++e) acc += sval[elist[e]] * Cv[(long long)scol[elist[e]] * NB + Ib];
+      const int *ec = ellc + (long long)nnzB * i0 + i;
+      const T *ev = ellv + (long long)nnzB * i0 + i;
+#pragma unroll 4
+      for (int f = 0; f < nf; ++f) {
+        const long long p = (long long)flist[f] * nb;
+        acc2 += ev[p] * Cv[(long long)Ia * NB + ec[p]];
+      }
+      Sv[Ib] = acc + acc2;
+    }
   }
 }
 
-static size_t gas_smem_bytes(size_t tsz, int nkA, int nkB, int npair, long long NB, int maxnnz, int ncB, int TJ) {
-  return tsz * ((size_t)nkA * npair + NB + (size_t)nkA * TJ + maxnnz) + 8 + sizeof(Repl) * (size_t)TJ * nkB +
-         sizeof(int) * ((size_t)maxnnz + nkA + ncB) + sizeof(uint16_t) * (size_t)ncB * nkA + NB + 16;
+static size_t gas_smem_bytes(size_t tsz, int nk, int noB, int npair, long long NB, int maxnnz, int nnzB, int TJ) {
+  return tsz * ((size_t)nk * npair + NB + (size_t)nk * TJ + maxnnz) + sizeof(int) * ((size_t)maxnnz + nk + TJ) +
+         8 * ((size_t)nk + maxnnz) + sizeof(uint16_t) * ((size_t)nk + noB + 1 + maxnnz + nnzB) + 24;
 }
 
 bool gas_sparse(const forte_ctx *ctx) {
-  if (!ctx->gas_on || ctx->detmask_on || !ctx->d_gas_rows || !ctx->d_gas_reach || ctx->gas_route == 0) return false;
+  if (!ctx->gas_on || ctx->detmask_on || !ctx->d_gas_rows || !ctx->d_gas_off || ctx->gas_route == 0) return false;
   return ctx->gas_route == 1 || 4 * ctx->gas_ndet <= ctx->Ndet;
 }
 
@@ -168,18 +292,16 @@ static int gas_sigma_t(forte_ctx *ctx, const T *C, T *S, int nvec) {
   cudaStream_t st = ctx->stream;
   FORTE_CUDA_TRY(cudaMemsetAsync(S, 0, sizeof(T) * ctx->Ndet * nvec, st));
   if (ctx->gas_nrows == 0) return FORTE_OK;
-  const int nkA = ctx->sh[0].nk, nkB = ctx->sh[1].nk, np = ctx->npair, ncB = ctx->gas_nc[1];
+  const int n = ctx->n, noA = ctx->na * (n - ctx->na), noB = ctx->nb * (n - ctx->nb);
+  const int np = ctx->npair, ncB = ctx->gas_nc[1], nnzB = ctx->sh[1].csr_ptr[1];
   // the widest source tile that keeps two blocks per SM, else one
+  auto bytes = [&](int TJ) {
+    return gas_smem_bytes(sizeof(T), noA + 1, noB, np, ctx->Nb, ctx->gas_maxnnz, nnzB, TJ);
+  };
   int TJ = 64;
-  size_t smem = gas_smem_bytes(sizeof(T), nkA, nkB, np, ctx->Nb, ctx->gas_maxnnz, ncB, TJ);
-  while (TJ > 16 && smem > 113 * 1024) {
-    TJ /= 2;
-    smem = gas_smem_bytes(sizeof(T), nkA, nkB, np, ctx->Nb, ctx->gas_maxnnz, ncB, TJ);
-  }
-  while (TJ > 8 && smem > 220 * 1024) {
-    TJ /= 2;
-    smem = gas_smem_bytes(sizeof(T), nkA, nkB, np, ctx->Nb, ctx->gas_maxnnz, ncB, TJ);
-  }
+  while (TJ > 16 && bytes(TJ) > 113 * 1024) TJ /= 2;
+  while (TJ > 8 && bytes(TJ) > 220 * 1024) TJ /= 2;
+  const size_t smem = bytes(TJ);
   if (smem > 220 * 1024) {
     set_error("restricted sigma needs %zu bytes of shared memory", smem);
     return FORTE_ERR_ARG;
@@ -187,15 +309,14 @@ static int gas_sigma_t(forte_ctx *ctx, const T *C, T *S, int nvec) {
   FORTE_CUDA_TRY(set_smem_optin_max((const void *)k_gas_sigma<T>));
   const bool f32 = sizeof(T) == 4;
   const T *valA = f32 ? (const T *)(const void *)ctx->sd[0].csr_val32 : (const T *)(const void *)ctx->sd[0].csr_val;
-  const T *valB = f32 ? (const T *)(const void *)ctx->sd[1].csr_val32 : (const T *)(const void *)ctx->sd[1].csr_val;
+  const T *ellv = f32 ? (const T *)(const void *)ctx->d_gas_ellv32 : (const T *)(const void *)ctx->d_gas_ellv;
   const T *gp = f32 ? (const T *)(const void *)ctx->d_gpair32 : (const T *)(const void *)ctx->d_gpair;
   dim3 grid((unsigned)ctx->gas_nrows, (unsigned)nvec);
   FORTE_PROF(ctx, f32 ? "gas_sigma_f32" : "gas_sigma");
   k_gas_sigma<T><<<grid, GAS_THREADS, smem, st>>>(
-      C, S, ctx->Nb, ctx->Ndet, ctx->sd[0].list, nkA, ctx->sd[1].list, nkB, ctx->sd[0].csr_ptr, ctx->sd[0].csr_col,
-      valA, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col, valB, gp, np, ctx->d_gas_cls[0], ctx->d_gas_cls[1],
-      ctx->d_gas_ok, ncB, ctx->d_gas_reach, ctx->d_gas_rows, ctx->d_gas_boff, ctx->d_gas_blist, ctx->d_gas_coff,
-      ctx->d_gas_cstr, TJ);
+      C, S, ctx->Nb, ctx->Ndet, ctx->sd[0].str, ctx->sd[0].off, noA, ctx->sd[0].csr_ptr, ctx->sd[0].csr_col, valA,
+      ctx->gas_maxnnz, ctx->d_gas_off, noB, ctx->d_gas_tcls, ctx->d_gas_ellc, ellv, nnzB, ctx->d_gas_ccls, gp, ctx->d_W,
+      np, ctx->d_gas_cls[0], ctx->d_gas_okm, ncB, ctx->d_gas_rows, ctx->d_gas_coff, ctx->d_gas_cstr, TJ);
   FORTE_LAUNCH_CHECK();
   return FORTE_OK;
 }
@@ -250,13 +371,21 @@ static void gas_release(forte_ctx *ctx) {
   cudaFree(ctx->d_gas_ok);
   ctx->d_gas_ok = nullptr;
   cudaFree(ctx->d_gas_rows);
-  cudaFree(ctx->d_gas_boff);
-  cudaFree(ctx->d_gas_blist);
   cudaFree(ctx->d_gas_coff);
   cudaFree(ctx->d_gas_cstr);
-  cudaFree(ctx->d_gas_reach);
-  ctx->d_gas_rows = ctx->d_gas_boff = ctx->d_gas_blist = ctx->d_gas_coff = ctx->d_gas_cstr = nullptr;
-  ctx->d_gas_reach = nullptr;
+  cudaFree(ctx->d_gas_off);
+  cudaFree(ctx->d_gas_okm);
+  ctx->d_gas_okm = nullptr;
+  cudaFree(ctx->d_gas_tcls);
+  cudaFree(ctx->d_gas_ellc);
+  cudaFree(ctx->d_gas_ellv);
+  cudaFree(ctx->d_gas_ellv32);
+  cudaFree(ctx->d_gas_ccls);
+  ctx->d_gas_rows = ctx->d_gas_coff = ctx->d_gas_cstr = ctx->d_gas_ellc = nullptr;
+  ctx->d_gas_off = nullptr;
+  ctx->d_gas_tcls = ctx->d_gas_ccls = nullptr;
+  ctx->d_gas_ellv = nullptr;
+  ctx->d_gas_ellv32 = nullptr;
   ctx->gas_nrows = 0;
   for (int t = 0; t < 2; ++t) ctx->gas_pick[t] = ctx->gas_pick_mode[t] = -1;
   ctx->gas_on = false;
@@ -341,58 +470,79 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     return FORTE_ERR_ALLOC;
   }
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_ok, ok.data(), ok.size()));
-  // lists of the restricted sigma: kept alpha rows; per alpha class the beta strings
-  // of its allowed classes (ascending)
+  // kept alpha rows, those with the most kept beta strings first (they take longest)
   {
-    std::vector<int> rowsv, boff(ncA + 1, 0), blist;
-    for (int a = 0; a < ncA; ++a) {
-      for (long long j = 0; j < ctx->sh[1].N; ++j)
-        if (ok[(size_t)a * ncB + cls[1][j]]) blist.push_back((int)j);
-      boff[a + 1] = (int)blist.size();
-    }
-    for (long long i = 0; i < ctx->sh[0].N; ++i)
-      if (boff[cls[0][i] + 1] > boff[cls[0][i]]) rowsv.push_back((int)i);
+    std::vector<long long> kept(ncA, 0);
+    for (int a = 0; a < ncA; ++a)
+      for (int b = 0; b < ncB; ++b)
+        if (ok[(size_t)a * ncB + b]) kept[a] += cnt[1][b];
+    std::vector<int> rowsv;
     int maxnnz = 0;
-    for (long long i = 0; i < ctx->sh[0].N; ++i)
+    for (long long i = 0; i < ctx->sh[0].N; ++i) {
+      if (kept[cls[0][i]] > 0) rowsv.push_back((int)i);
       maxnnz = std::max(maxnnz, ctx->sh[0].csr_ptr[i + 1] - ctx->sh[0].csr_ptr[i]);
-    if (blist.empty()) blist.push_back(0);
-    if (cudaMalloc(&ctx->d_gas_rows, sizeof(int) * std::max<size_t>(1, rowsv.size())) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_boff, sizeof(int) * boff.size()) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_blist, sizeof(int) * blist.size()) != cudaSuccess) {
+    }
+    std::stable_sort(rowsv.begin(), rowsv.end(), [&](int x, int y) { return kept[cls[0][x]] > kept[cls[0][y]]; });
+    if (cudaMalloc(&ctx->d_gas_rows, sizeof(int) * std::max<size_t>(1, rowsv.size())) != cudaSuccess) {
       gas_release(ctx);
-      set_error("cudaMalloc of the restricted-sigma lists failed");
+      set_error("cudaMalloc of the restricted-sigma rows failed");
       return FORTE_ERR_ALLOC;
     }
     if (!rowsv.empty())
       FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_rows, rowsv.data(), sizeof(int) * rowsv.size()));
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_boff, boff.data(), sizeof(int) * boff.size()));
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_blist, blist.data(), sizeof(int) * blist.size()));
     ctx->gas_nrows = (long long)rowsv.size();
     ctx->gas_maxnnz = maxnnz;
   }
-  // per beta class its strings (ascending) and the classes its replacements reach
-  // (bit masks: the kept-only sigma needs at most 64 beta classes)
-  if (ncB <= 64) {
+  // beta strings by class (ascending), and their lists by target class
+  if (ncB <= GAS_MAXCLS) {
     const SpinHost &B = ctx->sh[1];
-    std::vector<int> coff(ncB + 1, 0), cstr;
-    for (int b = 0; b < ncB; ++b) {
-      for (long long j = 0; j < B.N; ++j)
-        if (cls[1][j] == b) cstr.push_back((int)j);
-      coff[b + 1] = (int)cstr.size();
+    std::vector<int> coff(ncB + 1, 0), cstr(B.N);
+    for (int b = 0; b < ncB; ++b) coff[b + 1] = coff[b] + (int)cnt[1][b];
+    {
+      std::vector<int> at(coff.begin(), coff.end() - 1);
+      for (long long j = 0; j < B.N; ++j) cstr[at[cls[1][j]]++] = (int)j;
     }
-    std::vector<unsigned long long> reach(ncB, 0ull);
-    for (long long j = 0; j < B.N; ++j)
-      for (int m = 0; m < B.nk; ++m) reach[cls[1][j]] |= 1ull << cls[1][B.list[(size_t)j * B.nk + m].J];
+    const int noB = ctx->nb * (n - ctx->nb), nnz = B.csr_ptr[1];
+    const size_t ell = (size_t)nnz * B.N;
+    std::vector<unsigned long long> okm(ncA, 0ull);
+    for (int a = 0; a < ncA; ++a)
+      for (int b = 0; b < ncB; ++b)
+        if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
+    int *d_flag = nullptr, flag = 0;
     if (cudaMalloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_cstr, sizeof(int) * std::max<size_t>(1, cstr.size())) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_reach, sizeof(unsigned long long) * reach.size()) != cudaSuccess) {
+        cudaMalloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)B.N * noB)) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_tcls, (size_t)ncB * noB + 1) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
+        cudaMalloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || cudaMalloc(&d_flag, sizeof(int)) != cudaSuccess) {
       gas_release(ctx);
       set_error("cudaMalloc of the restricted-sigma class lists failed");
       return FORTE_ERR_ALLOC;
     }
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size()));
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size()));
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_reach, reach.data(), sizeof(unsigned long long) * reach.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_okm, okm.data(), sizeof(okm[0]) * okm.size()));
+    FORTE_CUDA_TRY(copy_in(ctx, d_flag, &flag, sizeof(int)));
+    const unsigned nbk = (unsigned)((B.N + 63) / 64);
+    k_gas_order<<<nbk, 64, 0, ctx->stream>>>(ctx->sd[1].off, noB, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col,
+                                             ctx->sd[1].csr_val, nnz, ctx->d_gas_cls[1], ncB, ctx->d_gas_coff,
+                                             ctx->d_gas_cstr, (int)B.N, ctx->d_gas_off, ctx->d_gas_tcls, ctx->d_gas_ellc,
+                                             ctx->d_gas_ellv, ctx->d_gas_ellv32, ctx->d_gas_ccls, d_flag);
+    FORTE_LAUNCH_CHECK();
+    k_gas_check<<<nbk, 64, 0, ctx->stream>>>(ctx->d_gas_off, noB, ctx->d_gas_tcls, ctx->d_gas_ellc, nnz, ctx->d_gas_ccls,
+                                             ctx->d_gas_cls[1], ctx->d_gas_coff, ctx->d_gas_cstr, (int)B.N, d_flag);
+    FORTE_LAUNCH_CHECK();
+    FORTE_CUDA_TRY(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+    FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+    cudaFree(d_flag);
+    if (flag) {
+      gas_release(ctx);
+      set_error("internal: strings of one class differ in their replacements");
+      return FORTE_ERR_ARG;
+    }
   }
   ctx->gas_nc[0] = ncA;
   ctx->gas_nc[1] = ncB;
