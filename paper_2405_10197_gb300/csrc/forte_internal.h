@@ -139,7 +139,7 @@ struct forte_ctx {
   float *d_hd_t32[2] = {nullptr, nullptr};
   void *d_gpair2 = nullptr;                      // (hi, lo) FP32 pairs of d_gpair
   void *d_csr_val2[2] = {nullptr, nullptr};      // (hi, lo) pairs of the CSR values
-  uint16_t *d_ozT = nullptr;    // [n*n][Nb padded to 64]: E_sr |Ib> of the beta strings (RDM Gram)
+  uint16_t *d_ozT = nullptr;    // [n(n+1)/2][Nb padded to 64]: sources of the beta strings (RDM Gram)
   double *d_g1tmp = nullptr;    // 1-RDM workspace of the tensor-core 2-RDM when the caller passes none
   float gmax = 0.f;             // max |(pq|rs)| (bounds the alpha-beta fixed-point scale)
   // FP64-class tensor-core alpha-beta term: digits of the integrals

@@ -27,6 +27,11 @@
 //    the only rounding being L_7 and L_8 to even integers and L_8 to units of
 //    2^5) and flushes it to an FP64 partial sum every 16 chunks.
 //
+// A row reads one entry of C per spin: of E_rs and E_sr at most one acts on a string, so a
+// merged table (k_oz_pairT) gives its source and sign.  The producers' instruction
+// stream bounds the kernel; one lookup instead of one per orientation took CAS(14,14) from
+// 24.3 + 20.4 ms (u, v) to 17.4 + 14.1 ms and the row maxima from 4.1 to 2.9 ms.
+//
 // Kernel structure (one CTA per SM, persistent over alpha strings Ia; 20 warps):
 //   * warps 0-2 (producers) form u or v for the 64 determinants (Ia, Ib0..Ib0+63)
 //     of a chunk from the fixed-point C (alpha part: rows C[E_sr Ia, :], beta
@@ -50,7 +55,7 @@ constexpr int OZ_KC = 64;
 constexpr int OZ_SLOTS = 4;
 constexpr int OZ_PROD_WARPS = 3;
 constexpr int OZ_MMA_WARP = OZ_PROD_WARPS;  // lane 0 issues the MMAs, the warp owns TMEM
-constexpr int OZ_RB = 4;                    // rows per producer load batch
+constexpr int OZ_RB = 8;                    // rows per producer load batch
 constexpr int OZ_EPI_WARPS = 16;
 constexpr int OZ_THREADS = 32 * (OZ_PROD_WARPS + 1 + OZ_EPI_WARPS);  // 20 warps: 96 registers
 constexpr int OZ_FLUSH = 16;
@@ -99,22 +104,6 @@ __global__ void k_oz_cfix(const double *__restrict__ C, long long NA, long long 
   }
 }
 
-// T[ps][Ib] = E_sr |Ib> of the beta strings (ps = s n + r), as J | (sgn < 0) << 15,
-// 0xFFFF where it vanishes or Ib >= NB.
-__global__ void k_oz_denseT(const int *__restrict__ dense, int n2, long long NB, long long NbP,
-                            uint16_t *__restrict__ T) {
-  const long long tot = (long long)n2 * NbP;
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
-    const long long ps = i / NbP, ib = i % NbP;
-    uint16_t w = 0xFFFFu;
-    if (ib < NB) {
-      const int x = dense[ib * n2 + ps];
-      if (x >= 0) w = (uint16_t)((x >> 1) | ((x & 1) << 15));
-    }
-    T[i] = w;
-  }
-}
-
 // Row (r, s) of the u rows (gram 0) or v rows (gram 1): pairs r > s first, in
 // the order r(r-1)/2 + s, then (for u) the diagonal (r, r).
 __device__ __forceinline__ void oz_row(int a, int n, int &r, int &s) {
@@ -129,65 +118,88 @@ __device__ __forceinline__ void oz_row(int a, int n, int &r, int &s) {
   s = a - x * (x - 1) / 2;
 }
 
-// x = (E_rs C)[Ia, Ib] for a pair of columns Ib, Ib+1 in fixed point:
-// alpha part sgn C[E_sr Ia, Ib] (ea = (J << 1) | neg, or -1), beta part
-// sgn C[Ia, E_sr Ib] from the staged row (tb = the two 16-bit table entries).
-__device__ __forceinline__ void oz_pair(int ea, uint32_t tb, const long long *__restrict__ Cfix, long long NbP,
-                                        long long Ib, const long long *crow, long long &x0, long long &x1) {
-  x0 = 0;
-  x1 = 0;
-  if (ea >= 0) {
-    const longlong2 c = __ldg((const longlong2 *)(Cfix + (long long)(ea >> 1) * NbP + Ib));
-    x0 = (ea & 1) ? -c.x : c.x;
-    x1 = (ea & 1) ? -c.y : c.y;
+// The replacement of a string that row (r, s) reads: E_sr I (the term of E_rs) or, for
+// r != s, E_rs I (the term of E_sr, negative in v).  At most one of them does not vanish.
+// Returns (J << 2) | (term of E_sr) << 1 | (sgn < 0), or -1.
+__device__ __forceinline__ int oz_source(const int *__restrict__ dense_row, int n, int r, int s) {
+  int x = dense_row[s * n + r], o = 0;
+  if (x < 0 && r != s) {
+    x = dense_row[r * n + s];
+    o = 2;
   }
-  const uint32_t w0 = tb & 0xFFFFu, w1 = tb >> 16;
-  if (w0 != 0xFFFFu) {
-    const long long c = crow[w0 & 0x7FFFu];
-    x0 += (w0 & 0x8000u) ? -c : c;
-  }
-  if (w1 != 0xFFFFu) {
-    const long long c = crow[w1 & 0x7FFFu];
-    x1 += (w1 & 0x8000u) ? -c : c;
+  return x < 0 ? -1 : ((x >> 1) << 2) | o | (x & 1);
+}
+
+// T[a][Ib] = the source of row a on the beta string Ib: J | (term of E_sr) << 14 |
+// (sgn < 0) << 15, 0xFFFF where there is none or Ib >= NB.
+__global__ void k_oz_pairT(const int *__restrict__ dense, int n, int nU, long long NB, long long NbP,
+                           uint16_t *__restrict__ T) {
+  const long long tot = (long long)nU * NbP;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (long long)gridDim.x * blockDim.x) {
+    const long long ib = i % NbP;
+    uint16_t w = 0xFFFFu;
+    if (ib < NB) {
+      int r, s;
+      oz_row((int)(i / NbP), n, r, s);
+      const int x = oz_source(dense + ib * n * n, n, r, s);
+      if (x >= 0) w = (uint16_t)((x >> 2) | ((x & 2) << 13) | ((x & 1) << 15));
+    }
+    T[i] = w;
   }
 }
 
-__device__ __forceinline__ long long oz_value(int gram, int r, int s, long long xrs, long long xsr) {
-  return gram ? xrs - xsr : (r == s ? xrs : xrs + xsr);
+// The table entries of two columns with bit 15 of each as the sign in u (gram 0) or v
+// (gram 1): there the E_sr term is negative.
+__device__ __forceinline__ uint32_t oz_signs(uint32_t tb, int gram) { return gram ? tb ^ ((tb & 0x40004000u) << 1) : tb; }
+__device__ __forceinline__ long long oz_neg(long long c, uint32_t neg) {  // neg: 0 or 1
+  const long long m = -(long long)neg;
+  return (c ^ m) - m;
+}
+// Beta part of a row at one column: sgn C[Ia, J] from the staged row (w: table entry with
+// its sign in bit 15, valid).
+__device__ __forceinline__ long long oz_beta(const long long *crow, uint32_t w) {
+  return oz_neg(crow[w & 0x3FFFu], (w >> 15) & 1u);
 }
 
 // rowmax[g][a] = max over determinants of |u_a| (g = 0) and |v_a| (g = 1).
 // One block per alpha string; warp w takes the pairs r >= s with index w, w + 8, ...
-// and forms D^{rs} and D^{sr} once for both u_rs = D^{rs} + D^{sr} and
-// v_rs = D^{rs} - D^{sr} (u_rr = D^{rr}).
+// and forms u and v from the same two entries of C.
 __global__ void __launch_bounds__(256) k_oz_rowmax(const long long *__restrict__ Cfix, const int *__restrict__ denseA,
                                                    const uint16_t *__restrict__ T, int n, long long NA, long long NB,
                                                    long long NbP, unsigned long long *__restrict__ rowmax) {
   extern __shared__ long long crow[];
-  __shared__ int atab[256];
-  const int n2 = n * n, nU = n * (n + 1) / 2;
+  __shared__ int atab[128];
+  const int nU = n * (n + 1) / 2, nV = n * (n - 1) / 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (long long Ia = blockIdx.x; Ia < NA; Ia += gridDim.x) {
     __syncthreads();
     for (long long i = threadIdx.x; i < NbP; i += blockDim.x) crow[i] = Cfix[Ia * NbP + i];
-    for (int i = threadIdx.x; i < n2; i += blockDim.x) atab[i] = denseA[Ia * n2 + i];
-    __syncthreads();
-    for (int a = warp; a < nU; a += 8) {  // u row index a: pairs r > s first, then the diagonal
+    for (int a = threadIdx.x; a < nU; a += blockDim.x) {
       int r, s;
       oz_row(a, n, r, s);
-      const int e1 = atab[s * n + r], e2 = atab[r * n + s];
-      const uint16_t *t1 = T + (size_t)(s * n + r) * NbP, *t2 = T + (size_t)(r * n + s) * NbP;
+      atab[a] = oz_source(denseA + Ia * n * n, n, r, s);
+    }
+    __syncthreads();
+    for (int a = warp; a < nU; a += 8) {  // u row index a: pairs r > s first, then the diagonal
+      const int ea = atab[a];
+      const uint16_t *t = T + (size_t)a * NbP;
+      const long long *ca = Cfix + (long long)(ea >> 2) * NbP;
       unsigned long long mu = 0, mv = 0;
       for (long long Ib = 2 * lane; Ib < NB; Ib += 64) {
-        long long a0, a1, b0 = 0, b1 = 0;
-        oz_pair(e1, *(const uint32_t *)(t1 + Ib), Cfix, NbP, Ib, crow, a0, a1);
-        if (r != s) oz_pair(e2, *(const uint32_t *)(t2 + Ib), Cfix, NbP, Ib, crow, b0, b1);
-        const long long u0 = oz_value(0, r, s, a0, b0), u1 = oz_value(0, r, s, a1, b1);
-        const long long v0 = a0 - b0, v1 = a1 - b1;
-        mu = max(mu, (unsigned long long)(u0 < 0 ? -u0 : u0));
-        mu = max(mu, (unsigned long long)(u1 < 0 ? -u1 : u1));
-        mv = max(mv, (unsigned long long)(v0 < 0 ? -v0 : v0));
-        mv = max(mv, (unsigned long long)(v1 < 0 ? -v1 : v1));
+        longlong2 c = make_longlong2(0, 0);
+        if (ea >= 0) c = __ldg((const longlong2 *)(ca + Ib));
+        const uint32_t tb = *(const uint32_t *)(t + Ib);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const uint32_t w = k ? tb >> 16 : tb & 0xFFFFu;
+          const long long x = oz_neg(k ? c.y : c.x, ea & 1);
+          const long long y = w != 0xFFFFu ? oz_beta(crow, w) : 0;
+          // in v the E_sr terms change sign: |v| = |x + y| when both or neither are, else |x - y|
+          const bool flip = (((uint32_t)ea >> 1) ^ (w >> 14)) & 1u;
+          const long long u = x + y, v = flip ? x - y : u;
+          mu = max(mu, (unsigned long long)(u < 0 ? -u : u));
+          mv = max(mv, (unsigned long long)(v < 0 ? -v : v));
+        }
       }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
@@ -195,8 +207,8 @@ __global__ void __launch_bounds__(256) k_oz_rowmax(const long long *__restrict__
         mv = max(mv, __shfl_xor_sync(0xffffffffu, mv, o));
       }
       if (lane == 0 && mu) atomicMax(rowmax + a, mu);
-      // the v rows are the pairs r > s in the same order (index a < n(n-1)/2)
-      if (lane == 0 && mv && r != s) atomicMax(rowmax + 128 + a, mv);
+      // the v rows are the pairs r > s in the same order
+      if (lane == 0 && mv && a < nV) atomicMax(rowmax + 128 + a, mv);
     }
   }
 }
@@ -292,10 +304,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sm = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   long long *crow = (long long *)(sm + L::OFF_CROW);
-  int *atab = (int *)(crow + NbP);
-  uint8_t *sR = (uint8_t *)(atab + 256);
-  uint8_t *sS = sR + 128;
-  int *sSh = (int *)(sS + 128);
+  int *atab = (int *)(crow + NbP);  // [128]: alpha source of each row, (J << 1) | negative, or -1
+  int *sSh = atab + 128;
   uint64_t *bar = (uint64_t *)(sSh + 128);
   uint64_t *full = bar, *empty = bar + 2, *tfull = bar + 4, *tempty = bar + 4 + OZ_SLOTS;
   uint64_t *rowbar = tempty + OZ_SLOTS;  // producer warps: staged row in use / ready
@@ -322,13 +332,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     abort_word_init(sAbort, err);
     fence_mbar_init();
   }
-  if (tid < 128) {
-    int r = 0, s = 0;
-    if (tid < nrows) oz_row(tid, n, r, s);
-    sR[tid] = (uint8_t)r;
-    sS[tid] = (uint8_t)s;
-    sSh[tid] = tid < nrows ? shv[gram * 128 + tid] : 0;
-  }
+  if (tid < 128) sSh[tid] = tid < nrows ? shv[gram * 128 + tid] : 0;
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -355,7 +359,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
       }
       for (long long i = tid; i < NbP / 2; i += 32 * OZ_PROD_WARPS)
         ((longlong2 *)crow)[i] = __ldg((const longlong2 *)(Cfix + Ia * NbP) + i);
-      for (int i = tid; i < n2; i += 32 * OZ_PROD_WARPS) atab[i] = denseA[Ia * n2 + i];
+      for (int a = tid; a < nrows; a += 32 * OZ_PROD_WARPS) {
+        int r, s;
+        oz_row(a, n, r, s);
+        const int x = oz_source(denseA + Ia * n2, n, r, s);
+        atab[a] = x < 0 ? -1 : ((x >> 2) << 1) | ((x ^ (gram ? x >> 1 : 0)) & 1);
+      }
       if (!meet()) {
         ok = false;
         break;
@@ -373,54 +382,31 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // rows a = warp + PW (b + RB c): the global loads of RB rows are issued
         // together, then the rows are formed, digited and stored
         for (int a0 = warp; a0 < nrows; a0 += OZ_PROD_WARPS * OZ_RB) {
-          int ea[OZ_RB][2];
-          uint32_t tb[OZ_RB][2];
-          longlong2 ca[OZ_RB][2];
+          int ea[OZ_RB];
+          uint32_t tb[OZ_RB];
+          longlong2 ca[OZ_RB];
 #pragma unroll
           for (int b = 0; b < OZ_RB; ++b) {
             const int a = a0 + OZ_PROD_WARPS * b;
-#pragma unroll
-            for (int o = 0; o < 2; ++o) {
-              ea[b][o] = -1;
-              tb[b][o] = 0xFFFFFFFFu;
-              ca[b][o] = make_longlong2(0, 0);
-            }
+            ea[b] = -1;
+            tb[b] = 0xFFFFFFFFu;
+            ca[b] = make_longlong2(0, 0);
             if (a < nrows) {
-              const int r = sR[a], s = sS[a];
-#pragma unroll
-              for (int o = 0; o < 2; ++o) {
-                if (o == 1 && r == s) break;
-                const int ps = o ? r * n + s : s * n + r;
-                ea[b][o] = atab[ps];
-                tb[b][o] = __ldg((const uint32_t *)(T + (size_t)ps * NbP + Ib));
-                if (ea[b][o] >= 0) ca[b][o] = __ldg((const longlong2 *)(Cfix + (long long)(ea[b][o] >> 1) * NbP + Ib));
-              }
+              ea[b] = atab[a];
+              tb[b] = __ldg((const uint32_t *)(T + (size_t)a * NbP + Ib));
+              if (ea[b] >= 0) ca[b] = __ldg((const longlong2 *)(Cfix + (long long)(ea[b] >> 1) * NbP + Ib));
             }
           }
 #pragma unroll
           for (int b = 0; b < OZ_RB; ++b) {
             const int a = a0 + OZ_PROD_WARPS * b;
             if (a >= nrows) break;
-            const int r = sR[a], s = sS[a];
-            long long x[2][2];
-#pragma unroll
-            for (int o = 0; o < 2; ++o) {
-              const bool neg = ea[b][o] & 1;
-              x[o][0] = neg ? -ca[b][o].x : ca[b][o].x;
-              x[o][1] = neg ? -ca[b][o].y : ca[b][o].y;
-              const uint32_t w0 = tb[b][o] & 0xFFFFu, w1 = tb[b][o] >> 16;
-              if (w0 != 0xFFFFu) {
-                const long long c = crow[w0 & 0x7FFFu];
-                x[o][0] += (w0 & 0x8000u) ? -c : c;
-              }
-              if (w1 != 0xFFFFu) {
-                const long long c = crow[w1 & 0x7FFFu];
-                x[o][1] += (w1 & 0x8000u) ? -c : c;
-              }
-            }
+            const uint32_t neg = ea[b] & 1, sg = oz_signs(tb[b], gram);
+            long long x0 = oz_neg(ca[b].x, neg), x1 = oz_neg(ca[b].y, neg);
+            if ((tb[b] & 0xFFFFu) != 0xFFFFu) x0 += oz_beta(crow, sg & 0xFFFFu);
+            if ((tb[b] >> 16) != 0xFFFFu) x1 += oz_beta(crow, sg >> 16);
             const int sh = sSh[a];
-            const long long X0 = oz_scale(oz_value(gram, r, s, x[0][0], x[1][0]), sh);
-            const long long X1 = oz_scale(oz_value(gram, r, s, x[0][1], x[1][1]), sh);
+            const long long X0 = oz_scale(x0, sh), X1 = oz_scale(x1, sh);
             uint32_t w[OZ_DIGITS];
             oz_digits2(X0, X1, w);
             uint8_t *dst = stage + swz((uint32_t)a, 4u * lane);
@@ -588,7 +574,7 @@ static int oz_pad16(int x) { return ((x + 15) / 16) * 16; }
 
 template <int N>
 static size_t oz_smem(long long NbP) {
-  return 1024 + (size_t)OzLayout<N>::OFF_CROW + 8 * (size_t)NbP + 4 * 256 + 128 + 128 + 4 * 128 +
+  return 1024 + (size_t)OzLayout<N>::OFF_CROW + 8 * (size_t)NbP + 4 * 128 + 4 * 128 +
          8 * (5 + 2 * OZ_SLOTS) + 32;
 }
 
@@ -607,7 +593,7 @@ static size_t oz_smem_n(int N, long long NbP) {
 
 bool rdm2_oz_supported(const forte_ctx *ctx) {
   const int n = ctx->n;
-  if (n < 2 || n > 15 || ctx->Nb >= 32768 || ctx->Na < 1) return false;
+  if (n < 2 || n > 15 || ctx->Nb >= 16384 || ctx->Na < 1) return false;
   const long long NbP = (ctx->Nb + OZ_KC - 1) / OZ_KC * OZ_KC;
   const size_t lim = 232448;
   return oz_smem_n(oz_pad16(n * (n + 1) / 2), NbP) <= lim && oz_smem_n(oz_pad16(std::max(1, n * (n - 1) / 2)), NbP) <= lim;
@@ -653,10 +639,10 @@ int rdm2_oz(forte_ctx *ctx, const double *C, const double *g1, double *g2) {
     if (rc_err) return rc_err;
   }
   if (!ctx->d_ozT) {
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozT, sizeof(uint16_t) * (size_t)n2 * NbP));
-    FORTE_PROF(ctx, "oz_denseT");
-    k_oz_denseT<<<(unsigned)std::min<long long>(((long long)n2 * NbP + 255) / 256, 152LL * 32), 256, 0, st>>>(
-        ctx->sd[1].dense, n2, NB, NbP, ctx->d_ozT);
+    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozT, sizeof(uint16_t) * (size_t)nU * NbP));
+    FORTE_PROF(ctx, "oz_pairT");
+    k_oz_pairT<<<(unsigned)std::min<long long>(((long long)nU * NbP + 255) / 256, 152LL * 32), 256, 0, st>>>(
+        ctx->sd[1].dense, n, nU, NB, NbP, ctx->d_ozT);
     FORTE_LAUNCH_CHECK();
   }
   // workspace: Cfix, max |C|, row maxima, shifts, partial Grams, G+, G-
