@@ -310,9 +310,21 @@ int vk_scale(forte_ctx *ctx, float *x, const float *src, double alpha, long long
 int vk_convert(forte_ctx *ctx, const double *x, float *y, long long n);
 int vk_convert(forte_ctx *ctx, const float *x, double *y, long long n);
 int vk_axpby(forte_ctx *ctx, double a, const double *x, double b, double *y, long long n);
-// rinv = 1 / max(|theta - H_II|, guard); z = r * rinv with dot_out = [r . z, r . r]
+// rinv = 1 / max(|theta - H_II|, guard)
 int vk_precond_inv(forte_ctx *ctx, double theta, double guard, double *rinv, long long n);
-int vk_precond_dot(forte_ctx *ctx, const double *r, const double *rinv, double *z, double *dot_out, long long n);
+// passes of the conjugate-gradient correction solve (V: nk vectors, leading dimension n):
+// q -= theta p, out = V^T q
+int vk_jd_shift(forte_ctx *ctx, double *q, const double *p, double theta, const double *V, int nk, long long n,
+                double *out);
+// q -= V c, out = p . q
+int vk_jd_project(forte_ctx *ctx, double *q, const double *p, const double *V, int nk, const double *c, long long n,
+                  double *out);
+// x += alpha p, r -= alpha q, z = r * rinv, out = [r . z, r . r, V^T z]
+int vk_jd_step(forte_ctx *ctx, double alpha, const double *p, const double *q, double *x, double *r, const double *rinv,
+               double *z, const double *V, int nk, long long n, double *out);
+// p = (z - V d) + beta p
+int vk_jd_turn(forte_ctx *ctx, double *p, const double *z, double beta, const double *V, int nk, const double *d,
+               long long n);
 int vk_argmin_k(forte_ctx *ctx, const double *x, long long n, int k, long long *idx_out);
 int vk_any_nonfinite(forte_ctx *ctx, const double *x, long long n, int *flag_host);
 

@@ -3,6 +3,8 @@
 // operands once; reductions go through per-block partial sums (FP64) and a second
 // pass, so results do not depend on atomic ordering.  FP32 kernels accumulate in
 // FP32 within a warp and in FP64 across warps and blocks.
+#include <type_traits>
+
 #include "forte_internal.h"
 
 namespace forte {
@@ -238,33 +240,6 @@ __global__ void k_axpby(double a, const double *__restrict__ x, double b, double
     y[j] = a * x[j] + b * y[j];
 }
 
-// z = r * rinv (the inverse of the preconditioner's diagonal); out = [r . z, r . r]
-__global__ void __launch_bounds__(VK_THREADS) k_precond_dot(const double *__restrict__ r, const double *__restrict__ rinv,
-                                                            double *__restrict__ z, long long n,
-                                                            double *__restrict__ part, double *__restrict__ out,
-                                                            unsigned *counter) {
-  __shared__ double red[32];
-  const long long base = (long long)blockIdx.x * VK_CHUNK + threadIdx.x;
-  double acc = 0.0, rr = 0.0;
-#pragma unroll 4
-  for (int e = 0; e < VK_EPT; ++e) {
-    long long j = base + (long long)e * VK_THREADS;
-    if (j >= n) break;
-    const double rv = r[j];
-    const double zv = rv * rinv[j];
-    z[j] = zv;
-    acc += rv * zv;
-    rr += rv * rv;
-  }
-  acc = block_sum(acc, red);
-  rr = block_sum(rr, red);
-  if (threadIdx.x == 0) {
-    part[2 * blockIdx.x] = acc;
-    part[2 * blockIdx.x + 1] = rr;
-  }
-  last_block_sums(part, 2, out, counter);
-}
-
 // rinv = 1 / |theta - hdiag| with the magnitude clamped below at guard: the FP64
 // divisions of the diagonal preconditioner, done once per correction solve (the FP64
 // pipe of this GPU makes a division per element and application the bound otherwise)
@@ -479,27 +454,6 @@ __global__ void __launch_bounds__(VS_T) k_residual_precond_s(const T *__restrict
     vs_dots(r, B, k, ld, hx, j0, n, 1, m, part);
   }
   last_block_sums(part, m, out, counter);
-}
-
-// z = r * rinv; out = [r . z, r . r]
-__global__ void __launch_bounds__(VS_T) k_precond_dot_s(const double *__restrict__ rv, const double *__restrict__ rinv,
-                                                        double *__restrict__ z, long long n, double *__restrict__ part,
-                                                        double *__restrict__ out, unsigned *counter) {
-  __shared__ VsRed r;
-  const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
-  double rz = 0.0, rr = 0.0;
-#pragma unroll
-  for (int e = 0; e < VS_E; ++e)
-    if (j0 + e * VS_T < n) {
-      const double x = rv[j0 + e * VS_T], y = x * rinv[j0 + e * VS_T];
-      z[j0 + e * VS_T] = y;
-      rz = fma(x, y, rz);
-      rr = fma(x, x, rr);
-    }
-  r.v[0][threadIdx.x] = rz;
-  r.v[1][threadIdx.x] = rr;
-  vs_columns(r, 0, 2, 2, part);
-  last_block_sums(part, 2, out, counter);
 }
 
 // ------------------------------------------------------------------ packet kernels
@@ -1036,42 +990,6 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_u(
   last_block_sums(part, m, out, counter);
 }
 
-// z = r * rinv; out[0] = r . z, out[1] = r . r
-__global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_precond_dot_p(const double *__restrict__ r,
-                                                                      const double *__restrict__ rinv,
-                                                                      double *__restrict__ z, long long np,
-                                                                      double *__restrict__ part, double *__restrict__ out,
-                                                                      unsigned *counter) {
-  __shared__ double sw[2 * VP_WARPS];
-  if (threadIdx.x < 2 * VP_WARPS) sw[threadIdx.x] = 0.0;
-  __syncthreads();
-  const long long nch = (np + VP_CH - 1) / VP_CH;
-  for (long long ch = blockIdx.x; ch < nch; ch += gridDim.x) {
-    const long long q0 = ch * VP_CH + threadIdx.x;
-    double acc = 0.0, rr = 0.0;
-#pragma unroll
-    for (int e = 0; e < VP_PER; ++e) {
-      const long long q = q0 + (long long)e * VK_THREADS;
-      if (q < np) {
-        double rv[2], iv[2], zv[2];
-        pk_ld(r, q, rv);
-        pk_ld(rinv, q, iv);
-#pragma unroll
-        for (int p = 0; p < 2; ++p) {
-          zv[p] = rv[p] * iv[p];
-          acc += rv[p] * zv[p];
-          rr += rv[p] * rv[p];
-        }
-        pk_st(z, q, zv);
-      }
-    }
-    warp_add(acc, sw);
-    warp_add(rr, sw + VP_WARPS);
-  }
-  block_partials(sw, 2, part);
-  last_block_sums(part, 2, out, counter);
-}
-
 // y = a x + b y and x = alpha src over packets (grid-stride).  With a or b equal to 1
 // the update is one fused multiply-add per element (the FP64 pipe is the bound of
 // these kernels on this GPU, not HBM).
@@ -1097,6 +1015,179 @@ __global__ void k_scale_p(T *x, const T *src, double alpha, long long np) {
 #pragma unroll
     for (int p = 0; p < P; ++p) v[p] = al * v[p];
     pk_st(x, q, v);
+  }
+}
+
+// ------------------------------------------------------------------ correction solve
+// One step of the preconditioned conjugate gradients on P (H - theta) P t = -r of the
+// Jacobi-Davidson refinement (P projects out V_0 .. V_nk-1) in four passes, FP64:
+//   shift    q -= theta p,                 out = V^T q
+//   project  q -= V c,                     out = p . q
+//   step     x += alpha p, r -= alpha q, z = r * rinv,   out = [r . z, r . r, V^T z]
+//   turn     p = (z - V d) + beta p
+// 21 vector reads and writes at nk = 1, where a kernel per operation with two
+// Gram-Schmidt passes per projection took 36 and twelve launches.  One pass is enough
+// here: it leaves 2^-53 of the vector, and the solve is stopped at a 50th of its start.
+// VEC: elements a thread takes at a time (2: 16-byte loads, for even counts).  Sums: per
+// thread, then a warp adds a column of the block's threads from shared memory, then
+// last_block_sums.  One GB300, CAS(14,14), one root: 0.70 -> 0.36 ms an inner iteration.
+constexpr int JD_T = 256;
+constexpr int JD_COLS = 8;  // columns reduced at a time
+
+template <int VEC>
+struct JdV {
+  double v[VEC];
+};
+template <int VEC>
+__device__ __forceinline__ JdV<VEC> jd_ld(const double *p, long long i) {
+  JdV<VEC> r;
+  if constexpr (VEC == 2) {
+    const double2 t = reinterpret_cast<const double2 *>(p)[i];
+    r.v[0] = t.x;
+    r.v[1] = t.y;
+  } else {
+    r.v[0] = p[i];
+  }
+  return r;
+}
+template <int VEC>
+__device__ __forceinline__ void jd_st(double *p, long long i, const JdV<VEC> &x) {
+  if constexpr (VEC == 2)
+    reinterpret_cast<double2 *>(p)[i] = make_double2(x.v[0], x.v[1]);
+  else
+    p[i] = x.v[0];
+}
+
+// part[block][c] = sum of the block's acc[c], c < m <= M; then the last block's totals.
+template <int M>
+__device__ __forceinline__ void jd_reduce(const double (&acc)[M], int m, double *part, double *out, unsigned *counter) {
+  __shared__ double red[JD_COLS][JD_T + 1];
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+#pragma unroll
+  for (int c0 = 0; c0 < M; c0 += JD_COLS) {
+    if (c0 < m) {
+      __syncthreads();
+#pragma unroll
+      for (int c = 0; c < JD_COLS; ++c)
+        if (c0 + c < M) red[c][threadIdx.x] = acc[c0 + c < M ? c0 + c : 0];
+      __syncthreads();
+      for (int c = threadIdx.x >> 5; c < JD_COLS && c0 + c < m; c += warps) {
+        double t = 0.0;
+        for (int k = lane; k < (int)blockDim.x; k += 32) t += red[c][k];
+        t = warp_sum(t);
+        if (lane == 0) part[(long long)blockIdx.x * m + c0 + c] = t;
+      }
+    }
+  }
+  last_block_sums(part, m, out, counter);
+}
+
+template <int VEC, int KM>
+__global__ void __launch_bounds__(JD_T) k_jd_shift(double *__restrict__ q, const double *__restrict__ p, double theta,
+                                                   const double *__restrict__ V, int nk, long long ld, long long n,
+                                                   double *__restrict__ part, double *__restrict__ out,
+                                                   unsigned *counter) {
+  double acc[KM];
+#pragma unroll
+  for (int k = 0; k < KM; ++k) acc[k] = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    JdV<VEC> y = jd_ld<VEC>(q, i);
+    const JdV<VEC> x = jd_ld<VEC>(p, i);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) y.v[e] = fma(-theta, x.v[e], y.v[e]);
+    jd_st<VEC>(q, i, y);
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      if (k < nk) {
+        const JdV<VEC> b = jd_ld<VEC>(V + (long long)k * ld, i);
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) acc[k] = fma(b.v[e], y.v[e], acc[k]);
+      }
+  }
+  jd_reduce(acc, nk, part, out, counter);
+}
+
+template <int VEC, int KM>
+__global__ void __launch_bounds__(JD_T) k_jd_project(double *__restrict__ q, const double *__restrict__ p,
+                                                     const double *__restrict__ V, int nk, long long ld,
+                                                     const double *__restrict__ c, long long n,
+                                                     double *__restrict__ part, double *__restrict__ out,
+                                                     unsigned *counter) {
+  double ck[KM], acc[1] = {0.0};
+#pragma unroll
+  for (int k = 0; k < KM; ++k) ck[k] = k < nk ? c[k] : 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    JdV<VEC> y = jd_ld<VEC>(q, i);
+    const JdV<VEC> x = jd_ld<VEC>(p, i);
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      if (k < nk) {
+        const JdV<VEC> b = jd_ld<VEC>(V + (long long)k * ld, i);
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) y.v[e] = fma(-ck[k], b.v[e], y.v[e]);
+      }
+    jd_st<VEC>(q, i, y);
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) acc[0] = fma(x.v[e], y.v[e], acc[0]);
+  }
+  jd_reduce(acc, 1, part, out, counter);
+}
+
+template <int VEC, int KM>
+__global__ void __launch_bounds__(JD_T) k_jd_step(double alpha, const double *__restrict__ p, const double *__restrict__ q,
+                                                  double *__restrict__ x, double *__restrict__ r,
+                                                  const double *__restrict__ rinv, double *__restrict__ z,
+                                                  const double *__restrict__ V, int nk, long long ld, long long n,
+                                                  double *__restrict__ part, double *__restrict__ out,
+                                                  unsigned *counter) {
+  double acc[KM + 2];
+#pragma unroll
+  for (int k = 0; k < KM + 2; ++k) acc[k] = 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const JdV<VEC> pv = jd_ld<VEC>(p, i), qv = jd_ld<VEC>(q, i), iv = jd_ld<VEC>(rinv, i);
+    JdV<VEC> xv = jd_ld<VEC>(x, i), rv = jd_ld<VEC>(r, i), zv;
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) {
+      xv.v[e] = fma(alpha, pv.v[e], xv.v[e]);
+      rv.v[e] = fma(-alpha, qv.v[e], rv.v[e]);
+      zv.v[e] = rv.v[e] * iv.v[e];
+      acc[0] = fma(rv.v[e], zv.v[e], acc[0]);
+      acc[1] = fma(rv.v[e], rv.v[e], acc[1]);
+    }
+    jd_st<VEC>(x, i, xv);
+    jd_st<VEC>(r, i, rv);
+    jd_st<VEC>(z, i, zv);
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      if (k < nk) {
+        const JdV<VEC> b = jd_ld<VEC>(V + (long long)k * ld, i);
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) acc[2 + k] = fma(b.v[e], zv.v[e], acc[2 + k]);
+      }
+  }
+  jd_reduce(acc, nk + 2, part, out, counter);
+}
+
+template <int VEC, int KM>
+__global__ void __launch_bounds__(JD_T) k_jd_turn(double *__restrict__ p, const double *__restrict__ z, double beta,
+                                                  const double *__restrict__ V, int nk, long long ld,
+                                                  const double *__restrict__ d, long long n) {
+  double dk[KM];
+#pragma unroll
+  for (int k = 0; k < KM; ++k) dk[k] = k < nk ? d[k] : 0.0;
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    JdV<VEC> y = jd_ld<VEC>(z, i);
+    const JdV<VEC> x = jd_ld<VEC>(p, i);
+#pragma unroll
+    for (int k = 0; k < KM; ++k)
+      if (k < nk) {
+        const JdV<VEC> b = jd_ld<VEC>(V + (long long)k * ld, i);
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) y.v[e] = fma(-dk[k], b.v[e], y.v[e]);
+      }
+#pragma unroll
+    for (int e = 0; e < VEC; ++e) y.v[e] = fma(beta, x.v[e], y.v[e]);
+    jd_st<VEC>(p, i, y);
   }
 }
 
@@ -1373,28 +1464,94 @@ int vk_axpby(forte_ctx *ctx, double a, const double *x, double b, double *y, lon
   return FORTE_OK;
 }
 
+// Launch shape of the correction-solve kernels: packets when the count, the leading
+// dimension and the bases allow 16-byte loads.
+struct JdShape {
+  bool vec;
+  long long n;  // packets or elements
+  unsigned nb, nt;
+};
+static JdShape jd_shape(const forte_ctx *ctx, long long n, long long ld, std::initializer_list<const void *> ptrs) {
+  JdShape s;
+  s.vec = vp_ok<double>(n, ld, ptrs);
+  s.n = s.vec ? n / 2 : n;
+  s.nt = n <= VS_MAX_N ? 64 : JD_T;  // short vectors: more, smaller blocks
+  int nsm = 0;
+  if (cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess || nsm <= 0) {
+    cudaGetLastError();
+    nsm = 152;
+  }
+  s.nb = (unsigned)std::max<long long>(1, std::min<long long>((s.n + s.nt - 1) / s.nt, 4LL * nsm));
+  return s;
+}
+// one launch of kernel<VEC, KM>, KM the smallest of 1, 2, 4, 8, 32 that holds nk
+#define FORTE_JD(kernel, ...)                                                                       \
+  do {                                                                                              \
+    auto go = [&](auto km) {                                                                        \
+      constexpr int KM = decltype(km)::value;                                                       \
+      if (sh.vec)                                                                                   \
+        kernel<2, KM><<<sh.nb, sh.nt, 0, ctx->stream>>>(__VA_ARGS__);                               \
+      else                                                                                          \
+        kernel<1, KM><<<sh.nb, sh.nt, 0, ctx->stream>>>(__VA_ARGS__);                               \
+    };                                                                                              \
+    if (nk <= 1) go(std::integral_constant<int, 1>{});                                              \
+    else if (nk <= 2) go(std::integral_constant<int, 2>{});                                         \
+    else if (nk <= 4) go(std::integral_constant<int, 4>{});                                         \
+    else if (nk <= 8) go(std::integral_constant<int, 8>{});                                         \
+    else go(std::integral_constant<int, 32>{});                                                     \
+  } while (0)
+
+int vk_jd_shift(forte_ctx *ctx, double *q, const double *p, double theta, const double *V, int nk, long long n,
+                double *out) {
+  if (nk < 1 || nk > 32) { set_error("correction solve: %d vectors", nk); return FORTE_ERR_ARG; }
+  const JdShape sh = jd_shape(ctx, n, n, {q, p, V});
+  double *part;
+  unsigned *cnt;
+  int rc = part_buffer(ctx, (size_t)sh.nb * nk, &part, &cnt);
+  if (rc) return rc;
+  FORTE_PROF(ctx, "jd_shift");
+  FORTE_JD(k_jd_shift, q, p, theta, V, nk, n, sh.n, part, out, cnt);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+int vk_jd_project(forte_ctx *ctx, double *q, const double *p, const double *V, int nk, const double *c, long long n,
+                  double *out) {
+  const JdShape sh = jd_shape(ctx, n, n, {q, p, V});
+  double *part;
+  unsigned *cnt;
+  int rc = part_buffer(ctx, (size_t)sh.nb, &part, &cnt);
+  if (rc) return rc;
+  FORTE_PROF(ctx, "jd_project");
+  FORTE_JD(k_jd_project, q, p, V, nk, n, c, sh.n, part, out, cnt);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+int vk_jd_step(forte_ctx *ctx, double alpha, const double *p, const double *q, double *x, double *r, const double *rinv,
+               double *z, const double *V, int nk, long long n, double *out) {
+  const JdShape sh = jd_shape(ctx, n, n, {p, q, x, r, rinv, z, V});
+  double *part;
+  unsigned *cnt;
+  int rc = part_buffer(ctx, (size_t)sh.nb * (nk + 2), &part, &cnt);
+  if (rc) return rc;
+  FORTE_PROF(ctx, "jd_step");
+  FORTE_JD(k_jd_step, alpha, p, q, x, r, rinv, z, V, nk, n, sh.n, part, out, cnt);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+int vk_jd_turn(forte_ctx *ctx, double *p, const double *z, double beta, const double *V, int nk, const double *d,
+               long long n) {
+  const JdShape sh = jd_shape(ctx, n, n, {p, z, V});
+  FORTE_PROF(ctx, "jd_turn");
+  FORTE_JD(k_jd_turn, p, z, beta, V, nk, n, d, sh.n);
+  FORTE_LAUNCH_CHECK();
+  return FORTE_OK;
+}
+#undef FORTE_JD
+
 int vk_precond_inv(forte_ctx *ctx, double theta, double guard, double *rinv, long long n) {
   FORTE_PROF(ctx, "precond_inv");
   k_precond_inv<<<(unsigned)std::min<long long>((n + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
       ctx->d_hdiag, theta, guard, rinv, n);
-  FORTE_LAUNCH_CHECK();
-  return FORTE_OK;
-}
-
-int vk_precond_dot(forte_ctx *ctx, const double *r, const double *rinv, double *z, double *dot_out, long long n) {
-  const bool vs = n <= VS_MAX_N, pk = vp_ok<double>(n, n, {r, z, rinv});
-  const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / 2) : vk_blocks(n);
-  double *part;
-  unsigned *cnt;
-  int rc = part_buffer(ctx, (size_t)2 * nb, &part, &cnt);
-  if (rc) return rc;
-  FORTE_PROF(ctx, "precond_dot");
-  if (vs)
-    k_precond_dot_s<<<nb, VS_T, 0, ctx->stream>>>(r, rinv, z, n, part, dot_out, cnt);
-  else if (pk)
-    k_precond_dot_p<<<nb, VK_THREADS, 0, ctx->stream>>>(r, rinv, z, n / 2, part, dot_out, cnt);
-  else
-    k_precond_dot<<<nb, VK_THREADS, 0, ctx->stream>>>(r, rinv, z, n, part, dot_out, cnt);
   FORTE_LAUNCH_CHECK();
   return FORTE_OK;
 }
