@@ -1005,14 +1005,7 @@ int forte_davidson(forte_ctx *ctx, int nroots, double tol) {
   if (rc) return rc;
   DvResult res;
   ctx->nroots_done = 0;
-  // Tiny spaces: a reduced-precision sigma saves nothing there, and the refinement's many
-  // short passes cost more than the FP64 iterations (one GB300, one root, FP64 against
-  // BF16x2: 7 orbitals with 4 + 3 electrons, 0.3 M products a sigma, 8.8 against
-  // 11.6 ms; 8 with 4 + 4, 1.9 M, 26.9 against 27.9 ms, and twice that for three roots
-  // either way).
-  const bool reduced = ctx->precision == FORTE_TF32 || ctx->precision == FORTE_BF16X2;
-  const int mode = reduced && !ctx->wait_budget && fp64_small(ctx, 1) && fp64_products(ctx) <= 1e6 ? FORTE_FP64
-                                                                                                  : ctx->precision;
+  const int mode = ctx->precision;
   if (mode == FORTE_FP64 || mode == FORTE_DF32 || mode == FORTE_OZ64) {
     rc = davidson_run<double>(ctx, nroots, tol, mode, ctx->d_guess, ctx->nguess, ctx->dv_max_iter,
                               ctx->d_roots, res);

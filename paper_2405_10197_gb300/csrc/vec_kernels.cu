@@ -55,20 +55,36 @@ __device__ __forceinline__ double block_sum_t(T v, double *red) {
 
 // Second pass of a reduction, fused into the kernel that writes the partials: every
 // block publishes its partials part[block][0..m) and counts itself in; the last block
-// to arrive sums part[b][c] over b into out[c] and resets the counter for the next
-// launch on the stream.  A group of `g` lanes (a power of two, m groups if they fit)
-// takes a column: the FP64 pipe issues a warp's addition in 16 clocks, so a block-wide
-// sum per column, most of whose lanes add zeros, took longer than the rest of a short
-// kernel.  No block waits for another.
-__device__ __forceinline__ void last_block_sums(const double *part, int m, double *__restrict__ out,
-                                                unsigned *counter) {
+// to arrive sums part[b][c] over b (strided by thread, then block_sum: the order of
+// a separate 256-thread pass) into out[c] and resets the counter for the next
+// launch on the stream.  No block waits for another.
+__device__ __forceinline__ bool last_block(unsigned *counter) {
   __shared__ bool s_last;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
   __syncthreads();
-  if (!s_last) return;
-  __threadfence();
+  if (s_last) __threadfence();
+  return s_last;
+}
+__device__ __forceinline__ void last_block_sums(const double *part, int m, double *__restrict__ out,
+                                                unsigned *counter, double *red) {
+  if (!last_block(counter)) return;
+  const int nblk = (int)gridDim.x;
+  for (int c = 0; c < m; ++c) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += __ldcg(part + (long long)b * m + c);
+    s = block_sum(s, red);
+    if (threadIdx.x == 0) out[c] = s;
+  }
+  if (threadIdx.x == 0) *counter = 0u;
+}
+// The same with a group of g lanes (a power of two, m groups if they fit) per column: the
+// FP64 pipe issues a warp's addition in 16 clocks, so a block-wide sum per column, most of
+// whose lanes add zeros, takes longer than the rest of a short kernel.
+__device__ __forceinline__ void last_block_lanes(const double *part, int m, double *__restrict__ out,
+                                                 unsigned *counter) {
+  if (!last_block(counter)) return;
   const int nblk = (int)gridDim.x;
   int g = 32;
   while (g > 4 && m * g > (int)blockDim.x) g >>= 1;
@@ -111,7 +127,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_multidot(const T *__restrict__ V
     const double at = block_sum_t<T>(a, red);
     if (threadIdx.x == 0) part[(long long)blockIdx.x * nv + i] = at;
   }
-  last_block_sums(part, nv, out, counter);
+  last_block_sums(part, nv, out, counter, red);
 }
 
 // out_{c0+c} = sum_i coef[i*ncomb + c0 + c] V_i  for c < NC.  NC is a template
@@ -171,7 +187,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_residual_precond(
   }
   const double rt = block_sum_t<T>(rr, red);
   if (threadIdx.x == 0) part[blockIdx.x] = rt;
-  last_block_sums(part, 1, out, counter);
+  last_block_sums(part, 1, out, counter, red);
 }
 
 // t_out = t_in - sum_i c_i B_i ; part[block][i] = B_i . t_out (i < k), part[block][k] = |t_out|^2.
@@ -230,7 +246,7 @@ __global__ void __launch_bounds__(VK_THREADS) k_orth_update(const T *__restrict_
   }
   const double nt = block_sum_t<T>(nn, red);
   if (threadIdx.x == 0) part[(long long)blockIdx.x * (k + 1) + k] = nt;
-  last_block_sums(part, k + 1, out, counter);
+  last_block_sums(part, k + 1, out, counter, red);
 }
 
 // y = a x + b y
@@ -312,7 +328,8 @@ __global__ void k_nonfinite(const double *__restrict__ x, long long n, int *flag
 // one chunk, so that the vectors spread over the SMs; the per-thread sums of a column
 // meet in shared memory, where 4 threads add one column (64 values), instead of a
 // five-step warp reduction per column.  Elements are loaded singly, so any count and
-// alignment will do.  One GB300, CAS(8,8) FP64 solve (133 iterations): residual pass 31 ->
+// alignment will do.  FP64 vectors only: the FP32 ones of the reduced-precision phase keep
+// the kernels above and below, whose order of sums its rounding follows.  One GB300, CAS(8,8) FP64 solve (133 iterations): residual pass 31 ->
 // 14 us, 11-vector dots 22 -> 9 us, whole solve 18.9 -> 14.0 ms.
 constexpr int VS_T = 64;
 constexpr int VS_E = 2;
@@ -371,7 +388,7 @@ __global__ void __launch_bounds__(VS_T) k_multidot_s(const T *__restrict__ V, in
 #pragma unroll
   for (int e = 0; e < VS_E; ++e) xr[e] = j0 + e * VS_T < n ? x[j0 + e * VS_T] : T(0);
   vs_dots(r, V, nv, ld, xr, j0, n, 0, nv, part);
-  last_block_sums(part, nv, out, counter);
+  last_block_lanes(part, nv, out, counter);
 }
 
 // As k_orth_update_p: t_out = scale (t_in - B c), out = [B^T t_out (zeros unless DOTS), |t_out|^2].
@@ -408,7 +425,7 @@ __global__ void __launch_bounds__(VS_T) k_orth_update_s(const T *__restrict__ B,
   } else {
     for (int i = threadIdx.x; i < k; i += VS_T) part[(long long)blockIdx.x * (k + 1) + i] = 0.0;
   }
-  last_block_sums(part, k + 1, out, counter);
+  last_block_lanes(part, k + 1, out, counter);
 }
 
 // As k_residual_precond_p: t = r / (theta - H_II), out = [|r|^2 (, B^T t, |t|^2)].
@@ -453,7 +470,7 @@ __global__ void __launch_bounds__(VS_T) k_residual_precond_s(const T *__restrict
     vs_columns(r, k + 1, 1, m, part);
     vs_dots(r, B, k, ld, hx, j0, n, 1, m, part);
   }
-  last_block_sums(part, m, out, counter);
+  last_block_lanes(part, m, out, counter);
 }
 
 // ------------------------------------------------------------------ packet kernels
@@ -542,6 +559,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_p(const T *__re
                                                            double *__restrict__ part, double *__restrict__ out,
                                                            unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[VK_MAXV * VP_WARPS];
   for (int i = threadIdx.x; i < nv * VP_WARPS; i += blockDim.x) sw[i] = 0.0;
   __syncthreads();
@@ -576,7 +594,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_p(const T *__re
     }
   }
   block_partials(sw, nv, part);
-  last_block_sums(part, nv, out, counter);
+  last_block_sums(part, nv, out, counter, red);
 }
 
 // The same for nv <= KMAX: loop over the vectors unrolled, partial sums of the
@@ -587,6 +605,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_u(const T *__re
                                                                    double *__restrict__ part,
                                                                    double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[KMAX * VP_WARPS];
   for (int i = threadIdx.x; i < nv * VP_WARPS; i += blockDim.x) sw[i] = 0.0;
   __syncthreads();
@@ -628,7 +647,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_multidot_u(const T *__re
   for (int i = 0; i < KMAX; ++i)
     if (i < nv) warp_add(acc[i], sw + i * VP_WARPS);
   block_partials(sw, nv, part);
-  last_block_sums(part, nv, out, counter);
+  last_block_sums(part, nv, out, counter, red);
 }
 
 // t_out = scale (t_in - sum_i c_i B_i); out = [B_i . t_out (i < k, zeros unless DOTS),
@@ -640,6 +659,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_p(const T *_
                                                               double *__restrict__ part, double *__restrict__ out,
                                                               unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[(VK_MAXV + 1) * VP_WARPS];
   __shared__ T sc[VK_MAXV];
   const int ku = c ? k : 0;
@@ -709,7 +729,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_p(const T *_
     }
   }
   block_partials(sw, k + 1, part);
-  last_block_sums(part, k + 1, out, counter);
+  last_block_sums(part, k + 1, out, counter, red);
 }
 
 // The same for k <= KMAX: loops over the basis unrolled, partial sums in registers.
@@ -720,6 +740,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_u(const T *_
                                                                       double *__restrict__ part,
                                                                       double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[(KMAX + 1) * VP_WARPS];
   __shared__ T sc[KMAX];
   const int ku = c ? k : 0;
@@ -800,7 +821,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_orth_update_u(const T *_
       if (i < k) warp_add(acc[i], sw + i * VP_WARPS);
   }
   block_partials(sw, k + 1, part);
-  last_block_sums(part, k + 1, out, counter);
+  last_block_sums(part, k + 1, out, counter, red);
 }
 
 // r = sum_i u_i S_i - theta sum_i u_i B_i ;  t = r / (theta - hdiag) (guarded).
@@ -815,6 +836,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_p(
     double theta, const double *__restrict__ hd, double guard, T *__restrict__ t, long long np,
     double *__restrict__ part, double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[(VK_MAXV + 2) * VP_WARPS];
   __shared__ T su[VK_MAXV];
   const int m = DOTS ? k + 2 : 1;
@@ -888,7 +910,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_p(
     }
   }
   block_partials(sw, m, part);
-  last_block_sums(part, m, out, counter);
+  last_block_sums(part, m, out, counter, red);
 }
 
 // The same for k <= KMAX with the loops over the basis unrolled (the loads of all k
@@ -900,6 +922,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_u(
     double theta, const double *__restrict__ hd, double guard, T *__restrict__ t, long long np,
     double *__restrict__ part, double *__restrict__ out, unsigned *counter) {
   constexpr int P = Pk<T>::P;
+  __shared__ double red[32];
   __shared__ double sw[(KMAX + 2) * VP_WARPS];
   __shared__ T su[KMAX];
   const int m = DOTS ? k + 2 : 1;
@@ -987,7 +1010,7 @@ __global__ void __launch_bounds__(VK_THREADS, VP_BPS) k_residual_precond_u(
       if (i < k) warp_add(acc[i], sw + (1 + i) * VP_WARPS);
   }
   block_partials(sw, m, part);
-  last_block_sums(part, m, out, counter);
+  last_block_sums(part, m, out, counter, red);
 }
 
 // y = a x + b y and x = alpha src over packets (grid-stride).  With a or b equal to 1
@@ -1030,7 +1053,7 @@ __global__ void k_scale_p(T *x, const T *src, double alpha, long long np) {
 // here: it leaves 2^-53 of the vector, and the solve is stopped at a 50th of its start.
 // VEC: elements a thread takes at a time (2: 16-byte loads, for even counts).  Sums: per
 // thread, then a warp adds a column of the block's threads from shared memory, then
-// last_block_sums.  One GB300, CAS(14,14), one root: 0.70 -> 0.36 ms an inner iteration.
+// last_block_lanes.  One GB300, CAS(14,14), one root: 0.70 -> 0.36 ms an inner iteration.
 constexpr int JD_T = 256;
 constexpr int JD_COLS = 8;  // columns reduced at a time
 
@@ -1079,7 +1102,7 @@ __device__ __forceinline__ void jd_reduce(const double (&acc)[M], int m, double 
       }
     }
   }
-  last_block_sums(part, m, out, counter);
+  last_block_lanes(part, m, out, counter);
 }
 
 template <int VEC, int KM>
@@ -1233,7 +1256,7 @@ template <typename T>
 static int vk_multidot_t(forte_ctx *ctx, const T *V, int nv, long long ld, const T *x, long long n, double *out) {
   if (nv <= 0) return FORTE_OK;
   if (nv > VK_MAXV) { set_error("multidot: too many vectors (%d)", nv); return FORTE_ERR_ARG; }
-  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {V, x});
+  const bool vs = sizeof(T) == 8 && n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {V, x});
   const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
   double *part;
   unsigned *cnt;
@@ -1283,7 +1306,7 @@ template <typename T>
 static int vk_residual_precond_t(forte_ctx *ctx, const T *B, const T *S, int k, long long ld, const double *u,
                                  double theta, double guard, T *t, double *rnorm2, long long n, double *dots) {
   if (k > VK_MAXV) { set_error("residual: subspace too large (%d)", k); return FORTE_ERR_ARG; }
-  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, S, t, ctx->d_hdiag});
+  const bool vs = sizeof(T) == 8 && n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, S, t, ctx->d_hdiag});
   if (dots && !pk && !vs) return -1;  // no fused dots: the caller forms them with vk_orth_update
   const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, 2 * (n / Pk<T>::P)) : vk_blocks(n);  // chunks of half the packets
   const int m = dots ? k + 2 : 1;
@@ -1343,7 +1366,7 @@ template <typename T>
 static int vk_orth_update_t(forte_ctx *ctx, const T *B, int k, long long ld, const double *c, const T *t_in,
                             T *t_out, double *dots_out, long long n, bool dots, double scale) {
   if (k + 1 > VK_MAXV) { set_error("orth: subspace too large (%d)", k); return FORTE_ERR_ARG; }
-  const bool vs = n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, t_in, t_out});
+  const bool vs = sizeof(T) == 8 && n <= VS_MAX_N, pk = vp_ok<T>(n, ld, {B, t_in, t_out});
   const unsigned nb = vs ? vs_blocks(n) : pk ? vp_grid(ctx, n / Pk<T>::P) : vk_blocks(n);
   double *part;
   unsigned *cnt;
