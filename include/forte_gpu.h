@@ -341,8 +341,10 @@ int forte_rdm3(forte_ctx *ctx, const double *C, double *g3);
  * threads with their own streams, concurrently with the class launches.  Before
  * the solve an autotuner times, for every class, the per-CTA sigma for each
  * (threads per CTA, beta tile width) candidate and keeps the fastest; it then
- * times one Davidson iteration of the class's first problem on the
- * single-problem path and sends the class there when
+ * times Davidson iterations of the class's first problem on the single-problem path
+ * (FP64 ones in the mixed modes) and, with t_single_iteration the time per problem and
+ * root (four fifths of the one measured alone: the workers overlap) and t_CTA_sigma the
+ * time of one sigma build (double-FP32 in the mixed modes), sends the class there when
  *   P x t_single_iteration < t_CTA_sigma x ceil(P / (resident CTAs per SM x SMs)).
  * Problems with more than 100,000 determinants or more than 3 roots always take
  * the single-problem path.  forte_batch_tuning reports the choices.
@@ -370,7 +372,7 @@ int forte_batch_solve(int nprob, const int *norb, const int *nalpha, const int *
  * beta tile width of the alpha-beta term, the measured time (ms) of one sigma
  * build of the class's first problems (one CTA each) with the chosen candidate,
  * the chosen path (0: class launch, 1: single-problem path), the measured time
- * (ms) of one single-problem-path Davidson iteration, the class's problem count
+ * (ms) of one single-problem-path Davidson iteration per root, the class's problem count
  * and the resident CTAs per SM of its launch.
  * Control entry point: the paper has no counterpart.
  */

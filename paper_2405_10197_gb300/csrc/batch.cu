@@ -1114,26 +1114,35 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
       cudaStreamDestroy(sx);
     }
   };
-  // Host wall time (ms) of one Davidson iteration of problem i on the single-problem
-  // path: forte_davidson capped at 2 and at 6 iterations after a 1-iteration run
-  // that builds the lazy tables; (t6 - t2) / 4 leaves out the set-up and the first
-  // sigma builds and keeps the per-iteration launch and host costs.
+  // Host wall time (ms) per problem and root (sigma build) of one Davidson iteration on the
+  // single-problem path:
+  // problem i capped at 2 and at 6 iterations (the faster of two runs each) after a
+  // 1-iteration run that builds the lazy tables; (t6 - t2) / 4 leaves out the set-up
+  // and the first sigma builds and keeps the launch and host costs of an iteration.  The
+  // workers' overlap brings the time per problem down by a fifth (8 problems of 6 to 8
+  // orbitals at once on one GB300: 0.053 - 0.069 ms, alone 0.064 - 0.085 ms).  FP64
+  // iterations stand for those of a mixed mode, whose solves are of two kinds of
+  // iteration and take about as long (8 orbitals, one root: 26.9 ms FP64, 27.9 ms
+  // BF16x2; 10 orbitals: 43 against 30 ms).
   auto single_iter_ms = [&](int i) -> double {
+    const int prec = precision == FORTE_TF32 || precision == FORTE_BF16X2 ? FORTE_FP64 : precision;
     forte_ctx *ctx = forte_cas_create(norb[i], nalpha[i], nbeta[i], h[i], eri[i]);
     if (!ctx) return INFINITY;
-    const int cap[3] = {1, 2, 6};
-    double t[3] = {0.0, 0.0, 0.0};
-    bool ok = forte_set_precision(ctx, precision) == FORTE_OK;
-    for (int r = 0; r < 3 && ok; ++r) {
-      ok = forte_set_davidson_params(ctx, 12, 2, cap[r], 1e-8) == FORTE_OK;
+    bool ok = forte_set_precision(ctx, prec) == FORTE_OK;
+    double t2 = INFINITY, t6 = INFINITY;
+    for (int cap : {1, 2, 6, 2, 6}) {
+      if (!ok) break;
+      ok = forte_set_davidson_params(ctx, 12, 2, cap, 1e-8) == FORTE_OK;
       const auto t0 = std::chrono::steady_clock::now();
       const int rc = ok ? forte_davidson(ctx, nroots[i], 1e-14) : FORTE_ERR_ARG;
-      t[r] = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+      const double t = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
+      if (cap == 2) t2 = std::min(t2, t);
+      if (cap == 6) t6 = std::min(t6, t);
       ok = (rc == FORTE_OK || rc == FORTE_ERR_NOT_CONVERGED);
     }
     forte_destroy(ctx);
     clear_error();
-    return ok ? std::max(1e-3, (t[2] - t[1]) / 4.0) : INFINITY;
+    return ok ? std::max(1e-3, 0.8 * (t6 - t2) / (4.0 * nroots[i])) : INFINITY;
   };
 
   // ---- one pooled device allocation for the batch
@@ -1240,18 +1249,30 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
           ch.TJ = tj;
         }
       }
-    cudaEventDestroy(a);
-    cudaEventDestroy(b);
     if (!any) {
+      cudaEventDestroy(a);
+      cudaEventDestroy(b);
       set_error("forte_batch_solve: no kernel configuration fits class (%d, %d, %d)", ch.n, ch.na, ch.nb);
       return FORTE_ERR_ARG;
     }
+    if (mode == 1) {  // the double-FP32 builds of the second phase take most of a mixed solve
+      probe.mode = 2;
+      probe.TJ = ch.TJ;
+      FORTE_CUDA_TRY(cudaEventRecord(a, guard.s[ci]));
+      FORTE_CUDA_TRY(launch_any(ch.NT, probe, class_smem(ch.dev, ar, ch.TJ), guard.s[ci]));
+      FORTE_CUDA_TRY(cudaEventRecord(b, guard.s[ci]));
+      FORTE_CUDA_TRY(cudaEventSynchronize(b));
+      float ms = 0.f;
+      FORTE_CUDA_TRY(cudaEventElapsedTime(&ms, a, b));
+      best = ms;
+    }
+    cudaEventDestroy(a);
+    cudaEventDestroy(b);
     ch.probe_ms = best;
     ch.dev.TJ = ch.TJ;
     ch.dev.probe = 0;
     // path: one class launch costs about probe_ms per sigma round for every wave of
-    // resident CTAs; the single-problem path costs single_iter_ms per problem and
-    // iteration (no credit for overlap between workers)
+    // resident CTAs; the single-problem path costs single_iter_ms per problem
     int per_sm = 0;
     cudaError_t oe = cudaSuccess;
     const size_t smem = class_smem(ch.dev, ar, ch.TJ);
