@@ -140,7 +140,10 @@ __device__ __forceinline__ float tf32_rne(double x) { return (float)rne_drop(x, 
 
 // Besides the row-padded copy it writes the copy in beta positions (row length
 // NBpos, strOf[b] = string at position b, -1 for padding) that the alpha-beta
-// kernel gathers; its rounding is the same.
+// kernel gathers.  A block takes a row at a time: an element is split once, kept in
+// shared memory as one word, and both copies are written from there in 32-bit (TF32:
+// 64-bit) stores.  HBM bounds it.  One GB300, CAS(14,14), FP32 vector: 105 -> 55 us (a
+// thread per element and copy, a 64-bit division and 16-bit stores each, before).
 template <int MODE, typename TI>
 __global__ void __launch_bounds__(256) k_split_rows(const TI *__restrict__ C, uint16_t *__restrict__ hi,
                                                     uint16_t *__restrict__ lo, float *__restrict__ t32, long long NA,
@@ -148,31 +151,50 @@ __global__ void __launch_bounds__(256) k_split_rows(const TI *__restrict__ C, ui
                                                     const int *__restrict__ strOf, long long NBpos,
                                                     uint16_t *__restrict__ phi, uint16_t *__restrict__ plo,
                                                     float *__restrict__ pt32) {
+  extern __shared__ uint32_t srow[];  // [NBp]: hi | lo << 16, or the TF32 value
   __shared__ unsigned red[8];
-  // grid-stride over (row, 256-column block) pairs; one atomic per block at the end
   const long long v = blockIdx.z;
-  const long long nbx = (std::max(NBp, strOf ? NBpos : 0LL) + 255) / 256;
+  const int nb = (int)NB, nbp = (int)NBp, npos = strOf ? (int)NBpos : 0;  // nbp and npos are even
   unsigned mx = 0u;
-  for (long long w = blockIdx.x; w < NA * nbx; w += gridDim.x) {
-    const long long row = w / nbx, b = (w % nbx) * 256 + threadIdx.x;
-    if (b < NBp && (hi || t32)) {
-      const TI x = b < NB ? C[(v * NA + row) * NB + b] : TI(0);
-      mx = max(mx, abs_bits(x));
-      const long long o = (v * NA + row) * NBp + b;
-      if (MODE == FORTE_BF16X2)
-        split_bf16(x, hi[o], lo[o]);
-      else
-        t32[o] = tf32_rne(x);
+  for (long long row = blockIdx.x; row < NA; row += gridDim.x) {
+    const TI *Cr = C + (v * NA + row) * NB;
+    const long long o = (v * NA + row) * NBp, op = (v * NA + row) * NBpos;
+    for (int b = 2 * threadIdx.x; b < nbp; b += 512) {
+      uint32_t w[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const TI x = b + k < nb ? Cr[b + k] : TI(0);
+        mx = max(mx, abs_bits(x));
+        if (MODE == FORTE_BF16X2) {
+          uint16_t h, l;
+          split_bf16(x, h, l);
+          w[k] = h | ((uint32_t)l << 16);
+        } else {
+          w[k] = __float_as_uint(tf32_rne(x));
+        }
+        srow[b + k] = w[k];
+      }
+      if (MODE == FORTE_BF16X2) {
+        if (hi) {
+          *reinterpret_cast<uint32_t *>(hi + o + b) = __byte_perm(w[0], w[1], 0x5410);
+          *reinterpret_cast<uint32_t *>(lo + o + b) = __byte_perm(w[0], w[1], 0x7632);
+        }
+      } else if (t32) {
+        *reinterpret_cast<uint2 *>(t32 + o + b) = make_uint2(w[0], w[1]);
+      }
     }
-    if (strOf && b < NBpos) {
-      const int J = strOf[b];
-      const TI x = J >= 0 ? C[(v * NA + row) * NB + J] : TI(0);
-      const long long o = (v * NA + row) * NBpos + b;
-      if (MODE == FORTE_BF16X2)
-        split_bf16(x, phi[o], plo[o]);
-      else
-        pt32[o] = tf32_rne(x);
+    __syncthreads();
+    for (int b = 2 * threadIdx.x; b < npos; b += 512) {
+      const int2 J = *reinterpret_cast<const int2 *>(strOf + b);
+      const uint32_t w0 = J.x >= 0 ? srow[J.x] : 0u, w1 = J.y >= 0 ? srow[J.y] : 0u;
+      if (MODE == FORTE_BF16X2) {
+        *reinterpret_cast<uint32_t *>(phi + op + b) = __byte_perm(w0, w1, 0x5410);
+        *reinterpret_cast<uint32_t *>(plo + op + b) = __byte_perm(w0, w1, 0x7632);
+      } else {
+        *reinterpret_cast<uint2 *>(pt32 + op + b) = make_uint2(w0, w1);
+      }
     }
+    __syncthreads();
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -916,14 +938,14 @@ static int sigma_mixed_t(forte_ctx *ctx, const T *C, T *S, int nvec, int mode) {
     const long long per = NA * NBp;
     dim3 grid((unsigned)std::min<long long>((per + 255) / 256, 152LL * 16), (unsigned)nvec);
     FORTE_PROF(ctx, "split");
-    const long long wcols = std::max(NBp, ab ? NBpos : 0LL);
-    dim3 g2((unsigned)std::min<long long>(NA * ((wcols + 255) / 256), 152LL * 8), 1u, (unsigned)nvec);
+    const dim3 g2((unsigned)std::min<long long>(NA, 152LL * 8), 1u, (unsigned)nvec);
+    const size_t srow = sizeof(uint32_t) * (size_t)NBp;  // at most 26 KB (6435 strings)
     if (!C32w) {  // no FP32 copy wanted: the row kernel writes both copies
       if (mode == FORTE_BF16X2)
-        k_split_rows<FORTE_BF16X2, T><<<g2, 256, 0, st>>>(C, Chi, Clo, nullptr, NA, NB, NBp, cmax, strOf, NBpos, Phi,
+        k_split_rows<FORTE_BF16X2, T><<<g2, 256, srow, st>>>(C, Chi, Clo, nullptr, NA, NB, NBp, cmax, strOf, NBpos, Phi,
                                                           Plo, nullptr);
       else
-        k_split_rows<FORTE_TF32, T><<<g2, 256, 0, st>>>(C, nullptr, nullptr, Ct32, NA, NB, NBp, cmax, strOf, NBpos,
+        k_split_rows<FORTE_TF32, T><<<g2, 256, srow, st>>>(C, nullptr, nullptr, Ct32, NA, NB, NBp, cmax, strOf, NBpos,
                                                         nullptr, nullptr, Pt32);
     } else {
       if (mode == FORTE_BF16X2)
@@ -933,10 +955,10 @@ static int sigma_mixed_t(forte_ctx *ctx, const T *C, T *S, int nvec, int mode) {
       FORTE_LAUNCH_CHECK();
       if (ab) {  // positional copy only (the row copy is written above)
         if (mode == FORTE_BF16X2)
-          k_split_rows<FORTE_BF16X2, T><<<g2, 256, 0, st>>>(C, nullptr, nullptr, nullptr, NA, NB, NBp, cmax, strOf,
+          k_split_rows<FORTE_BF16X2, T><<<g2, 256, srow, st>>>(C, nullptr, nullptr, nullptr, NA, NB, NBp, cmax, strOf,
                                                             NBpos, Phi, Plo, nullptr);
         else
-          k_split_rows<FORTE_TF32, T><<<g2, 256, 0, st>>>(C, nullptr, nullptr, nullptr, NA, NB, NBp, cmax, strOf,
+          k_split_rows<FORTE_TF32, T><<<g2, 256, srow, st>>>(C, nullptr, nullptr, nullptr, NA, NB, NBp, cmax, strOf,
                                                           NBpos, nullptr, nullptr, Pt32);
       }
     }
