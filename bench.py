@@ -182,8 +182,10 @@ def kernel_work(name, prob, n_sig64, n_sigm, n_rdm, tables):
     nka, nkb = nk(prob.nalpha), nk(prob.nbeta)
     npair = n * (n + 1) // 2
     nnz_a, nnz_b = tables
+    # moving replacements, and one entry for all that move no electron
+    mka, mkb = nka - prob.nalpha + 1, nkb - prob.nbeta + 1
     if name == "ab_fp64":
-        return 2.0 * nd * nka * nkb * n_sig64, "TFLOP/s", "alu", FP64_PEAK_TFLOPS, "FP64 pipe, nominal"
+        return 2.0 * nd * mka * mkb * n_sig64, "TFLOP/s", "alu", FP64_PEAK_TFLOPS, "FP64 pipe, nominal"
     if name == "ss_spmm":
         return (2.0 * (nnz_a * prob.nb + nnz_b * prob.na) * n_sig64, "TFLOP/s", "alu", FP64_PEAK_TFLOPS,
                 "FP64 pipe, nominal")
@@ -197,8 +199,8 @@ def kernel_work(name, prob, n_sig64, n_sigm, n_rdm, tables):
         return (2.0 * nd * npair * nka * n_sigm, "TFLOP/s", "tensor", bf16s * TF32_OVER_BF16,
                 f"bf16 dense sustained ({src}) x nominal tf32/bf16 ratio")
     if name == "gram":
-        nt = (n * n + 63) // 64  # symmetric Gram: tiles ta <= tb of 64 x 64
-        return (2.0 * 64 * 64 * nt * (nt + 1) // 2 * nd * n_rdm, "TFLOP/s", "alu", FP64_PEAK_TFLOPS,
+        nu, nv = npair, npair - n  # Grams of the symmetric and antisymmetric images
+        return (1.0 * (nu * (nu + 1) + nv * (nv + 1)) * nd * n_rdm, "TFLOP/s", "alu", FP64_PEAK_TFLOPS,
                 "FP64 pipe, nominal")
     if name == "ss_mma_bf16x2":
         # one GEMM [H_a | C] [C^T | H_b]^T per vector, 3 BF16 products
@@ -208,7 +210,7 @@ def kernel_work(name, prob, n_sig64, n_sigm, n_rdm, tables):
         return (2.0 * prob.na * prob.nb * (prob.na + prob.nb) * n_sigm, "TFLOP/s", "tensor",
                 bf16s * TF32_OVER_BF16, f"bf16 dense sustained ({src}) x nominal tf32/bf16 ratio")
     if name == "ab_df":
-        return (2.0 * nd * nka * nkb * n_sig64, "TFLOP/s", "alu", DF32_PEAK_TFLOPS,
+        return (2.0 * nd * mka * mkb * n_sig64, "TFLOP/s", "alu", DF32_PEAK_TFLOPS,
                 "FP32 pipe / 6 (12 FP32 operations per double-FP32 multiply-add)")
     if name == "ss_spmm_df":
         return (2.0 * (nnz_a * prob.nb + nnz_b * prob.na) * n_sig64, "TFLOP/s", "alu", DF32_PEAK_TFLOPS,
@@ -835,7 +837,8 @@ def run_extensions(args):
         E, C, rn, it = prob.davidson(nroots=1, tol=1e-8)
         g3 = torch.empty((n,) * 6, dtype=torch.float64, device="cuda")
         ms = ev_ms(lambda: fg.forte_rdm3(prob.ctx, C[0], g3, n), 3)
-        flop = 2.0 * n ** 6 * prob.ndet
+        nu, nv = n * (n + 1) // 2, n * (n - 1) // 2  # components (S,S,S) and (A,A,S)
+        flop = 2.0 * (nu * (nu + 1) * (nu + 2) // 6 + nu * nv * (nv + 1) // 2) * prob.ndet
         x1["cases"].append({"workload": f"CAS({n},{n})", "n_det": prob.ndet, "ms": ms,
                             "gram_fp64_tflops": flop / (ms * 1e-3) / 1e12,
                             "frac_of_nominal_fp64_1.25": flop / (ms * 1e-3) / 1.25e12})

@@ -65,7 +65,10 @@ enum {
                        FP32 products via FMA, compensated sums; relative error
                        ~2^-46 per term.  Davidson as for FORTE_FP64 (FP64 vectors).
                        Not part of the paper's schemes: an FP64 substitute for
-                       GPUs whose FP64 pipe is narrow. */
+                       GPUs whose FP64 pipe is narrow.  Spaces of up to 40 M
+                       products a call take the FP64 kernels here and in
+                       FORTE_OZ64 (faster there), FORTE_OZ64 only without a wait
+                       budget of the caller's. */
   FORTE_OZ64 = 4    /* FP64-class sigma whose alpha-beta term is formed on the BF16
                        tensor cores from exact products of 8-bit digit slices
                        (integrals and C in 45-bit fixed point per row / 64-string tile,
@@ -112,7 +115,7 @@ int forte_set_stream(forte_ctx *ctx, void *cuda_stream);
 
 /* Select FORTE_FP64, FORTE_TF32, FORTE_BF16X2, FORTE_DF32 or FORTE_OZ64 for forte_sigma,
  * forte_davidson and forte_rdms (every mode but FORTE_FP64 forms the 2-RDM with
- * the tensor-core Gram).  Default FORTE_FP64.  FORTE_ERR_ARG for other values.
+ * the tensor-core Gram, unless the FP64 one has at most 80 M products).  Default FORTE_FP64.  FORTE_ERR_ARG for other values.
  * The paper computes in FP64 (FORTE_FP64); the other modes extend it and have no
  * counterpart there.
  */
@@ -321,9 +324,10 @@ int forte_tdm1(forte_ctx *ctx, const double *bra, const double *ket, double *t1)
  *      = <E_pq E_rs E_tu> - d_qt Gamma_purs - d_st Gamma_pqru
  *        - d_qr (Gamma_pstu + d_st gamma_pu)
  * (chemist order: each pair (p,q), (r,s), (t,u) shares one spin sum).
- * FP64 in every precision mode.  Workspace 2 n^2 N_det doubles plus 64 n^4;
- * work n^2 Gram products of n^2 x n^2 over N_det, so it is meant for the
- * active spaces where the 3-RDM is used (n up to ~10).  Asynchronous on the
+ * FP64 in every precision mode.  Workspace n(n+1)/2 N_det doubles plus
+ * the partial Grams; one launch over all third pair indices, about n^6 / 6 flops per
+ * determinant, so it is meant for the active spaces where the 3-RDM is used (n up to
+ * ~10).  Asynchronous on the
  * context stream; FORTE_ERR_ALLOC when the workspace cannot be allocated. */
 int forte_rdm3(forte_ctx *ctx, const double *C, double *g3);
 
