@@ -122,12 +122,16 @@ __device__ __forceinline__ void gas_compact(int w, int cnt, F ok, uint16_t *list
   if ((int)(threadIdx.x >> 5) != w) return;
   const int lane = threadIdx.x & 31;
   int m = 0;
-  for (int p0 = 0; p0 < cnt; p0 += 32) {
-    const int p = p0 + lane;
-    const bool k = p < cnt && ok(p);
-    const unsigned bal = __ballot_sync(0xffffffffu, k);
-    if (k) list[m + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)p;
-    m += __popc(bal);
+  for (int p0 = 0; p0 < cnt; p0 += 128) {  // four tests at a time: their loads overlap
+    bool k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) k[u] = p0 + 32 * u + lane < cnt && ok(p0 + 32 * u + lane);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned bal = __ballot_sync(0xffffffffu, k[u]);
+      if (k[u]) list[m + __popc(bal & ((1u << lane) - 1u))] = (uint16_t)(p0 + 32 * u + lane);
+      m += __popc(bal);
+    }
   }
   if (lane == 0) *n = m;
 }
@@ -144,8 +148,11 @@ __device__ __forceinline__ void gas_compact(int w, int cnt, F ok, uint16_t *list
 //  (2) per kept output: the accumulator plus the same-spin terms
 //      sum_Ja H_aa[Ia][Ja] C[Ja][Ib] + sum_Jb H_bb[Ib][Jb] C[Ia][Jb] over allowed sources.
 // The FP64 pipe bounds it.  One GB300, CAS(14,14) with at most 2 holes in orbitals 0-3
-// and 2 particles in 10-13 (369,712 of 11.8 M determinants): 4.73 -> 2.80 ms (before, a lane
+// and 2 particles in 10-13 (369,712 of 11.8 M determinants): 4.73 -> 2.75 ms (before, a lane
 // whose replacement was not allowed idled, and the same-spin sums ran over all entries).
+// Small spaces wait on memory latency, many classes holding a few strings each; there the
+// lanes of a warp share an output: 5 + 6 electrons in 12 orbitals, 1 hole in 0-3, 2 particles
+// in 9-11: 167 us before the class lists, 285 us with a thread per output, 137 us so.
 // T: FP64, or FP32 for the FP32 vectors of the reduced-precision phase.
 template <typename T>
 __global__ void __launch_bounds__(GAS_THREADS) k_gas_sigma(
@@ -231,19 +238,21 @@ __global__ void __launch_bounds__(GAS_THREADS) k_gas_sigma(
         atomicAdd(&srow[f & 0xFFFFu], (f >> 31) ? -acc : acc);
       }
       if (self) {
-        // the unmoved replacements of Jb, the rows split over the threads
-        const int parts = GAS_THREADS / TJ, part = threadIdx.x / TJ, j = threadIdx.x - part * TJ;
-        if (part < parts && j < tj) {
+        // the unmoved replacements of Jb: npp integral sums with row Ia itself (k = 0) and one
+        // with each other row, split over up to 16 threads a string
+        const int parts = min(16, GAS_THREADS / tj), part = threadIdx.x / tj, j = threadIdx.x - part * tj;
+        const int z = klist[0] == 0 ? npp : 0, lead = z ? 1 : 0;
+        if (part < parts) {
           T acc = T(0);
-          for (int kk = part; kk < kc; kk += parts) {
-            const int e = klist[kk];
-            const T d = D[kk * TJ + j];
-            if (e == 0) {
-              for (int m = 0; m < npp; ++m) acc += (T)W[(size_t)s_pp[m] * NB + sj[j]] * d;
+#pragma unroll 2
+          for (int u = part; u < z + kc - lead; u += parts) {
+            if (u < z) {
+              acc += (T)W[(size_t)s_pp[u] * NB + sj[j]] * D[j];
             } else {
-              const uint32_t w = la[e - 1];
+              const int kk = u - z + lead;
+              const uint32_t w = la[klist[kk] - 1];
               const T x = (T)W[(size_t)((w >> 16) & 0xFFu) * NB + sj[j]];
-              acc += ((w >> 31) ? -x : x) * d;
+              acc += ((w >> 31) ? -x : x) * D[kk * TJ + j];
             }
           }
           atomicAdd(&srow[sj[j]], acc);
@@ -259,19 +268,27 @@ __global__ void __launch_bounds__(GAS_THREADS) k_gas_sigma(
     gas_compact(1, nnzB, [&](int p) { return (okA >> ccls[b * nnzB + p]) & 1ull; }, flist, &s_n[1]);
     __syncthreads();
     const int ne = s_n[0], nf = s_n[1];
-    for (int i = threadIdx.x; i < nb; i += GAS_THREADS) {
-      const int Ib = cstr[i0 + i];
-      T acc = srow[Ib], acc2 = T(0);
+    // small classes: up to 32 neighbouring lanes share an output's terms
+    int parts = 1;
+    while (parts < 32 && 2 * parts * nb <= GAS_THREADS) parts *= 2;
+    const int q = threadIdx.x % parts;
+    for (int i1 = 0; i1 < nb; i1 += GAS_THREADS / parts) {
+      const int i = i1 + threadIdx.x / parts, Ib = i < nb ? cstr[i0 + i] : 0;
+      T acc = T(0), acc2 = T(0);
+      if (i < nb) {
 #pragma unroll 4
-      for (int e = 0; e < ne; ++e) acc += sval[elist[e]] * Cv[(long long)scol[elist[e]] * NB + Ib];
-      const int *ec = ellc + (long long)nnzB * i0 + i;
-      const T *ev = ellv + (long long)nnzB * i0 + i;
+        for (int e = q; e < ne; e += parts) acc += sval[elist[e]] * Cv[(long long)scol[elist[e]] * NB + Ib];
+        const int *ec = ellc + (long long)nnzB * i0 + i;
+        const T *ev = ellv + (long long)nnzB * i0 + i;
 #pragma unroll 4
-      for (int f = 0; f < nf; ++f) {
-        const long long p = (long long)flist[f] * nb;
-        acc2 += ev[p] * Cv[(long long)Ia * NB + ec[p]];
+        for (int f = q; f < nf; f += parts) {
+          const long long p = (long long)flist[f] * nb;
+          acc2 += ev[p] * Cv[(long long)Ia * NB + ec[p]];
+        }
       }
-      Sv[Ib] = acc + acc2;
+      acc += acc2;
+      for (int o = parts >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (i < nb && q == 0) Sv[Ib] = srow[Ib] + acc;
     }
   }
 }
