@@ -65,10 +65,9 @@ enum {
                        FP32 products via FMA, compensated sums; relative error
                        ~2^-46 per term.  Davidson as for FORTE_FP64 (FP64 vectors).
                        Not part of the paper's schemes: an FP64 substitute for
-                       GPUs whose FP64 pipe is narrow.  Spaces of up to 40 M
-                       products a call take the FP64 kernels here and in
-                       FORTE_OZ64 (faster there), FORTE_OZ64 only without a wait
-                       budget of the caller's. */
+                       GPUs whose FP64 pipe is narrow.  Calls of up to 40 M
+                       products take the FP64 kernels here and in FORTE_OZ64
+                       (faster there; forte_set_small_route). */
   FORTE_OZ64 = 4    /* FP64-class sigma whose alpha-beta term is formed on the BF16
                        tensor cores from exact products of 8-bit digit slices
                        (integrals and C in 45-bit fixed point per row / 64-string tile,
@@ -115,11 +114,25 @@ int forte_set_stream(forte_ctx *ctx, void *cuda_stream);
 
 /* Select FORTE_FP64, FORTE_TF32, FORTE_BF16X2, FORTE_DF32 or FORTE_OZ64 for forte_sigma,
  * forte_davidson and forte_rdms (every mode but FORTE_FP64 forms the 2-RDM with
- * the tensor-core Gram, unless the FP64 one has at most 80 M products).  Default FORTE_FP64.  FORTE_ERR_ARG for other values.
+ * the tensor-core Gram, unless the FP64 one has at most 80 M products:
+ * forte_set_small_route).  Default FORTE_FP64.  FORTE_ERR_ARG for other values.
  * The paper computes in FP64 (FORTE_FP64); the other modes extend it and have no
  * counterpart there.
  */
 int forte_set_precision(forte_ctx *ctx, int mode);
+
+/* Small spaces in the modes other than FORTE_FP64, where the FP64 kernels are the faster
+ * ones: a sigma of up to 40 M products in FORTE_DF32, FORTE_OZ64 and the refinement of
+ * FORTE_TF32 / FORTE_BF16X2 (spaces with the gathered FP64 kernels), the 2-RDM of up to
+ * 80 M products in every such mode.
+ *   -1  (default) the FP64 kernels; in place of tensor-core kernels (FORTE_OZ64 and the
+ *       2-RDM) only while no wait budget of the caller's is set
+ *    0  the mode's own kernels at every size
+ *    1  the FP64 kernels whatever the wait budget
+ * FORTE_ERR_ARG for other values.
+ * Control entry point: the paper has no counterpart.
+ */
+int forte_set_small_route(forte_ctx *ctx, int route);
 
 /* N_alpha = C(n, nalpha), N_beta = C(n, nbeta) (host outputs, either may be NULL).
  * Control entry point: the paper has no counterpart.

@@ -83,6 +83,7 @@ def library():
         "forte_rdm3": [vp, vp, vp],
         "forte_set_gas": [vp, i, vp, vp, vp, vp],
         "forte_set_gas_route": [vp, i],
+        "forte_set_small_route": [vp, i],
         "forte_get_gas_route": [vp, vp, vp, vp],
         "forte_set_spin_parity": [vp, i],
         "forte_aci": [vp, d, d, i, d, i, vp, vp, vp, vp, vp],
@@ -265,6 +266,12 @@ def forte_set_gas(ctx, spaces, gmin, gmax):
 def forte_set_gas_route(ctx, route):
     """Restricted sigma route: -1 timed choice (default), 0 full grid, 1 kept determinants."""
     return _check(library().forte_set_gas_route(ctx, int(route)))
+
+
+def forte_set_small_route(ctx, route):
+    """Small spaces in the modes other than FP64: -1 the FP64 kernels (default), 0 the mode's
+    own kernels, 1 the FP64 kernels whatever the wait budget."""
+    return _check(library().forte_set_small_route(ctx, int(route)))
 
 
 def forte_get_gas_route(ctx):

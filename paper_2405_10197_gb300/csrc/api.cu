@@ -1097,6 +1097,14 @@ int forte_set_gas_route(forte_ctx *ctx, int route) {
   return FORTE_OK;
 }
 
+int forte_set_small_route(forte_ctx *ctx, int route) {
+  if (!ctx) { set_error("NULL context"); return FORTE_ERR_ARG; }
+  if (route < -1 || route > 1) { set_error("route must be -1, 0 or 1"); return FORTE_ERR_ARG; }
+  ctx->small_route = route;
+  for (int t = 0; t < 2; ++t) ctx->gas_pick[t] = ctx->gas_pick_mode[t] = -1;  // timed against other kernels
+  return FORTE_OK;
+}
+
 int forte_get_gas_route(const forte_ctx *ctx, int *route_fp64, int *route_fp32, double *ms) {
   if (!ctx) { set_error("NULL context"); return FORTE_ERR_ARG; }
   const bool cand = ctx->gas_on && !ctx->detmask_on && ctx->d_gas_off;

@@ -122,6 +122,7 @@ struct forte_ctx {
   float *d_gT_t32 = nullptr;
   int *d_err = nullptr;         // device status of bounded waits: [0] flag (0 = ok), [2..3] wait budget
   unsigned long long wait_budget = 0;  // clock cycles of one pipeline wait (0: the default)
+  int small_route = -1;                // forte_set_small_route
   // beta-string positions of the tensor-core alpha-beta kernel: strings grouped by a
   // linear 5-bit hash of their masks, one string per hash value in each aligned group
   // of 32 positions, so that the scatter of one warp meets 32 distinct banks
@@ -250,10 +251,14 @@ int upload_tables(forte_ctx *ctx);
 int sigma_fp64(forte_ctx *ctx, const double *C, double *S, int nvec);
 // the same with caller-provided beta-beta scratch T1, T2 (nvec * Ndet doubles each)
 int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, double *T1, double *T2);
-// FP64 multiply-adds of one sigma vector, and whether the FP64 kernels are the better
-// choice for nvec vectors in a mode that only asks for FP64-class results
+// FP64 multiply-adds of one sigma vector, and whether nvec vectors are few enough of them
+// for the FP64 kernels to be the better choice in a mode that only asks for FP64-class
+// results
 double fp64_products(const forte_ctx *ctx);
 bool fp64_small(const forte_ctx *ctx, int nvec);
+// Whether such a space takes the FP64 kernels (forte_set_small_route); waits: in place of
+// tensor-core kernels, whose waits a budget of the caller's is for
+bool small_route(const forte_ctx *ctx, bool waits);
 int hdiag_build(forte_ctx *ctx);
 // FP64-class sigma in double-FP32 arithmetic (relative error ~2^-46 per term);
 // with_ab = false leaves out the alpha-beta term (same-spin terms only)

@@ -491,11 +491,10 @@ int rdm12_fp64(forte_ctx *ctx, const double *bra, const double *ket, double *g1,
   if (g2 && !same) { set_error("the 2-RDM needs one state"); return FORTE_ERR_ARG; }
   // Small spaces keep the FP64 Gram in every mode (one GB300, forte_rdms: 27 M products, 9
   // orbitals with 5 + 4 electrons, 161 us against 202 us; 163 M, 10 with 5 + 5, 485
-  // against 361), unless the caller has set a wait budget, which is for the tensor-core
-  // kernels' waits.
+  // against 361).
   const double uv_products = (double)ND * (n2 * (n2 + 1.0) / 4);
   const bool oz = tensor_ok && g2 && ctx->precision != FORTE_FP64 && rdm2_oz_supported(ctx) &&
-                  (ctx->wait_budget || uv_products > 80e6);
+                  !(uv_products <= 80e6 && small_route(ctx, true));
   UvPlan pl = {};
   int rc;
   if (g2 && !oz && (rc = uv_plan<false>(n, ND, pl))) return rc;

@@ -326,6 +326,10 @@ bool fp64_small(const forte_ctx *ctx, int nvec) {
   return ctx->sd[1].ell_col && fp64_products(ctx) * nvec <= 40e6;
 }
 
+bool small_route(const forte_ctx *ctx, bool waits) {
+  return ctx->small_route == 1 || (ctx->small_route == -1 && !(waits && ctx->wait_budget));
+}
+
 // Columns per block: as many threads share an output as leave two blocks an SM busy, and
 // 32 columns once the grid is larger than that.
 static int sm_columns(long long NA, long long NB, int nvec) {
@@ -867,7 +871,8 @@ static int df_setup(forte_ctx *ctx) {
 }
 
 int sigma_df(forte_ctx *ctx, const double *C, double *S, int nvec, bool with_ab) {
-  if (with_ab && fp64_small(ctx, nvec)) return sigma_fp64(ctx, C, S, nvec);  // faster and more exact there
+  if (with_ab && small_route(ctx, false) && fp64_small(ctx, nvec))
+    return sigma_fp64(ctx, C, S, nvec);  // faster and more exact there
   int rc = df_setup(ctx);
   if (rc) return rc;
   cudaStream_t st = ctx->stream;

@@ -601,8 +601,7 @@ static int sigma_ab_oz(forte_ctx *ctx, const double *C, double *S, int nvec) {
 // tensor-core one does not apply (more than 15 orbitals, n_kl > 64).
 int sigma_oz64(forte_ctx *ctx, const double *C, double *S, int nvec) {
   if (!oz_ab_supported(ctx)) return sigma_df(ctx, C, S, nvec, true);
-  // (a wait budget the caller has set is for the tensor-core kernels' waits: they run)
-  if (!ctx->wait_budget && fp64_small(ctx, nvec)) return sigma_fp64(ctx, C, S, nvec);
+  if (small_route(ctx, true) && fp64_small(ctx, nvec)) return sigma_fp64(ctx, C, S, nvec);
   const bool ab = ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0;
   int rc = ab ? oz_ab_setup(ctx) : FORTE_OK;  // (waits for its uploads: before anything is queued)
   if (rc) return rc;
