@@ -123,6 +123,9 @@ struct forte_ctx {
   int *d_err = nullptr;         // device status of bounded waits: [0] flag (0 = ok), [2..3] wait budget
   unsigned long long wait_budget = 0;  // clock cycles of one pipeline wait (0: the default)
   int small_route = -1;                // forte_set_small_route
+  // lazily built tables that are complete (their pointers alone do not say so: an
+  // allocation may have failed between them)
+  bool df_ready = false, oz_ready = false, ozT_ready = false, mixed_ready = false, hd_ready = false;
   // beta-string positions of the tensor-core alpha-beta kernel: strings grouped by a
   // linear 5-bit hash of their masks, one string per hash value in each aligned group
   // of 32 positions, so that the scatter of one warp meets 32 distinct banks
@@ -241,6 +244,11 @@ cudaError_t set_smem_optin_max(const void *func);
 // afterwards see it.  (cudaMemcpy from pageable memory may return before its last chunk
 // has reached the device, and work on a non-blocking stream does not wait for it.)
 cudaError_t copy_in(const forte_ctx *ctx, void *dst, const void *src, size_t bytes);
+// Allocate *p, or keep it when an earlier set-up that could not be completed has.
+template <typename T>
+inline cudaError_t alloc_once(T **p, size_t bytes) {
+  return *p ? cudaSuccess : cudaMalloc((void **)p, bytes);
+}
 int build_spin_tables(forte_ctx *ctx);
 // Spaces whose gathered alpha rows fit in shared memory next to a second block: the FP64
 // sigma runs without transposes or atomics there (sigma_fp64.cu).

@@ -638,12 +638,13 @@ int rdm2_oz(forte_ctx *ctx, const double *C, const double *g1, double *g2) {
     const int rc_err = err_word_setup(ctx);
     if (rc_err) return rc_err;
   }
-  if (!ctx->d_ozT) {
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozT, sizeof(uint16_t) * (size_t)nU * NbP));
+  if (!ctx->ozT_ready) {
+    FORTE_CUDA_TRY(alloc_once(&ctx->d_ozT, sizeof(uint16_t) * (size_t)nU * NbP));
     FORTE_PROF(ctx, "oz_pairT");
     k_oz_pairT<<<(unsigned)std::min<long long>(((long long)nU * NbP + 255) / 256, 152LL * 32), 256, 0, st>>>(
         ctx->sd[1].dense, n, nU, NB, NbP, ctx->d_ozT);
     FORTE_LAUNCH_CHECK();
+    ctx->ozT_ready = true;
   }
   // workspace: Cfix, max |C|, row maxima, shifts, partial Grams, G+, G-
   size_t off = 0;

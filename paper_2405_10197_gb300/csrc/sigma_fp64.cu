@@ -845,21 +845,21 @@ static int ab_df(forte_ctx *ctx, const float *Chi, const float *Clo, double *S, 
 }
 
 static int df_setup(forte_ctx *ctx) {
-  if (ctx->d_gpair2) return FORTE_OK;
+  if (ctx->df_ready) return FORTE_OK;
   const int np = ctx->npair;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gpair2, sizeof(float2) * (size_t)np * np));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gpair2, sizeof(float2) * (size_t)np * np));
   k_df_pairs<<<(unsigned)std::min<long long>(((long long)np * np + 255) / 256, 1024), 256, 0, ctx->stream>>>(
       ctx->d_gpair, (float2 *)ctx->d_gpair2, (long long)np * np);
   FORTE_LAUNCH_CHECK();
   const long long nw = (long long)np * ctx->Nb;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_W2, sizeof(float2) * (size_t)nw));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_W2, sizeof(float2) * (size_t)nw));
   k_df_pairs<<<(unsigned)std::min<long long>((nw + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
       ctx->d_W, (float2 *)ctx->d_W2, nw);
   FORTE_LAUNCH_CHECK();
   const int nsp = ctx->same_strings ? 1 : 2;
   for (int s = 0; s < nsp; ++s) {
     const long long nnz = (long long)ctx->sh[s].csr_col.size();
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_csr_val2[s], sizeof(float2) * (size_t)std::max(1LL, nnz)));
+    FORTE_CUDA_TRY(alloc_once(&ctx->d_csr_val2[s], sizeof(float2) * (size_t)std::max(1LL, nnz)));
     if (nnz > 0) {
       k_df_pairs<<<(unsigned)std::min<long long>((nnz + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
           ctx->sd[s].csr_val, (float2 *)ctx->d_csr_val2[s], nnz);
@@ -867,6 +867,7 @@ static int df_setup(forte_ctx *ctx) {
     }
   }
   if (ctx->same_strings) ctx->d_csr_val2[1] = ctx->d_csr_val2[0];
+  ctx->df_ready = true;
   return FORTE_OK;
 }
 

@@ -766,7 +766,6 @@ static uint64_t splitmix64_next(uint64_t &state) {
 // one whose largest hash class is smallest is kept (fewest padding positions; at
 // CAS(14,14) 3584 positions for 3432 strings).
 static int ab_positions(forte_ctx *ctx) {
-  if (ctx->d_abTab) return FORTE_OK;
   const SpinHost &B = ctx->sh[ctx->same_strings ? 0 : 1];
   const int n = ctx->n;
   const long long NB = B.N;
@@ -849,14 +848,14 @@ static int ab_positions(forte_ctx *ctx) {
       const Repl &r = B.list[(size_t)J * B.nk + e];
       dcnt[r.J] = (int8_t)(dcnt[r.J] + (r.sgn < 0 ? -1 : 1));
     }
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abDcnt, dcnt.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_abDcnt, dcnt.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abDcnt, dcnt.data(), dcnt.size()));
   ctx->ab_split = split;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abTabL, sizeof(uint16_t) * tabL.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_abTabL, sizeof(uint16_t) * tabL.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abTabL, tabL.data(), sizeof(uint16_t) * tabL.size()));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abPosOf, sizeof(uint16_t) * posOf.size()));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abStrOf, sizeof(int) * strOf.size()));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_abTab, sizeof(uint16_t) * tab.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_abPosOf, sizeof(uint16_t) * posOf.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_abStrOf, sizeof(int) * strOf.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_abTab, sizeof(uint16_t) * tab.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abPosOf, posOf.data(), sizeof(uint16_t) * posOf.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abStrOf, strOf.data(), sizeof(int) * strOf.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_abTab, tab.data(), sizeof(uint16_t) * tab.size()));
@@ -866,14 +865,14 @@ static int ab_positions(forte_ctx *ctx) {
 
 int mixed_setup(forte_ctx *ctx) {
   const int np = ctx->npair;
-  if (ctx->d_gT_hi) return FORTE_OK;
+  if (ctx->mixed_ready) return FORTE_OK;
   double gm = 0.0;
   for (double x : ctx->eri) gm = std::max(gm, fabs(x));
   ctx->gmax = (float)(gm * (1.0 + 1e-6));
   size_t cnt = (size_t)128 * np;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gT_hi, cnt * sizeof(uint16_t)));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gT_lo, cnt * sizeof(uint16_t)));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gT_t32, cnt * sizeof(float)));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gT_hi, cnt * sizeof(uint16_t)));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gT_lo, cnt * sizeof(uint16_t)));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gT_t32, cnt * sizeof(float)));
   if (!ctx->d_err) {
     const int rc_err = err_word_setup(ctx);
     if (rc_err) return rc_err;
@@ -881,12 +880,16 @@ int mixed_setup(forte_ctx *ctx) {
   k_split_g<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_gpair, np, ctx->d_gT_hi, ctx->d_gT_lo,
                                                                     ctx->d_gT_t32);
   FORTE_LAUNCH_CHECK();
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gTT_hi, cnt * sizeof(uint16_t)));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_gTT_lo, cnt * sizeof(uint16_t)));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gTT_hi, cnt * sizeof(uint16_t)));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_gTT_lo, cnt * sizeof(uint16_t)));
   k_pair_major<<<(unsigned)((cnt + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_gT_hi, ctx->d_gT_lo, np, ctx->d_gTT_hi,
                                                                        ctx->d_gTT_lo);
   FORTE_LAUNCH_CHECK();
-  if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0) return ab_positions(ctx);
+  if (ctx->sh[0].nk > 0 && ctx->sh[ctx->same_strings ? 0 : 1].nk > 0) {
+    const int rc = ab_positions(ctx);
+    if (rc) return rc;
+  }
+  ctx->mixed_ready = true;
   return FORTE_OK;
 }
 

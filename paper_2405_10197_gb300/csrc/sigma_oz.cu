@@ -498,7 +498,7 @@ bool oz_ab_supported(const forte_ctx *ctx) {
 // Digits of the integrals: Gd[d][pq][rs] = digit d_(d+1) of rint((pq|rs) 2^ga[rs])
 // (BF16 bits, rs < 128, zero for rs >= npair), ga[rs] = 45 - e(max_pq |(pq|rs)|).
 static int oz_ab_setup(forte_ctx *ctx) {
-  if (ctx->d_ozG) return FORTE_OK;
+  if (ctx->oz_ready) return FORTE_OK;
   const int np = ctx->npair;
   std::vector<double> g((size_t)np * np);
   FORTE_CUDA_TRY(cudaMemcpy(g.data(), ctx->d_gpair, sizeof(double) * g.size(), cudaMemcpyDeviceToHost));
@@ -526,18 +526,19 @@ static int oz_ab_setup(forte_ctx *ctx) {
   }
   ctx->oz_gmax = gmax;
   const long long NBp = (ctx->Nb + ZB_TN - 1) / ZB_TN * ZB_TN;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozTabT, sizeof(uint16_t) * 128 * NBp));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_ozTabT, sizeof(uint16_t) * 128 * NBp));
   k_zb_tabT<<<(unsigned)std::min<long long>((128 * NBp + 255) / 256, 152LL * 16), 256, 0, ctx->stream>>>(
       ctx->sd[1].tabJ, ctx->Nb, NBp, ctx->d_ozTabT);
   FORTE_LAUNCH_CHECK();
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozG, sizeof(uint16_t) * gd.size()));
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_ozGa, sizeof(int) * 128));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_ozG, sizeof(uint16_t) * gd.size()));
+  FORTE_CUDA_TRY(alloc_once(&ctx->d_ozGa, sizeof(int) * 128));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_ozG, gd.data(), sizeof(uint16_t) * gd.size()));
   FORTE_CUDA_TRY(copy_in(ctx, ctx->d_ozGa, ga.data(), sizeof(int) * 128));
   if (!ctx->d_err) {
     const int rc_err = err_word_setup(ctx);
     if (rc_err) return rc_err;
   }
+  ctx->oz_ready = true;
   return FORTE_OK;
 }
 

@@ -373,14 +373,14 @@ bool ss_mma_supported(const forte_ctx *ctx) {
 }
 
 static int ss_dense_setup(forte_ctx *ctx) {
-  if (ctx->d_hd_hi[0]) return FORTE_OK;
+  if (ctx->hd_ready) return FORTE_OK;
   const int nsp = ctx->same_strings ? 1 : 2;
   for (int s = 0; s < nsp; ++s) {
     const long long N = s == 0 ? ctx->Na : ctx->Nb, Np = pad16(N);
     const size_t cnt = (size_t)N * Np;
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_hd_hi[s], cnt * sizeof(uint16_t)));
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_hd_lo[s], cnt * sizeof(uint16_t)));
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_hd_t32[s], cnt * sizeof(float)));
+    FORTE_CUDA_TRY(alloc_once(&ctx->d_hd_hi[s], cnt * sizeof(uint16_t)));
+    FORTE_CUDA_TRY(alloc_once(&ctx->d_hd_lo[s], cnt * sizeof(uint16_t)));
+    FORTE_CUDA_TRY(alloc_once(&ctx->d_hd_t32[s], cnt * sizeof(float)));
     FORTE_CUDA_TRY(cudaMemsetAsync(ctx->d_hd_hi[s], 0, cnt * sizeof(uint16_t), ctx->stream));
     FORTE_CUDA_TRY(cudaMemsetAsync(ctx->d_hd_lo[s], 0, cnt * sizeof(uint16_t), ctx->stream));
     FORTE_CUDA_TRY(cudaMemsetAsync(ctx->d_hd_t32[s], 0, cnt * sizeof(float), ctx->stream));
@@ -393,6 +393,7 @@ static int ss_dense_setup(forte_ctx *ctx) {
     ctx->d_hd_lo[1] = ctx->d_hd_lo[0];
     ctx->d_hd_t32[1] = ctx->d_hd_t32[0];
   }
+  ctx->hd_ready = true;
   return FORTE_OK;
 }
 

@@ -1,0 +1,125 @@
+"""A failed device allocation, at every place where a call makes one: the call reports it,
+the next call on the same context succeeds and launches the kernels of an undisturbed
+context with no table missing, and nothing is left allocated after the context is gone.
+
+Runs on the CPU: the library's host code in a process of its own on a runtime that records
+launches and fails the allocation it is told to (fake_cudart.cpp)."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+DRIVER = r"""
+import ctypes, sys
+import numpy as np
+import paper_2405_10197_gb300 as fg
+import synth_inputs as si
+
+fake = ctypes.CDLL(FAKE)
+fake.fake_log.restype = ctypes.c_char_p
+for f in (fake.fake_allocs, fake.fake_live):
+    f.restype = ctypes.c_longlong
+fake.fake_fail_at.argtypes = [ctypes.c_longlong]
+lib = fg.library()
+N, NA, NB = 6, 3, 2
+h, eri = si.integrals(N, 2 * N, seed=1)
+C = np.random.default_rng(0).normal(size=(2, 20, 15))
+S = np.zeros_like(C)
+G = [np.zeros((N,) * k) for k in (2, 4)]
+
+def log():
+    out = fake.fake_log().decode().split("\n")[:-1]
+    fake.fake_clear_log()
+    return out
+
+def create():
+    return lib.forte_cas_create(N, NA, NB, h.ctypes.data, eri.ctypes.data)
+
+def setup(mode):
+    ctx = create()
+    assert ctx
+    fg.forte_set_precision(ctx, mode)
+    fg.forte_set_small_route(ctx, 0)
+    log()
+    return ctx
+
+def each_failure(make, call):
+    # yields (context, codes of the disturbed and of the next call, launches of both)
+    k = 0
+    while True:
+        k += 1
+        ctx = make()
+        log()
+        fake.fake_fail_at(k)
+        before = fake.fake_allocs()
+        r1 = call(ctx)
+        made = fake.fake_allocs() - before
+        fake.fake_fail_at(-1)
+        if made < k:
+            assert r1 == 0
+            lib.forte_destroy(ctx)
+            assert k > 1, "the call allocates nothing: it tests nothing"
+            return
+        fake.cudaGetLastError()
+        l1 = log()
+        r2 = call(ctx)
+        yield k, ctx, r1, r2, l1, log()
+
+def check_call(make, call):
+    ctx = make()
+    log()
+    first = (call(ctx), log())[1]
+    steady = (call(ctx), log())[1]
+    lib.forte_destroy(ctx)
+    known = set(first) | set(steady)
+    for k, ctx, r1, r2, l1, l2 in each_failure(make, call):
+        what = f"allocation {k}: "
+        assert r1 in (fg.FORTE_ERR_ALLOC, fg.FORTE_ERR_CUDA), what + f"code {r1}"
+        assert r2 == 0, what + f"the next call returns {r2}: {fg.forte_last_error()}"
+        assert set(l1) <= known and set(l2) <= known, what + f"launches {sorted((set(l1) | set(l2)) - known)}"
+        it = iter(l2)
+        assert all(x in it for x in steady), what + f"launches {l2}, undisturbed {steady}"
+        r3, l3 = call(ctx), log()
+        assert r3 == 0 and l3 == steady, what + f"third call {l3}"
+        lib.forte_destroy(ctx)
+        assert fake.fake_live() == 0, what + f"{fake.fake_live()} allocations left"
+
+def sigma(ctx):
+    return lib.forte_sigma(ctx, C.ctypes.data, S.ctypes.data, 2)
+
+def test_sigma(mode):
+    check_call(lambda: setup(mode), sigma)
+
+def test_rdms(mode):
+    check_call(lambda: setup(mode), lambda ctx: lib.forte_rdms(ctx, C.ctypes.data, G[0].ctypes.data, G[1].ctypes.data))
+
+name, mode = sys.argv[1], int(sys.argv[2])
+globals()["test_" + name](mode)
+print("done")
+"""
+
+CALLS = [("sigma", m) for m in range(1, 5)] + [("rdms", 2)]
+
+
+@pytest.fixture(scope="module")
+def fake_runtime(tmp_path_factory):
+    from paper_2405_10197_gb300 import build
+    build.build()
+    inc = os.path.join(os.path.dirname(build._cuda_lib_dir(build._nvcc())), "include")
+    out = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
+    subprocess.run([shutil.which("g++"), "-shared", "-fPIC", "-std=c++17", "-I", inc,
+                    os.path.join(HERE, "fake_cudart.cpp"), "-o", out], check=True)
+    return out
+
+
+@pytest.mark.parametrize("call,mode", CALLS)
+def test_failed_allocations_are_reported_and_recovered_from(fake_runtime, call, mode):
+    code = f"FAKE = {fake_runtime!r}\n" + DRIVER
+    env = dict(os.environ, LD_PRELOAD=fake_runtime, PYTHONPATH=os.pathsep.join([ROOT, HERE]))
+    r = subprocess.run([sys.executable, "-c", code, call, str(mode)], env=env, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "done", r.stdout + r.stderr[-2000:]
