@@ -97,7 +97,7 @@ void sym_eig(int k, const double *A, double *w, double *U) {
 }
 
 int err_word_setup(forte_ctx *ctx) {
-  if (!ctx->d_err) FORTE_CUDA_TRY(cudaMalloc(&ctx->d_err, 4 * sizeof(int)));
+  if (!ctx->d_err) FORTE_CUDA_TRY(dev_alloc(&ctx->d_err, 4 * sizeof(int)));
   const unsigned long long b = ctx->wait_budget ? ctx->wait_budget : 4000000000ull;
   const int w[4] = {0, 0, (int)(unsigned)(b & 0xFFFFFFFFull), (int)(unsigned)(b >> 32)};
   FORTE_CUDA_TRY(cudaMemcpyAsync(ctx->d_err, w, sizeof(w), cudaMemcpyHostToDevice, ctx->stream));
@@ -972,7 +972,7 @@ int forte_set_guess(forte_ctx *ctx, const double *C, int nvec) {
   ctx->d_guess = nullptr;
   ctx->nguess = 0;
   if (nvec == 0) return FORTE_OK;
-  FORTE_CUDA_TRY(cudaMalloc(&ctx->d_guess, sizeof(double) * ctx->Ndet * nvec));
+  FORTE_CUDA_TRY(dev_alloc(&ctx->d_guess, sizeof(double) * ctx->Ndet * nvec));
   FORTE_CUDA_TRY(cudaMemcpyAsync(ctx->d_guess, C, sizeof(double) * ctx->Ndet * nvec, cudaMemcpyDeviceToDevice,
                                  ctx->stream));
   ctx->nguess = nvec;
@@ -987,7 +987,7 @@ static int ensure_roots(forte_ctx *ctx, int nroots) {
     cudaFree(ctx->d_roots);
     ctx->d_roots = nullptr;
     ctx->d_roots_cap = 0;
-    if (cudaMalloc(&ctx->d_roots, want) != cudaSuccess) {
+    if (dev_alloc(&ctx->d_roots, want) != cudaSuccess) {
       set_error("cudaMalloc roots failed");
       return FORTE_ERR_ALLOC;
     }

@@ -1148,7 +1148,7 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
   // ---- one pooled device allocation for the batch
   char *dbuf = nullptr;
   if (!classes.empty()) {
-    cudaError_t e = cudaMalloc(&dbuf, total_bytes);
+    cudaError_t e = dev_alloc(&dbuf, total_bytes);
     if (e != cudaSuccess) {
       set_error("forte_batch_solve: cudaMalloc(%zu) failed: %s", total_bytes, cudaGetErrorString(e));
       return FORTE_ERR_ALLOC;

@@ -21,6 +21,7 @@ void clear_error();
     if (e_ != cudaSuccess) {                                                               \
       forte::set_error("%s failed: %s (%s:%d)", #expr, cudaGetErrorString(e_), __FILE__,   \
                        __LINE__);                                                          \
+      cudaGetLastError(); /* reported here: not the next launch's error */                 \
       return FORTE_ERR_CUDA;                                                               \
     }                                                                                      \
   } while (0)
@@ -34,6 +35,18 @@ void clear_error();
       return FORTE_ERR_CUDA;                                                               \
     }                                                                                      \
   } while (0)
+
+// cudaMalloc whose failure is the return value alone: left in the runtime's last error, it
+// would be taken for the failure of the next launch.
+template <typename T>
+inline cudaError_t dev_alloc(T **p, size_t bytes) {
+  const cudaError_t e = cudaMalloc((void **)p, bytes);
+  if (e != cudaSuccess) {
+    *p = nullptr;
+    cudaGetLastError();
+  }
+  return e;
+}
 
 // One entry of the compact single-replacement list of a string I:
 // E_pq |I> = sgn |J>,  valid when q is in I and (p not in I or p == q).
@@ -247,7 +260,7 @@ cudaError_t copy_in(const forte_ctx *ctx, void *dst, const void *src, size_t byt
 // Allocate *p, or keep it when an earlier set-up that could not be completed has.
 template <typename T>
 inline cudaError_t alloc_once(T **p, size_t bytes) {
-  return *p ? cudaSuccess : cudaMalloc((void **)p, bytes);
+  return *p ? cudaSuccess : dev_alloc(p, bytes);
 }
 int build_spin_tables(forte_ctx *ctx);
 // Spaces whose gathered alpha rows fit in shared memory next to a second block: the FP64

@@ -474,14 +474,14 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     return FORTE_OK;
   }
   for (int s = 0; s < 2; ++s) {
-    if (cudaMalloc(&ctx->d_gas_cls[s], sizeof(int) * cls[s].size()) != cudaSuccess) {
+    if (dev_alloc(&ctx->d_gas_cls[s], sizeof(int) * cls[s].size()) != cudaSuccess) {
       gas_release(ctx);
       set_error("cudaMalloc of the string classes failed");
       return FORTE_ERR_ALLOC;
     }
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cls[s], cls[s].data(), sizeof(int) * cls[s].size()));
   }
-  if (cudaMalloc(&ctx->d_gas_ok, ok.size()) != cudaSuccess) {
+  if (dev_alloc(&ctx->d_gas_ok, ok.size()) != cudaSuccess) {
     gas_release(ctx);
     set_error("cudaMalloc of the class table failed");
     return FORTE_ERR_ALLOC;
@@ -500,7 +500,7 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
       maxnnz = std::max(maxnnz, ctx->sh[0].csr_ptr[i + 1] - ctx->sh[0].csr_ptr[i]);
     }
     std::stable_sort(rowsv.begin(), rowsv.end(), [&](int x, int y) { return kept[cls[0][x]] > kept[cls[0][y]]; });
-    if (cudaMalloc(&ctx->d_gas_rows, sizeof(int) * std::max<size_t>(1, rowsv.size())) != cudaSuccess) {
+    if (dev_alloc(&ctx->d_gas_rows, sizeof(int) * std::max<size_t>(1, rowsv.size())) != cudaSuccess) {
       gas_release(ctx);
       set_error("cudaMalloc of the restricted-sigma rows failed");
       return FORTE_ERR_ALLOC;
@@ -526,15 +526,15 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
       for (int b = 0; b < ncB; ++b)
         if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
     int *d_flag = nullptr, flag = 0;
-    if (cudaMalloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)B.N * noB)) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_tcls, (size_t)ncB * noB + 1) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
-        cudaMalloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || cudaMalloc(&d_flag, sizeof(int)) != cudaSuccess) {
+    if (dev_alloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)B.N * noB)) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_tcls, (size_t)ncB * noB + 1) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
+        dev_alloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || dev_alloc(&d_flag, sizeof(int)) != cudaSuccess) {
       gas_release(ctx);
       set_error("cudaMalloc of the restricted-sigma class lists failed");
       return FORTE_ERR_ALLOC;

@@ -508,7 +508,7 @@ int rdm12_fp64(forte_ctx *ctx, const double *bra, const double *ket, double *g1,
   double *P = (double *)(w + off_P);
   double *g1w = g1 ? g1 : (double *)(w + off_g1);
   if (oz && !g1) {  // the Gram step reallocates sc_rdm: keep the 1-RDM elsewhere
-    if (!ctx->d_g1tmp) FORTE_CUDA_TRY(cudaMalloc(&ctx->d_g1tmp, sizeof(double) * n2));
+    if (!ctx->d_g1tmp) FORTE_CUDA_TRY(dev_alloc(&ctx->d_g1tmp, sizeof(double) * n2));
     g1w = ctx->d_g1tmp;
   }
 

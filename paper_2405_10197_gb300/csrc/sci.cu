@@ -295,8 +295,8 @@ forte_sci *forte_sci_create(int norb, const double *h, const double *eri) {
     if (!std::isfinite(eri[k])) { set_error("forte_sci_create: eri contains NaN/Inf"); return nullptr; }
   forte_sci *s = new forte_sci();
   s->n = norb;
-  if (cudaGetDevice(&s->device) != cudaSuccess || cudaMalloc(&s->d_h, sizeof(double) * n * n) != cudaSuccess ||
-      cudaMalloc(&s->d_eri, sizeof(double) * n4) != cudaSuccess ||
+  if (cudaGetDevice(&s->device) != cudaSuccess || dev_alloc(&s->d_h, sizeof(double) * n * n) != cudaSuccess ||
+      dev_alloc(&s->d_eri, sizeof(double) * n4) != cudaSuccess ||
       cudaMemcpy(s->d_h, h, sizeof(double) * n * n, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(s->d_eri, eri, sizeof(double) * n4, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaStreamSynchronize(nullptr) != cudaSuccess) {  // (the handle's stream may not wait for the default one)

@@ -240,7 +240,7 @@ bool sigma_small(const forte_ctx *ctx) {
 template <typename T>
 static int upload(T **dst, const T *src, size_t count) {
   size_t bytes = sizeof(T) * (count ? count : 1);
-  cudaError_t e = cudaMalloc((void **)dst, bytes);
+  cudaError_t e = dev_alloc(dst, bytes);
   if (e != cudaSuccess) {
     set_error("cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
     return FORTE_ERR_ALLOC;
@@ -272,7 +272,7 @@ int upload_tables(forte_ctx *ctx) {
       }
     if ((st = upload(&D.dense, dense.data(), dense.size()))) return st;
     const int nko = H.nel * (n - H.nel);
-    if (cudaMalloc(&D.off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)H.N * nko)) != cudaSuccess) {
+    if (dev_alloc(&D.off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)H.N * nko)) != cudaSuccess) {
       set_error("cudaMalloc of the replacement lists failed");
       return FORTE_ERR_ALLOC;
     }
@@ -302,7 +302,7 @@ int upload_tables(forte_ctx *ctx) {
   if ((st = upload(&ctx->d_gpair, gp.data(), gp.size()))) return st;
   {
     const SpinHost &B = ctx->sh[ctx->same_strings ? 0 : 1];
-    if (cudaMalloc(&ctx->d_W, sizeof(double) * (size_t)np * B.N) != cudaSuccess) {
+    if (dev_alloc(&ctx->d_W, sizeof(double) * (size_t)np * B.N) != cudaSuccess) {
       set_error("cudaMalloc of the occupation sums failed");
       return FORTE_ERR_ALLOC;
     }
@@ -337,7 +337,7 @@ int Scratch::ensure(size_t want) {
   }
   ptr = nullptr;
   bytes = 0;
-  cudaError_t e = cudaMalloc(&ptr, want);
+  cudaError_t e = dev_alloc(&ptr, want);
   if (e != cudaSuccess) {
     ptr = nullptr;
     set_error("cudaMalloc(%zu) failed: %s", want, cudaGetErrorString(e));

@@ -508,10 +508,10 @@ int hdiag_build(forte_ctx *ctx) {
       W[(size_t)ia * n + j] = v;
     }
   double *dW = nullptr;
-  FORTE_CUDA_TRY(cudaMalloc(&dW, sizeof(double) * W.size()));
+  FORTE_CUDA_TRY(dev_alloc(&dW, sizeof(double) * W.size()));
   FORTE_CUDA_TRY(copy_in(ctx, dW, W.data(), sizeof(double) * W.size()));
   if (!ctx->d_hdiag) {
-    cudaError_t e = cudaMalloc(&ctx->d_hdiag, sizeof(double) * ctx->Ndet);
+    cudaError_t e = dev_alloc(&ctx->d_hdiag, sizeof(double) * ctx->Ndet);
     if (e != cudaSuccess) {
       cudaFree(dW);
       set_error("cudaMalloc hdiag failed: %s", cudaGetErrorString(e));

@@ -1223,7 +1223,7 @@ static int part_buffer(forte_ctx *ctx, size_t doubles, double **p, unsigned **co
   if (rc) return rc;
   *p = (double *)ctx->sc_small.ptr;
   if (!ctx->d_vk_count) {
-    FORTE_CUDA_TRY(cudaMalloc(&ctx->d_vk_count, sizeof(unsigned)));
+    FORTE_CUDA_TRY(dev_alloc(&ctx->d_vk_count, sizeof(unsigned)));
     FORTE_CUDA_TRY(cudaMemsetAsync(ctx->d_vk_count, 0, sizeof(unsigned), ctx->stream));
   }
   *counter = ctx->d_vk_count;

@@ -15,7 +15,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 
 DRIVER = r"""
-import ctypes, sys
+import ctypes, math, sys
 import numpy as np
 import paper_2405_10197_gb300 as fg
 import synth_inputs as si
@@ -26,11 +26,11 @@ for f in (fake.fake_allocs, fake.fake_live):
     f.restype = ctypes.c_longlong
 fake.fake_fail_at.argtypes = [ctypes.c_longlong]
 lib = fg.library()
-N, NA, NB = 6, 3, 2
+N, NA, NB = map(int, sys.argv[3:6])
 h, eri = si.integrals(N, 2 * N, seed=1)
-C = np.random.default_rng(0).normal(size=(2, 20, 15))
+C = np.zeros((2, math.comb(N, NA), math.comb(N, NB)))
 S = np.zeros_like(C)
-G = [np.zeros((N,) * k) for k in (2, 4)]
+G = [np.zeros((N,) * k) for k in (2, 4, 6)]
 
 def log():
     out = fake.fake_log().decode().split("\n")[:-1]
@@ -65,7 +65,6 @@ def each_failure(make, call):
             lib.forte_destroy(ctx)
             assert k > 1, "the call allocates nothing: it tests nothing"
             return
-        fake.cudaGetLastError()
         l1 = log()
         r2 = call(ctx)
         yield k, ctx, r1, r2, l1, log()
@@ -92,18 +91,36 @@ def check_call(make, call):
 def sigma(ctx):
     return lib.forte_sigma(ctx, C.ctypes.data, S.ctypes.data, 2)
 
+def test_create():
+    for k in range(1, 1000):
+        fake.fake_fail_at(k)
+        ctx = create()
+        if ctx:
+            lib.forte_destroy(ctx)
+            fake.fake_fail_at(-1)
+            assert k > 10
+            break
+        assert fake.fake_live() == 0, f"allocation {k}: {fake.fake_live()} left"
+        log()
+    assert fake.fake_live() == 0
+
 def test_sigma(mode):
     check_call(lambda: setup(mode), sigma)
 
 def test_rdms(mode):
     check_call(lambda: setup(mode), lambda ctx: lib.forte_rdms(ctx, C.ctypes.data, G[0].ctypes.data, G[1].ctypes.data))
 
+def test_rdm3(mode):
+    check_call(lambda: setup(mode), lambda ctx: lib.forte_rdm3(ctx, C.ctypes.data, G[2].ctypes.data))
+
 name, mode = sys.argv[1], int(sys.argv[2])
-globals()["test_" + name](mode)
+globals()["test_" + name](*([mode] if mode >= 0 else []))
 print("done")
 """
 
-CALLS = [("sigma", m) for m in range(1, 5)] + [("rdms", 2)]
+SMALL, TILED = (6, 3, 2), (11, 4, 5)  # orbitals, electrons: gathered and tiled FP64 sigma
+CALLS = ([("create", -1, SMALL), ("sigma", 0, TILED), ("rdm3", 0, SMALL)] + [("sigma", m, SMALL) for m in range(1, 5)] +
+         [("rdms", m, SMALL) for m in (0, 2)])
 
 
 @pytest.fixture(scope="module")
@@ -117,9 +134,9 @@ def fake_runtime(tmp_path_factory):
     return out
 
 
-@pytest.mark.parametrize("call,mode", CALLS)
-def test_failed_allocations_are_reported_and_recovered_from(fake_runtime, call, mode):
+@pytest.mark.parametrize("call,mode,space", CALLS)
+def test_failed_allocations_are_reported_and_recovered_from(fake_runtime, call, mode, space):
     code = f"FAKE = {fake_runtime!r}\n" + DRIVER
     env = dict(os.environ, LD_PRELOAD=fake_runtime, PYTHONPATH=os.pathsep.join([ROOT, HERE]))
-    r = subprocess.run([sys.executable, "-c", code, call, str(mode)], env=env, capture_output=True, text=True, timeout=300)
+    r = subprocess.run([sys.executable, "-c", code, call, *map(str, (mode, *space))], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "done", r.stdout + r.stderr[-2000:]
