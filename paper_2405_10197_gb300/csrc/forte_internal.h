@@ -72,6 +72,14 @@ struct SpinHost {
   std::vector<double> diag;        // H_ss[I][I]
 };
 
+// Device memory of a function's own.
+struct DevTemp {
+  void *ptr = nullptr;
+  ~DevTemp() {
+    if (ptr) cudaFree(ptr);
+  }
+};
+
 // Device-side copies of one spin's tables.
 struct SpinDev {
   Repl *list = nullptr;

@@ -525,7 +525,8 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     for (int a = 0; a < ncA; ++a)
       for (int b = 0; b < ncB; ++b)
         if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
-    int *d_flag = nullptr, flag = 0;
+    DevTemp tmp;
+    int flag = 0;
     if (dev_alloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
         dev_alloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
         dev_alloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
@@ -534,7 +535,7 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
         dev_alloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
         dev_alloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
         dev_alloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || dev_alloc(&d_flag, sizeof(int)) != cudaSuccess) {
+        dev_alloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || dev_alloc(&tmp.ptr, sizeof(int)) != cudaSuccess) {
       gas_release(ctx);
       set_error("cudaMalloc of the restricted-sigma class lists failed");
       return FORTE_ERR_ALLOC;
@@ -542,6 +543,7 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size()));
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size()));
     FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_okm, okm.data(), sizeof(okm[0]) * okm.size()));
+    int *d_flag = (int *)tmp.ptr;
     FORTE_CUDA_TRY(copy_in(ctx, d_flag, &flag, sizeof(int)));
     const unsigned nbk = (unsigned)((B.N + 63) / 64);
     k_gas_order<<<nbk, 64, 0, ctx->stream>>>(ctx->sd[1].off, noB, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col,
@@ -554,7 +556,6 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     FORTE_LAUNCH_CHECK();
     FORTE_CUDA_TRY(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
     FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    cudaFree(d_flag);
     if (flag) {
       gas_release(ctx);
       set_error("internal: strings of one class differ in their replacements");

@@ -507,13 +507,13 @@ int hdiag_build(forte_ctx *ctx) {
         if ((A.str[ia] >> i) & 1u) v += ctx->eri[(((size_t)i * n + i) * n + j) * n + j];
       W[(size_t)ia * n + j] = v;
     }
-  double *dW = nullptr;
-  FORTE_CUDA_TRY(dev_alloc(&dW, sizeof(double) * W.size()));
+  DevTemp tmp;
+  FORTE_CUDA_TRY(dev_alloc(&tmp.ptr, sizeof(double) * W.size()));
+  double *dW = (double *)tmp.ptr;
   FORTE_CUDA_TRY(copy_in(ctx, dW, W.data(), sizeof(double) * W.size()));
   if (!ctx->d_hdiag) {
     cudaError_t e = dev_alloc(&ctx->d_hdiag, sizeof(double) * ctx->Ndet);
     if (e != cudaSuccess) {
-      cudaFree(dW);
       set_error("cudaMalloc hdiag failed: %s", cudaGetErrorString(e));
       return FORTE_ERR_ALLOC;
     }
@@ -523,7 +523,6 @@ int hdiag_build(forte_ctx *ctx) {
       ctx->sd[0].diag, ctx->sd[1].diag, dW, ctx->sd[1].str, n, ctx->Na, ctx->Nb, ctx->d_hdiag);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-  cudaFree(dW);
   if (e != cudaSuccess) {
     set_error("hdiag kernel failed: %s", cudaGetErrorString(e));
     return FORTE_ERR_CUDA;

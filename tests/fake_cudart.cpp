@@ -1,8 +1,9 @@
 // A CUDA runtime without a GPU, for tests of the library's host code on the CPU: preloaded
 // before libforte_gpu.so, it takes the place of the runtime calls the library makes.
 // Device memory is host memory, kernels are not run: a launch is recorded with the
-// kernel's name and the positions of its null pointer arguments.  The n-th allocation
-// from now on can be made to fail (fake_fail_at), and live allocations are counted.
+// kernel's name and the positions of its null pointer arguments.  The n-th allocation or
+// asynchronous copy from now on can be made to fail (fake_fail_at, fake_fail_copy_at), and
+// live allocations are counted.
 #include <cuda_runtime_api.h>
 #include <cxxabi.h>
 
@@ -20,7 +21,7 @@ struct Kernel {
 struct State {
   std::map<const void *, Kernel> kernels;
   std::map<void *, size_t> live;
-  long long allocs = 0, fail_at = -1;
+  long long allocs = 0, fail_at = -1, copies = 0, fail_copy_at = -1;
   cudaError_t last = cudaSuccess;
   std::string log;
   dim3 grid, block;
@@ -99,6 +100,7 @@ int no_tensor_map(...) { return 0; }  // cuTensorMapEncodeTiled
 extern "C" {
 // ---- for the tests
 void fake_fail_at(long long n) { st().fail_at = n < 0 ? -1 : st().allocs + n; }
+void fake_fail_copy_at(long long n) { st().fail_copy_at = n < 0 ? -1 : st().copies + n; }
 long long fake_allocs() { return st().allocs; }
 long long fake_live() { return (long long)st().live.size(); }
 int fake_last_error() { return (int)st().last; }
@@ -150,6 +152,7 @@ cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) {
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  if (++st().copies == st().fail_copy_at) return fail(cudaErrorInvalidValue);
   memmove(d, s, n);
   return cudaSuccess;
 }

@@ -1,9 +1,10 @@
 """A failed device allocation, at every place where a call makes one: the call reports it,
 the next call on the same context succeeds and launches the kernels of an undisturbed
 context with no table missing, and nothing is left allocated after the context is gone.
+Failed copies leave nothing allocated either.
 
 Runs on the CPU: the library's host code in a process of its own on a runtime that records
-launches and fails the allocation it is told to (fake_cudart.cpp)."""
+launches and fails the allocation or copy it is told to (fake_cudart.cpp)."""
 import os
 import shutil
 import subprocess
@@ -24,7 +25,8 @@ fake = ctypes.CDLL(FAKE)
 fake.fake_log.restype = ctypes.c_char_p
 for f in (fake.fake_allocs, fake.fake_live):
     f.restype = ctypes.c_longlong
-fake.fake_fail_at.argtypes = [ctypes.c_longlong]
+for f in (fake.fake_fail_at, fake.fake_fail_copy_at):
+    f.argtypes = [ctypes.c_longlong]
 lib = fg.library()
 N, NA, NB = map(int, sys.argv[3:6])
 h, eri = si.integrals(N, 2 * N, seed=1)
@@ -113,6 +115,25 @@ def test_rdms(mode):
 def test_rdm3(mode):
     check_call(lambda: setup(mode), lambda ctx: lib.forte_rdm3(ctx, C.ctypes.data, G[2].ctypes.data))
 
+def gas(ctx):
+    a = ctypes.c_int * 3
+    return lib.forte_set_gas(ctx, 3, a(2, 2, 2), a(3, 0, 0), a(4, 4, 1), None)
+
+def test_gas_copies(mode):
+    k = 0
+    while True:
+        k += 1
+        ctx = setup(mode)
+        fake.fake_fail_copy_at(k)
+        rc = gas(ctx)
+        fake.fake_fail_copy_at(-1)
+        lib.forte_destroy(ctx)
+        assert fake.fake_live() == 0, f"copy {k}: {fake.fake_live()} allocations left"
+        if rc == 0:
+            break
+        assert rc == fg.FORTE_ERR_CUDA
+    assert k > 5
+
 name, mode = sys.argv[1], int(sys.argv[2])
 globals()["test_" + name](*([mode] if mode >= 0 else []))
 print("done")
@@ -120,7 +141,7 @@ print("done")
 
 SMALL, TILED = (6, 3, 2), (11, 4, 5)  # orbitals, electrons: gathered and tiled FP64 sigma
 CALLS = ([("create", -1, SMALL), ("sigma", 0, TILED), ("rdm3", 0, SMALL)] + [("sigma", m, SMALL) for m in range(1, 5)] +
-         [("rdms", m, SMALL) for m in (0, 2)])
+         [("rdms", m, SMALL) for m in (0, 2)] + [("gas_copies", 0, SMALL)])
 
 
 @pytest.fixture(scope="module")
