@@ -72,6 +72,14 @@ struct SpinHost {
   std::vector<double> diag;        // H_ss[I][I]
 };
 
+// Whether all rows of a CSR matrix have as many entries as the first.  (Those of a string
+// Hamiltonian do: every string has as many single and double replacements.)
+inline bool rows_alike(const std::vector<int> &ptr) {
+  for (size_t i = 1; i + 1 < ptr.size(); ++i)
+    if (ptr[i + 1] - ptr[i] != ptr[1] - ptr[0]) return false;
+  return true;
+}
+
 // Device memory of a function's own.
 struct DevTemp {
   void *ptr = nullptr;

@@ -59,7 +59,8 @@ __global__ void k_det_fill(T *__restrict__ x, long long total, long long nd, con
 //   gas_ellc / gas_ellv (and FP32 values): H_bb rows by column class, entry-major within a
 //             class (base nnz coff[class], then [nnz][strings of the class])
 //   gas_ccls  [class][nnz]: column class of each position
-// Built on the device; one thread per beta string (in class order).
+// Built on the device, from rows of nnz entries each; one thread per beta string (in class
+// order).
 constexpr int GAS_MAXCLS = 64;
 
 __global__ void k_gas_order(const uint32_t *__restrict__ off, int no, const int *__restrict__ ptr,
@@ -67,7 +68,7 @@ __global__ void k_gas_order(const uint32_t *__restrict__ off, int no, const int 
                             const int *__restrict__ cls, int nc, const int *__restrict__ coff,
                             const int *__restrict__ cstr, int N, uint32_t *__restrict__ goff,
                             uint8_t *__restrict__ tcls, int *__restrict__ ellc, double *__restrict__ ellv,
-                            float *__restrict__ ellv32, uint8_t *__restrict__ ccls, int *__restrict__ flag) {
+                            float *__restrict__ ellv32, uint8_t *__restrict__ ccls) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
   const int J = cstr[i], b = cls[J], i0 = coff[b], nb = coff[b + 1] - i0, ii = i - i0;
@@ -83,10 +84,6 @@ __global__ void k_gas_order(const uint32_t *__restrict__ off, int no, const int 
     const int c = ot(e), p = at[c]++;
     goff[(long long)J * no + p] = off[(long long)J * no + e];
     if (ii == 0) tcls[b * no + p] = (uint8_t)c;
-  }
-  if (ptr[J + 1] - ptr[J] != nnz) {
-    *flag = 1;
-    return;
   }
   auto ct = [&](int e) { return cls[col[ptr[J] + e]]; };
   starts(ct, nnz);
@@ -525,6 +522,11 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     for (int a = 0; a < ncA; ++a)
       for (int b = 0; b < ncB; ++b)
         if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
+    if (!rows_alike(B.csr_ptr)) {  // before any kernel takes nnz entries from a row
+      gas_release(ctx);
+      set_error("internal: string Hamiltonian rows of different lengths");
+      return FORTE_ERR_ARG;
+    }
     DevTemp tmp;
     int flag = 0;
     if (dev_alloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
@@ -549,7 +551,7 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     k_gas_order<<<nbk, 64, 0, ctx->stream>>>(ctx->sd[1].off, noB, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col,
                                              ctx->sd[1].csr_val, nnz, ctx->d_gas_cls[1], ncB, ctx->d_gas_coff,
                                              ctx->d_gas_cstr, (int)B.N, ctx->d_gas_off, ctx->d_gas_tcls, ctx->d_gas_ellc,
-                                             ctx->d_gas_ellv, ctx->d_gas_ellv32, ctx->d_gas_ccls, d_flag);
+                                             ctx->d_gas_ellv, ctx->d_gas_ellv32, ctx->d_gas_ccls);
     FORTE_LAUNCH_CHECK();
     k_gas_check<<<nbk, 64, 0, ctx->stream>>>(ctx->d_gas_off, noB, ctx->d_gas_tcls, ctx->d_gas_ellc, nnz, ctx->d_gas_ccls,
                                              ctx->d_gas_cls[1], ctx->d_gas_coff, ctx->d_gas_cstr, (int)B.N, d_flag);

@@ -232,9 +232,7 @@ bool sigma_small(const forte_ctx *ctx) {
   const SpinHost &A = ctx->sh[0], &B = ctx->sh[ctx->same_strings ? 0 : 1];
   const long long k = A.nel * (ctx->n - A.nel) + 1;
   if (8 * k * (B.N + ctx->npair) > 100 * 1024) return false;
-  for (long long j = 0; j < B.N; ++j)  // rows of one length (they are, for string Hamiltonians)
-    if (B.csr_ptr[j + 1] - B.csr_ptr[j] != B.csr_ptr[1]) return false;
-  return true;
+  return rows_alike(B.csr_ptr);
 }
 
 template <typename T>

@@ -161,3 +161,18 @@ def test_failed_allocations_are_reported_and_recovered_from(fake_runtime, call, 
     env = dict(os.environ, LD_PRELOAD=fake_runtime, PYTHONPATH=os.pathsep.join([ROOT, HERE]))
     r = subprocess.run([sys.executable, "-c", code, call, *map(str, (mode, *space))], env=env, capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "done", r.stdout + r.stderr[-2000:]
+
+
+def test_rows_of_different_lengths_are_seen_before_they_are_read(tmp_path):
+    """rows_alike guards the kernels that take as many entries from every row as the first has."""
+    from paper_2405_10197_gb300 import build
+    inc = os.path.join(os.path.dirname(build._cuda_lib_dir(build._nvcc())), "include")
+    src = tmp_path / "rows.cpp"
+    src.write_text('#include "forte_internal.h"\n#include <cstdio>\nint main() {\n'
+                   '  for (const std::vector<int> &p : std::vector<std::vector<int>>{\n'
+                   '           {0, 3}, {0, 3, 6, 9}, {0, 3, 6, 8}, {0, 2, 5, 8}, {0, 3, 7, 10}, {0, 0, 0}, {0, 0, 1}, {0}})\n'
+                   '    printf("%d", (int)forte::rows_alike(p));\n}\n')
+    exe = str(tmp_path / "rows")
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-I", inc, "-I", os.path.join(ROOT, "paper_2405_10197_gb300", "csrc"),
+                    str(src), "-o", exe], check=True)
+    assert subprocess.run([exe], capture_output=True, text=True, check=True).stdout == "11000101"
