@@ -166,7 +166,8 @@ int forte_get_hdiag(const forte_ctx *ctx, double *hdiag);
  * projected.  Vectors keep the full [N_alpha][N_beta] layout, zero outside.
  * The RDM calls act on whatever vectors they are given.  When at most a quarter
  * of the determinants is kept (and the beta strings fall in at most 64
- * occupation classes), sigma has a second exact route besides the full-grid
+ * occupation classes, and there was memory for the lists of its kernel, 16 bytes an
+ * entry of the beta string Hamiltonian), sigma has a second exact route besides the full-grid
  * kernels of the precision mode followed by the projection: a kernel over the
  * kept determinants only, in FP64 (FP32 for the FP32 vectors of the
  * reduced-precision Davidson phase), whose cost follows the kept space.  By
@@ -182,7 +183,7 @@ int forte_set_gas(forte_ctx *ctx, int nspace, const int *size, const int *gmin, 
 
 /* Route of the restricted sigma (see forte_set_gas): -1 timed choice (default),
  * 0 full-grid kernels + projection, 1 the kept-determinant kernel (for any
- * restriction with at most 64 beta occupation classes; otherwise the full grid).
+ * restriction that has it; otherwise the full grid).
  * Clears earlier timings.  FORTE_ERR_ARG for other values.
  * Control entry point: the paper has no counterpart.
  */

@@ -376,6 +376,23 @@ long long space_dim(const forte_ctx *ctx) {
   return (K - D) / 2 + (ctx->spin_parity > 0 ? D : 0);
 }
 
+// The lists of the kept-determinant kernel; without them sigma runs on the full grid.
+static void gas_lists_release(forte_ctx *ctx) {
+  auto drop = [](auto *&p) {
+    cudaFree(p);
+    p = nullptr;
+  };
+  drop(ctx->d_gas_coff);
+  drop(ctx->d_gas_cstr);
+  drop(ctx->d_gas_off);
+  drop(ctx->d_gas_okm);
+  drop(ctx->d_gas_tcls);
+  drop(ctx->d_gas_ellc);
+  drop(ctx->d_gas_ellv);
+  drop(ctx->d_gas_ellv32);
+  drop(ctx->d_gas_ccls);
+}
+
 static void gas_release(forte_ctx *ctx) {
   for (int s = 0; s < 2; ++s) {
     cudaFree(ctx->d_gas_cls[s]);
@@ -385,21 +402,8 @@ static void gas_release(forte_ctx *ctx) {
   cudaFree(ctx->d_gas_ok);
   ctx->d_gas_ok = nullptr;
   cudaFree(ctx->d_gas_rows);
-  cudaFree(ctx->d_gas_coff);
-  cudaFree(ctx->d_gas_cstr);
-  cudaFree(ctx->d_gas_off);
-  cudaFree(ctx->d_gas_okm);
-  ctx->d_gas_okm = nullptr;
-  cudaFree(ctx->d_gas_tcls);
-  cudaFree(ctx->d_gas_ellc);
-  cudaFree(ctx->d_gas_ellv);
-  cudaFree(ctx->d_gas_ellv32);
-  cudaFree(ctx->d_gas_ccls);
-  ctx->d_gas_rows = ctx->d_gas_coff = ctx->d_gas_cstr = ctx->d_gas_ellc = nullptr;
-  ctx->d_gas_off = nullptr;
-  ctx->d_gas_tcls = ctx->d_gas_ccls = nullptr;
-  ctx->d_gas_ellv = nullptr;
-  ctx->d_gas_ellv32 = nullptr;
+  ctx->d_gas_rows = nullptr;
+  gas_lists_release(ctx);
   ctx->gas_nrows = 0;
   for (int t = 0; t < 2; ++t) ctx->gas_pick[t] = ctx->gas_pick_mode[t] = -1;
   ctx->gas_on = false;
@@ -408,6 +412,66 @@ static void gas_release(forte_ctx *ctx) {
 }
 
 void gas_free(forte_ctx *ctx) { gas_release(ctx); }
+
+// Beta strings by class (ascending), and their lists by target class.  Where the memory
+// for them (16 bytes an entry of H_bb, 175 MB at 16 orbitals) cannot be had, there are no
+// lists.
+static int gas_lists(forte_ctx *ctx, const std::vector<int> &cls, const std::vector<long long> &cnt,
+                     const std::vector<uint8_t> &ok, int ncA) {
+  const SpinHost &B = ctx->sh[1];
+  const int n = ctx->n, ncB = (int)cnt.size();
+  if (!rows_alike(B.csr_ptr)) {  // before any kernel takes nnz entries from a row
+    set_error("internal: string Hamiltonian rows of different lengths");
+    return FORTE_ERR_ARG;
+  }
+  std::vector<int> coff(ncB + 1, 0), cstr(B.N);
+  for (int b = 0; b < ncB; ++b) coff[b + 1] = coff[b] + (int)cnt[b];
+  {
+    std::vector<int> at(coff.begin(), coff.end() - 1);
+    for (long long j = 0; j < B.N; ++j) cstr[at[cls[j]]++] = (int)j;
+  }
+  const int noB = ctx->nb * (n - ctx->nb), nnz = B.csr_ptr[1];
+  const size_t ell = (size_t)nnz * B.N;
+  std::vector<unsigned long long> okm(ncA, 0ull);
+  for (int a = 0; a < ncA; ++a)
+    for (int b = 0; b < ncB; ++b)
+      if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
+  DevTemp tmp;
+  int flag = 0;
+  if (dev_alloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)B.N * noB)) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_tcls, (size_t)ncB * noB + 1) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
+      dev_alloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || dev_alloc(&tmp.ptr, sizeof(int)) != cudaSuccess) {
+    gas_lists_release(ctx);
+    return FORTE_OK;
+  }
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size()));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size()));
+  FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_okm, okm.data(), sizeof(okm[0]) * okm.size()));
+  int *d_flag = (int *)tmp.ptr;
+  FORTE_CUDA_TRY(copy_in(ctx, d_flag, &flag, sizeof(int)));
+  const unsigned nbk = (unsigned)((B.N + 63) / 64);
+  k_gas_order<<<nbk, 64, 0, ctx->stream>>>(ctx->sd[1].off, noB, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col,
+                                           ctx->sd[1].csr_val, nnz, ctx->d_gas_cls[1], ncB, ctx->d_gas_coff,
+                                           ctx->d_gas_cstr, (int)B.N, ctx->d_gas_off, ctx->d_gas_tcls, ctx->d_gas_ellc,
+                                           ctx->d_gas_ellv, ctx->d_gas_ellv32, ctx->d_gas_ccls);
+  FORTE_LAUNCH_CHECK();
+  k_gas_check<<<nbk, 64, 0, ctx->stream>>>(ctx->d_gas_off, noB, ctx->d_gas_tcls, ctx->d_gas_ellc, nnz, ctx->d_gas_ccls,
+                                           ctx->d_gas_cls[1], ctx->d_gas_coff, ctx->d_gas_cstr, (int)B.N, d_flag);
+  FORTE_LAUNCH_CHECK();
+  FORTE_CUDA_TRY(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
+  FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  if (flag) {
+    set_error("internal: strings of one class differ in their replacements");
+    return FORTE_ERR_ARG;
+  }
+  return FORTE_OK;
+}
 
 int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const int *gmax, long long *ndet_out) {
   const int n = ctx->n;
@@ -507,62 +571,9 @@ int gas_set(forte_ctx *ctx, int nspace, const int *size, const int *gmin, const 
     ctx->gas_nrows = (long long)rowsv.size();
     ctx->gas_maxnnz = maxnnz;
   }
-  // beta strings by class (ascending), and their lists by target class
-  if (ncB <= GAS_MAXCLS) {
-    const SpinHost &B = ctx->sh[1];
-    std::vector<int> coff(ncB + 1, 0), cstr(B.N);
-    for (int b = 0; b < ncB; ++b) coff[b + 1] = coff[b] + (int)cnt[1][b];
-    {
-      std::vector<int> at(coff.begin(), coff.end() - 1);
-      for (long long j = 0; j < B.N; ++j) cstr[at[cls[1][j]]++] = (int)j;
-    }
-    const int noB = ctx->nb * (n - ctx->nb), nnz = B.csr_ptr[1];
-    const size_t ell = (size_t)nnz * B.N;
-    std::vector<unsigned long long> okm(ncA, 0ull);
-    for (int a = 0; a < ncA; ++a)
-      for (int b = 0; b < ncB; ++b)
-        if (ok[(size_t)a * ncB + b]) okm[a] |= 1ull << b;
-    if (!rows_alike(B.csr_ptr)) {  // before any kernel takes nnz entries from a row
-      gas_release(ctx);
-      set_error("internal: string Hamiltonian rows of different lengths");
-      return FORTE_ERR_ARG;
-    }
-    DevTemp tmp;
-    int flag = 0;
-    if (dev_alloc(&ctx->d_gas_coff, sizeof(int) * coff.size()) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_cstr, sizeof(int) * cstr.size()) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_okm, sizeof(okm[0]) * okm.size()) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_off, sizeof(uint32_t) * std::max<size_t>(1, (size_t)B.N * noB)) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_tcls, (size_t)ncB * noB + 1) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_ellc, sizeof(int) * ell) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_ellv, sizeof(double) * ell) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_ellv32, sizeof(float) * ell) != cudaSuccess ||
-        dev_alloc(&ctx->d_gas_ccls, (size_t)ncB * nnz) != cudaSuccess || dev_alloc(&tmp.ptr, sizeof(int)) != cudaSuccess) {
-      gas_release(ctx);
-      set_error("cudaMalloc of the restricted-sigma class lists failed");
-      return FORTE_ERR_ALLOC;
-    }
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_coff, coff.data(), sizeof(int) * coff.size()));
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_cstr, cstr.data(), sizeof(int) * cstr.size()));
-    FORTE_CUDA_TRY(copy_in(ctx, ctx->d_gas_okm, okm.data(), sizeof(okm[0]) * okm.size()));
-    int *d_flag = (int *)tmp.ptr;
-    FORTE_CUDA_TRY(copy_in(ctx, d_flag, &flag, sizeof(int)));
-    const unsigned nbk = (unsigned)((B.N + 63) / 64);
-    k_gas_order<<<nbk, 64, 0, ctx->stream>>>(ctx->sd[1].off, noB, ctx->sd[1].csr_ptr, ctx->sd[1].csr_col,
-                                             ctx->sd[1].csr_val, nnz, ctx->d_gas_cls[1], ncB, ctx->d_gas_coff,
-                                             ctx->d_gas_cstr, (int)B.N, ctx->d_gas_off, ctx->d_gas_tcls, ctx->d_gas_ellc,
-                                             ctx->d_gas_ellv, ctx->d_gas_ellv32, ctx->d_gas_ccls);
-    FORTE_LAUNCH_CHECK();
-    k_gas_check<<<nbk, 64, 0, ctx->stream>>>(ctx->d_gas_off, noB, ctx->d_gas_tcls, ctx->d_gas_ellc, nnz, ctx->d_gas_ccls,
-                                             ctx->d_gas_cls[1], ctx->d_gas_coff, ctx->d_gas_cstr, (int)B.N, d_flag);
-    FORTE_LAUNCH_CHECK();
-    FORTE_CUDA_TRY(cudaMemcpyAsync(&flag, d_flag, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
-    FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
-    if (flag) {
-      gas_release(ctx);
-      set_error("internal: strings of one class differ in their replacements");
-      return FORTE_ERR_ARG;
-    }
+  if (ncB <= GAS_MAXCLS && (rc = gas_lists(ctx, cls[1], cnt[1], ok, ncA))) {
+    gas_release(ctx);
+    return rc;
   }
   ctx->gas_nc[0] = ncA;
   ctx->gas_nc[1] = ncB;

@@ -1,7 +1,8 @@
 """A failed device allocation, at every place where a call makes one: the call reports it,
 the next call on the same context succeeds and launches the kernels of an undisturbed
 context with no table missing, and nothing is left allocated after the context is gone.
-Failed copies leave nothing allocated either.
+Failed copies leave nothing allocated either.  Memory that only the faster of two routes
+needs is not refused for: the other route serves the call.
 
 Runs on the CPU: the library's host code in a process of its own on a runtime that records
 launches and fails the allocation or copy it is told to (fake_cudart.cpp)."""
@@ -119,6 +120,40 @@ def gas(ctx):
     a = ctypes.c_int * 3
     return lib.forte_set_gas(ctx, 3, a(2, 2, 2), a(3, 0, 0), a(4, 4, 1), None)
 
+def test_gas(mode):
+    def kept_route():
+        ctx = setup(mode)
+        fg.forte_set_gas_route(ctx, 1)
+        return ctx
+
+    ctx = kept_route()
+    assert gas(ctx) == 0
+    log()
+    kept = (sigma(ctx), log())[1]
+    fg.forte_set_gas_route(ctx, 0)
+    grid = (sigma(ctx), log())[1]
+    lib.forte_destroy(ctx)
+    assert any("k_gas_sigma" in x for x in kept) and not any("k_gas_sigma" in x for x in grid)
+    served = 0
+    for k, ctx, r1, r2, _, _ in each_failure(kept_route, gas):
+        what = f"allocation {k}: "
+        assert r2 == 0, what + f"the next call returns {r2}: {fg.forte_last_error()}"
+        assert sigma(ctx) == 0 and log() == kept, what
+        lib.forte_destroy(ctx)
+        # the restriction that met the failure: refused, or served by the full grid
+        ctx = kept_route()
+        fake.fake_fail_at(k)
+        assert gas(ctx) == r1
+        if r1 == 0:
+            log()
+            assert sigma(ctx) == 0 and log() == grid, what
+            served += 1
+        else:
+            assert r1 in (fg.FORTE_ERR_ALLOC, fg.FORTE_ERR_CUDA), what + f"code {r1}"
+        lib.forte_destroy(ctx)
+        assert fake.fake_live() == 0, what + f"{fake.fake_live()} allocations left"
+    assert served == 10, f"served without {served} of the lists of the kept-determinant kernel"
+
 def test_gas_copies(mode):
     k = 0
     while True:
@@ -141,7 +176,7 @@ print("done")
 
 SMALL, TILED = (6, 3, 2), (11, 4, 5)  # orbitals, electrons: gathered and tiled FP64 sigma
 CALLS = ([("create", -1, SMALL), ("sigma", 0, TILED), ("rdm3", 0, SMALL)] + [("sigma", m, SMALL) for m in range(1, 5)] +
-         [("rdms", m, SMALL) for m in (0, 2)] + [("gas_copies", 0, SMALL)])
+         [("rdms", m, SMALL) for m in (0, 2)] + [("gas", 0, SMALL), ("gas_copies", 0, SMALL)])
 
 
 @pytest.fixture(scope="module")
