@@ -125,11 +125,13 @@ int forte_set_precision(forte_ctx *ctx, int mode);
  * ones: a sigma of up to 40 M products in FORTE_DF32, FORTE_OZ64 and the refinement of
  * FORTE_TF32 / FORTE_BF16X2 (spaces with the gathered FP64 kernels), the 2-RDM of up to
  * 80 M products in every such mode.
- *   -1  (default) the FP64 kernels; in place of tensor-core kernels (FORTE_OZ64 and the
- *       2-RDM) only while no wait budget of the caller's is set
+ *   -1  (default) the FP64 kernels, but not in place of tensor-core kernels (FORTE_OZ64
+ *       and the 2-RDM) while a wait budget below the default one is set: that is for
+ *       their waits (forte_set_wait_budget)
  *    0  the mode's own kernels at every size
  *    1  the FP64 kernels whatever the wait budget
- * FORTE_ERR_ARG for other values.
+ * Both kinds of kernels meet the error bounds of the mode; the last bits differ.  Clears
+ * the timings of the restricted sigma's routes.  FORTE_ERR_ARG for other values.
  * Control entry point: the paper has no counterpart.
  */
 int forte_set_small_route(forte_ctx *ctx, int route);
@@ -439,8 +441,11 @@ int forte_get_status(forte_ctx *ctx);
 
 /* Clock budget (cycles) of one pipeline wait of the context's tensor-core kernels;
  * 0 restores the default (4e9 cycles, about two seconds).  Meant for tests of the
- * failure path: a budget of a few cycles makes the waits expire.  Synchronises the
- * context stream.
+ * failure path: a budget of a few cycles makes the waits expire.  While a budget
+ * below the default is set, small spaces take the tensor-core kernels too
+ * (forte_set_small_route 0 or 1 fixes the kernels); a longer one changes no result.
+ * Clears the timings of the restricted sigma's routes and synchronises the context
+ * stream.
  * Control entry point: the paper has no counterpart.
  */
 int forte_set_wait_budget(forte_ctx *ctx, unsigned long long cycles);

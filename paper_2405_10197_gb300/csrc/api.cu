@@ -98,7 +98,7 @@ void sym_eig(int k, const double *A, double *w, double *U) {
 
 int err_word_setup(forte_ctx *ctx) {
   if (!ctx->d_err) FORTE_CUDA_TRY(dev_alloc(&ctx->d_err, 4 * sizeof(int)));
-  const unsigned long long b = ctx->wait_budget ? ctx->wait_budget : 4000000000ull;
+  const unsigned long long b = ctx->wait_budget ? ctx->wait_budget : WAIT_BUDGET_DEFAULT;
   const int w[4] = {0, 0, (int)(unsigned)(b & 0xFFFFFFFFull), (int)(unsigned)(b >> 32)};
   FORTE_CUDA_TRY(cudaMemcpyAsync(ctx->d_err, w, sizeof(w), cudaMemcpyHostToDevice, ctx->stream));
   FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
@@ -1177,6 +1177,7 @@ int forte_sa_energy(const forte_ctx *ctx, int nstates, const double *weights, do
 int forte_set_wait_budget(forte_ctx *ctx, unsigned long long cycles) {
   if (!ctx) { set_error("NULL context"); return FORTE_ERR_ARG; }
   ctx->wait_budget = cycles;
+  for (int t = 0; t < 2; ++t) ctx->gas_pick[t] = ctx->gas_pick_mode[t] = -1;  // as in forte_set_small_route
   return err_word_setup(ctx);
 }
 

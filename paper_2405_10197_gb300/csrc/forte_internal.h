@@ -80,6 +80,9 @@ inline bool rows_alike(const std::vector<int> &ptr) {
   return true;
 }
 
+// Clock cycles of one pipeline wait of the tensor-core kernels (about two seconds).
+constexpr unsigned long long WAIT_BUDGET_DEFAULT = 4000000000ull;
+
 // Device memory of a function's own.
 struct DevTemp {
   void *ptr = nullptr;
@@ -294,7 +297,7 @@ int sigma_fp64_scratch(forte_ctx *ctx, const double *C, double *S, int nvec, dou
 double fp64_products(const forte_ctx *ctx);
 bool fp64_small(const forte_ctx *ctx, int nvec);
 // Whether such a space takes the FP64 kernels (forte_set_small_route); waits: in place of
-// tensor-core kernels, whose waits a budget of the caller's is for
+// tensor-core kernels, whose waits a budget of the caller's cuts short
 bool small_route(const forte_ctx *ctx, bool waits);
 int hdiag_build(forte_ctx *ctx);
 // FP64-class sigma in double-FP32 arithmetic (relative error ~2^-46 per term);

@@ -327,7 +327,10 @@ bool fp64_small(const forte_ctx *ctx, int nvec) {
 }
 
 bool small_route(const forte_ctx *ctx, bool waits) {
-  return ctx->small_route == 1 || (ctx->small_route == -1 && !(waits && ctx->wait_budget));
+  // (a longer wait changes nothing but the time of a failure; a shorter one is for the
+  // kernels that wait, so they run)
+  const bool cut = ctx->wait_budget != 0 && ctx->wait_budget < WAIT_BUDGET_DEFAULT;
+  return ctx->small_route == 1 || (ctx->small_route == -1 && !(waits && cut));
 }
 
 // Columns per block: as many threads share an output as leave two blocks an SM busy, and

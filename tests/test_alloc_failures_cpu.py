@@ -9,36 +9,17 @@ launches and fails the allocation or copy it is told to (fake_cudart.cpp)."""
 import os
 import shutil
 import subprocess
-import sys
 
 import pytest
 
-HERE = os.path.dirname(os.path.abspath(__file__))
-ROOT = os.path.dirname(HERE)
+import fake_runtime as fr
 
 DRIVER = r"""
-import ctypes, math, sys
-import numpy as np
-import paper_2405_10197_gb300 as fg
-import synth_inputs as si
-
-fake = ctypes.CDLL(FAKE)
-fake.fake_log.restype = ctypes.c_char_p
-for f in (fake.fake_allocs, fake.fake_live):
-    f.restype = ctypes.c_longlong
-for f in (fake.fake_fail_at, fake.fake_fail_copy_at):
-    f.argtypes = [ctypes.c_longlong]
-lib = fg.library()
 N, NA, NB = map(int, sys.argv[3:6])
 h, eri = si.integrals(N, 2 * N, seed=1)
 C = np.zeros((2, math.comb(N, NA), math.comb(N, NB)))
 S = np.zeros_like(C)
 G = [np.zeros((N,) * k) for k in (2, 4, 6)]
-
-def log():
-    out = fake.fake_log().decode().split("\n")[:-1]
-    fake.fake_clear_log()
-    return out
 
 def create():
     return lib.forte_cas_create(N, NA, NB, h.ctypes.data, eri.ctypes.data)
@@ -171,7 +152,6 @@ def test_gas_copies(mode):
 
 name, mode = sys.argv[1], int(sys.argv[2])
 globals()["test_" + name](*([mode] if mode >= 0 else []))
-print("done")
 """
 
 SMALL, TILED = (6, 3, 2), (11, 4, 5)  # orbitals, electrons: gathered and tiled FP64 sigma
@@ -180,34 +160,23 @@ CALLS = ([("create", -1, SMALL), ("sigma", 0, TILED), ("rdm3", 0, SMALL)] + [("s
 
 
 @pytest.fixture(scope="module")
-def fake_runtime(tmp_path_factory):
-    from paper_2405_10197_gb300 import build
-    build.build()
-    inc = os.path.join(os.path.dirname(build._cuda_lib_dir(build._nvcc())), "include")
-    out = str(tmp_path_factory.mktemp("fake") / "libfake_cudart.so")
-    subprocess.run([shutil.which("g++"), "-shared", "-fPIC", "-std=c++17", "-I", inc,
-                    os.path.join(HERE, "fake_cudart.cpp"), "-o", out], check=True)
-    return out
+def fake(tmp_path_factory):
+    return fr.compile_fake(tmp_path_factory.mktemp("fake"))
 
 
 @pytest.mark.parametrize("call,mode,space", CALLS)
-def test_failed_allocations_are_reported_and_recovered_from(fake_runtime, call, mode, space):
-    code = f"FAKE = {fake_runtime!r}\n" + DRIVER
-    env = dict(os.environ, LD_PRELOAD=fake_runtime, PYTHONPATH=os.pathsep.join([ROOT, HERE]))
-    r = subprocess.run([sys.executable, "-c", code, call, *map(str, (mode, *space))], env=env, capture_output=True, text=True, timeout=300)
-    assert r.returncode == 0 and r.stdout.strip() == "done", r.stdout + r.stderr[-2000:]
+def test_failed_allocations_are_reported_and_recovered_from(fake, call, mode, space):
+    fr.run(fake, DRIVER, call, mode, *space)
 
 
 def test_rows_of_different_lengths_are_seen_before_they_are_read(tmp_path):
     """rows_alike guards the kernels that take as many entries from every row as the first has."""
-    from paper_2405_10197_gb300 import build
-    inc = os.path.join(os.path.dirname(build._cuda_lib_dir(build._nvcc())), "include")
     src = tmp_path / "rows.cpp"
     src.write_text('#include "forte_internal.h"\n#include <cstdio>\nint main() {\n'
                    '  for (const std::vector<int> &p : std::vector<std::vector<int>>{\n'
                    '           {0, 3}, {0, 3, 6, 9}, {0, 3, 6, 8}, {0, 2, 5, 8}, {0, 3, 7, 10}, {0, 0, 0}, {0, 0, 1}, {0}})\n'
                    '    printf("%d", (int)forte::rows_alike(p));\n}\n')
     exe = str(tmp_path / "rows")
-    subprocess.run([shutil.which("g++"), "-std=c++17", "-I", inc, "-I", os.path.join(ROOT, "paper_2405_10197_gb300", "csrc"),
+    subprocess.run([shutil.which("g++"), "-std=c++17", "-I", fr.include_dir(), "-I", os.path.join(fr.ROOT, "paper_2405_10197_gb300", "csrc"),
                     str(src), "-o", exe], check=True)
     assert subprocess.run([exe], capture_output=True, text=True, check=True).stdout == "11000101"
