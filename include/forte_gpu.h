@@ -362,9 +362,11 @@ int forte_rdm3(forte_ctx *ctx, const double *C, double *g3);
  * the solve an autotuner times, for every class, the per-CTA sigma for each
  * (threads per CTA, beta tile width) candidate and keeps the fastest; it then
  * times Davidson iterations of the class's first problem on the single-problem path
- * (FP64 ones in the mixed modes) and, with t_single_iteration the time per problem and
- * root (four fifths of the one measured alone: the workers overlap) and t_CTA_sigma the
- * time of one sigma build (double-FP32 in the mixed modes), sends the class there when
+ * (those on FP32 vectors in the mixed modes).  With t_single_iteration the time per
+ * problem and root, the measured one times 0.4 + 0.6 / min(P, 8) for the workers'
+ * overlap (and 0.72 in the mixed modes, whose solves take fewer iterations), and
+ * t_CTA_sigma the time of one sigma build (double-FP32 in the mixed modes), it sends the
+ * class there when
  *   P x t_single_iteration < t_CTA_sigma x ceil(P / (resident CTAs per SM x SMs)).
  * Problems with more than 100,000 determinants or more than 3 roots always take
  * the single-problem path.  forte_batch_tuning reports the choices.
@@ -389,11 +391,10 @@ int forte_batch_solve(int nprob, const int *norb, const int *nalpha, const int *
 /* Autotuner choices of the last forte_batch_solve, one entry per size class below
  * the in-CTA limits (host outputs of length max_classes, any may be NULL;
  * *nclass = number of classes): orbital and electron counts, threads per CTA,
- * beta tile width of the alpha-beta term, the measured time (ms) of one sigma
- * build of the class's first problems (one CTA each) with the chosen candidate,
- * the chosen path (0: class launch, 1: single-problem path), the measured time
- * (ms) of one single-problem-path Davidson iteration per root, the class's problem count
- * and the resident CTAs per SM of its launch.
+ * beta tile width of the alpha-beta term, t_CTA_sigma (ms): the measured time of one
+ * sigma build of the class's first problems (one CTA each) with the chosen candidate,
+ * the chosen path (0: class launch, 1: single-problem path), t_single_iteration (ms),
+ * the class's problem count and the resident CTAs per SM of its launch.
  * Control entry point: the paper has no counterpart.
  */
 int forte_batch_tuning(int max_classes, int *nclass, int *norb, int *nalpha, int *nbeta, int *threads, int *tile,

@@ -996,6 +996,27 @@ static int ensure_roots(forte_ctx *ctx, int nroots) {
   return FORTE_OK;
 }
 
+}  // extern "C"
+
+// The first iters Davidson-Liu iterations of a solve in the context's mode (FP32 vectors in
+// the reduced-precision modes), without the refinement: for timing.
+int forte::davidson_iterations(forte_ctx *ctx, int nroots, int iters) {
+  int rc = ensure_roots(ctx, nroots);
+  if (rc) return rc;
+  ctx->nroots_done = 0;
+  DvResult res;
+  const int mode = ctx->precision;
+  rc = mode == FORTE_TF32 || mode == FORTE_BF16X2
+           ? davidson_run<float>(ctx, nroots, 1e-14, mode, nullptr, 0, iters, ctx->d_roots, res)
+           : davidson_run<double>(ctx, nroots, 1e-14, mode, nullptr, 0, iters, ctx->d_roots, res);
+  if (rc) return rc;
+  if ((rc = mixed_status(ctx))) return rc;
+  FORTE_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  return FORTE_OK;
+}
+
+extern "C" {
+
 int forte_davidson(forte_ctx *ctx, int nroots, double tol) {
   if (!ctx) { set_error("NULL context"); return FORTE_ERR_ARG; }
   if (nroots < 1 || nroots > space_dim(ctx) || nroots > 31) { set_error("nroots out of range"); return FORTE_ERR_ARG; }

@@ -26,17 +26,17 @@
 // the per-CTA sigma runs once on the first problems of the class for every
 // candidate (threads per CTA x beta tile width of the alpha-beta term) that fits
 // in shared memory; the fastest candidate (CUDA events) is used for the solve
-// and reported by forte_batch_tuning.  It then times one Davidson iteration of
-// the class's first problem on the single-problem path (forte_cas_create /
-// forte_davidson, with the tensor-core sigma in the reduced-precision modes) and
-// sends the class there when P iterations of that path cost less than one class
-// sigma round (t_sigma x waves of resident CTAs).
+// and reported by forte_batch_tuning.  It then times Davidson iterations of the class's
+// first problem on the single-problem path (forte_cas_create / forte_davidson; on FP32
+// vectors in the reduced-precision modes) and sends the class there when an iteration of
+// each of its P problems costs less that way (single_path_ms in batch_rule.h) than one
+// class sigma round (t_sigma x waves of resident CTAs; double-FP32 in those modes).
 //
 // Problems with more than BT_MAX_DET determinants are large enough to occupy the
 // whole GPU on their own and always take the single-problem path.  (One CTA per
 // such problem would spend minutes per FP64 solve on one SM.)  The class launches
 // are captured into one graph and launched without waiting; the single-problem
-// path runs meanwhile on BT_WORKERS host threads with their own streams.
+// path runs meanwhile on BATCH_WORKERS host threads with their own streams.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -50,6 +50,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "batch_rule.h"
 #include "forte_internal.h"
 
 namespace forte {
@@ -63,7 +64,6 @@ constexpr int BT_LD = 37;                 // leading dimension of the small matr
 constexpr int BT_SEG = 512;               // CSR entries staged per pass
 constexpr long long BT_MAX_DET = 100000;  // larger problems take the single-problem path
 constexpr int BT_MAX_ROOTS = 3;
-constexpr int BT_WORKERS = 8;             // host threads of the single-problem path
 
 enum { AR_F64 = 0, AR_F32 = 1, AR_DF = 2 };
 
@@ -1114,35 +1114,27 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
       cudaStreamDestroy(sx);
     }
   };
-  // Host wall time (ms) per problem and root (sigma build) of one Davidson iteration on the
-  // single-problem path:
-  // problem i capped at 2 and at 6 iterations (the faster of two runs each) after a
-  // 1-iteration run that builds the lazy tables; (t6 - t2) / 4 leaves out the set-up
-  // and the first sigma builds and keeps the launch and host costs of an iteration.  The
-  // workers' overlap brings the time per problem down by a fifth (8 problems of 6 to 8
-  // orbitals at once on one GB300: 0.053 - 0.069 ms, alone 0.064 - 0.085 ms).  FP64
-  // iterations stand for those of a mixed mode, whose solves are of two kinds of
-  // iteration and take about as long (8 orbitals, one root: 26.9 ms FP64, 27.9 ms
-  // BF16x2; 10 orbitals: 43 against 30 ms).
-  auto single_iter_ms = [&](int i) -> double {
-    const int prec = precision == FORTE_TF32 || precision == FORTE_BF16X2 ? FORTE_FP64 : precision;
+  // Host wall time (ms) of one Davidson iteration of problem i, of a class of P, as
+  // single_path_ms counts it: capped at 2 and at 6 iterations (the faster of two runs each)
+  // after a 1-iteration run that builds the lazy tables; (t6 - t2) / 4 leaves out the
+  // set-up and the first sigma builds and keeps the launch and host costs of an iteration.
+  auto single_iter_ms = [&](int i, int P) -> double {
     forte_ctx *ctx = forte_cas_create(norb[i], nalpha[i], nbeta[i], h[i], eri[i]);
     if (!ctx) return INFINITY;
-    bool ok = forte_set_precision(ctx, prec) == FORTE_OK;
+    bool ok = forte_set_precision(ctx, precision) == FORTE_OK &&
+              forte_set_davidson_params(ctx, 12, 2, max_iter, 1e-8) == FORTE_OK;
     double t2 = INFINITY, t6 = INFINITY;
     for (int cap : {1, 2, 6, 2, 6}) {
-      if (!ok) break;
-      ok = forte_set_davidson_params(ctx, 12, 2, cap, 1e-8) == FORTE_OK;
       const auto t0 = std::chrono::steady_clock::now();
-      const int rc = ok ? forte_davidson(ctx, nroots[i], 1e-14) : FORTE_ERR_ARG;
+      ok = ok && davidson_iterations(ctx, nroots[i], cap) == FORTE_OK;
       const double t = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
       if (cap == 2) t2 = std::min(t2, t);
       if (cap == 6) t6 = std::min(t6, t);
-      ok = (rc == FORTE_OK || rc == FORTE_ERR_NOT_CONVERGED);
     }
     forte_destroy(ctx);
     clear_error();
-    return ok ? std::max(1e-3, 0.8 * (t6 - t2) / (4.0 * nroots[i])) : INFINITY;
+    const bool mixed = precision == FORTE_TF32 || precision == FORTE_BF16X2;
+    return ok ? std::max(1e-3, single_path_ms((t6 - t2) / 4.0, nroots[i], mixed, P)) : INFINITY;
   };
 
   // ---- one pooled device allocation for the batch
@@ -1272,7 +1264,10 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
     ch.dev.TJ = ch.TJ;
     ch.dev.probe = 0;
     // path: one class launch costs about probe_ms per sigma round for every wave of
-    // resident CTAs; the single-problem path costs single_iter_ms per problem
+    // resident CTAs; the single-problem path costs single_iter_ms per problem.  Measured on
+    // one GB300 (ms of the solve, class launch / single path): FP64, 24 problems of 5, 6
+    // and 7 orbitals 32 / 61, 71 / 65, 269 / 81; 96 of 7 270 / 335; BF16x2, 24 of 6, 7 and 8
+    // 63 / 87, 134 / 120, 332 / 126
     int per_sm = 0;
     cudaError_t oe = cudaSuccess;
     const size_t smem = class_smem(ch.dev, ar, ch.TJ);
@@ -1282,7 +1277,7 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
     if (oe != cudaSuccess || per_sm < 1) per_sm = 1;
     const int P = ch.dev.P;
     const double waves = std::ceil((double)P / (double)(per_sm * nsm));
-    ch.single_ms = single_iter_ms(ch.probs[0]);
+    ch.single_ms = single_iter_ms(ch.probs[0], P);
     ch.path = (best * waves <= (double)P * ch.single_ms) ? 0 : 1;
     std::lock_guard<std::mutex> lock(g_tune_mu);
     g_tune.push_back(TuneRecord{ch.n, ch.na, ch.nb, ch.NT, ch.TJ, best, ch.path, ch.single_ms, P, per_sm});
@@ -1335,7 +1330,7 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
   }
   {
     std::vector<std::thread> workers;
-    for (int w = 0; w < std::min<int>(BT_WORKERS, (int)singles.size()); ++w) workers.emplace_back(single_worker);
+    for (int w = 0; w < std::min<int>(BATCH_WORKERS, (int)singles.size()); ++w) workers.emplace_back(single_worker);
     for (auto &x : workers) x.join();
   }
   if (!launched.empty()) {
@@ -1370,7 +1365,7 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
       singles = retry;
       next_single = 0;
       std::vector<std::thread> workers;
-      for (int w = 0; w < std::min<int>(BT_WORKERS, (int)singles.size()); ++w) workers.emplace_back(single_worker);
+      for (int w = 0; w < std::min<int>(BATCH_WORKERS, (int)singles.size()); ++w) workers.emplace_back(single_worker);
       for (auto &x : workers) x.join();
     }
     n_retried = (int)retry.size();

@@ -387,6 +387,7 @@ int gas_sigma(forte_ctx *ctx, const float *C, float *S, int nvec);
 long long space_dim(const forte_ctx *ctx);           // dimension of the space Davidson works in
 int det_mask_fill(forte_ctx *ctx, double *x, int nvec, double value);  // value at the masked-out entries
 int sigma_grid(forte_ctx *ctx, const double *C, double *S, int nvec);  // api.cu: unrestricted FP64-class sigma
+int davidson_iterations(forte_ctx *ctx, int nroots, int iters);        // api.cu: for timing
 
 // aci.cu: adaptive CI on the determinant grid
 int aci_run(forte_ctx *ctx, double sigma, double gamma, int max_cycles, double tol, int parity, double *E_out,
