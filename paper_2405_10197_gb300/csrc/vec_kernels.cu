@@ -329,8 +329,9 @@ __global__ void k_nonfinite(const double *__restrict__ x, long long n, int *flag
 // meet in shared memory, where 4 threads add one column (64 values), instead of a
 // five-step warp reduction per column.  Elements are loaded singly, so any count and
 // alignment will do.  FP64 vectors only: the FP32 ones of the reduced-precision phase keep
-// the kernels above and below, whose order of sums its rounding follows.  One GB300, CAS(8,8) FP64 solve (133 iterations): residual pass 31 ->
-// 14 us, 11-vector dots 22 -> 9 us, whole solve 18.9 -> 14.0 ms.
+// the kernels above and below, whose order of sums its rounding follows.  One GB300,
+// CAS(8,8) FP64 solve (133 iterations): residual pass 31 -> 14 us, 11-vector dots 22 ->
+// 9 us, whole solve 18.9 -> 14.0 ms.
 constexpr int VS_T = 64;
 constexpr int VS_E = 2;
 constexpr long long VS_CHUNK = VS_T * VS_E;
@@ -360,52 +361,50 @@ __device__ __forceinline__ void vs_columns(VsRed &r, int c0, int nc, int m, doub
 }
 
 // part[block][col0 + i] = sum over the chunk of V_i . x, i < nv (m columns in all).
-template <typename T>
-__device__ __forceinline__ void vs_dots(VsRed &r, const T *__restrict__ V, int nv, long long ld, const T (&x)[VS_E],
+__device__ __forceinline__ void vs_dots(VsRed &r, const double *__restrict__ V, int nv, long long ld, const double (&x)[VS_E],
                                         long long j0, long long n, int col0, int m, double *part) {
   for (int i0 = 0; i0 < nv; i0 += VS_COLS) {
     const int nc = min(VS_COLS, nv - i0);
 #pragma unroll 4
     for (int i = 0; i < nc; ++i) {
-      const T *v = V + (long long)(i0 + i) * ld;
-      T a = 0;
+      const double *v = V + (long long)(i0 + i) * ld;
+      double a = 0;
 #pragma unroll
       for (int e = 0; e < VS_E; ++e)
         if (j0 + e * VS_T < n) a += v[j0 + e * VS_T] * x[e];
-      r.v[i][threadIdx.x] = (double)a;
+      r.v[i][threadIdx.x] = a;
     }
     vs_columns(r, col0 + i0, nc, m, part);
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(VS_T) k_multidot_s(const T *__restrict__ V, int nv, long long ld,
-                                                     const T *__restrict__ x, long long n, double *__restrict__ part,
+__global__ void __launch_bounds__(VS_T) k_multidot_s(const double *__restrict__ V, int nv, long long ld,
+                                                     const double *__restrict__ x, long long n, double *__restrict__ part,
                                                      double *__restrict__ out, unsigned *counter) {
   __shared__ VsRed r;
   const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
-  T xr[VS_E];
+  double xr[VS_E];
 #pragma unroll
-  for (int e = 0; e < VS_E; ++e) xr[e] = j0 + e * VS_T < n ? x[j0 + e * VS_T] : T(0);
+  for (int e = 0; e < VS_E; ++e) xr[e] = j0 + e * VS_T < n ? x[j0 + e * VS_T] : 0.0;
   vs_dots(r, V, nv, ld, xr, j0, n, 0, nv, part);
   last_block_lanes(part, nv, out, counter);
 }
 
 // As k_orth_update_p: t_out = scale (t_in - B c), out = [B^T t_out (zeros unless DOTS), |t_out|^2].
-template <typename T, bool DOTS>
-__global__ void __launch_bounds__(VS_T) k_orth_update_s(const T *__restrict__ B, int k, long long ld,
-                                                        const double *__restrict__ c, const T *t_in, T *t_out,
+template <bool DOTS>
+__global__ void __launch_bounds__(VS_T) k_orth_update_s(const double *__restrict__ B, int k, long long ld,
+                                                        const double *__restrict__ c, const double *t_in, double *t_out,
                                                         long long n, double scale, double *__restrict__ part,
                                                         double *__restrict__ out, unsigned *counter) {
   __shared__ VsRed r;
-  __shared__ T sc[VK_MAXV];
+  __shared__ double sc[VK_MAXV];
   const int ku = c ? k : 0;
-  for (int i = threadIdx.x; i < ku; i += VS_T) sc[i] = (T)c[i];
+  for (int i = threadIdx.x; i < ku; i += VS_T) sc[i] = c[i];
   __syncthreads();
   const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
-  T t[VS_E], nn = 0;
+  double t[VS_E], nn = 0;
 #pragma unroll
-  for (int e = 0; e < VS_E; ++e) t[e] = j0 + e * VS_T < n ? t_in[j0 + e * VS_T] : T(0);
+  for (int e = 0; e < VS_E; ++e) t[e] = j0 + e * VS_T < n ? t_in[j0 + e * VS_T] : 0.0;
 #pragma unroll 4
   for (int i = 0; i < ku; ++i)
 #pragma unroll
@@ -414,11 +413,11 @@ __global__ void __launch_bounds__(VS_T) k_orth_update_s(const T *__restrict__ B,
 #pragma unroll
   for (int e = 0; e < VS_E; ++e)
     if (j0 + e * VS_T < n) {
-      if (scale != 1.0) t[e] *= (T)scale;
+      if (scale != 1.0) t[e] *= scale;
       t_out[j0 + e * VS_T] = t[e];
       nn += t[e] * t[e];
     }
-  r.v[0][threadIdx.x] = (double)nn;
+  r.v[0][threadIdx.x] = nn;
   vs_columns(r, k, 1, k + 1, part);
   if (DOTS) {
     vs_dots(r, B, k, ld, t, j0, n, 0, k + 1, part);
@@ -429,19 +428,19 @@ __global__ void __launch_bounds__(VS_T) k_orth_update_s(const T *__restrict__ B,
 }
 
 // As k_residual_precond_p: t = r / (theta - H_II), out = [|r|^2 (, B^T t, |t|^2)].
-template <typename T, bool DOTS>
-__global__ void __launch_bounds__(VS_T) k_residual_precond_s(const T *__restrict__ B, const T *__restrict__ S, int k,
+template <bool DOTS>
+__global__ void __launch_bounds__(VS_T) k_residual_precond_s(const double *__restrict__ B, const double *__restrict__ S, int k,
                                                              long long ld, const double *__restrict__ u, double theta,
                                                              const double *__restrict__ hd, double guard,
-                                                             T *__restrict__ t, long long n, double *__restrict__ part,
+                                                             double *__restrict__ t, long long n, double *__restrict__ part,
                                                              double *__restrict__ out, unsigned *counter) {
   __shared__ VsRed r;
-  __shared__ T su[VK_MAXV];
+  __shared__ double su[VK_MAXV];
   const int m = DOTS ? k + 2 : 1;
-  for (int i = threadIdx.x; i < k; i += VS_T) su[i] = (T)u[i];
+  for (int i = threadIdx.x; i < k; i += VS_T) su[i] = u[i];
   __syncthreads();
   const long long j0 = (long long)blockIdx.x * VS_CHUNK + threadIdx.x;
-  T hx[VS_E], xv[VS_E], rr = 0, tt = 0;
+  double hx[VS_E], xv[VS_E], rr = 0, tt = 0;
 #pragma unroll
   for (int e = 0; e < VS_E; ++e) hx[e] = xv[e] = 0;
 #pragma unroll 4
@@ -455,18 +454,18 @@ __global__ void __launch_bounds__(VS_T) k_residual_precond_s(const T *__restrict
 #pragma unroll
   for (int e = 0; e < VS_E; ++e)
     if (j0 + e * VS_T < n) {
-      const T res = hx[e] - (T)theta * xv[e];
+      const double res = hx[e] - theta * xv[e];
       rr += res * res;
       double den = theta - hd[j0 + e * VS_T];
       if (fabs(den) < guard) den = (den >= 0.0) ? guard : -guard;
-      hx[e] = res / (T)den;  // hx now holds t
+      hx[e] = res / den;  // hx now holds t
       tt += hx[e] * hx[e];
       t[j0 + e * VS_T] = hx[e];
     }
-  r.v[0][threadIdx.x] = (double)rr;
+  r.v[0][threadIdx.x] = rr;
   vs_columns(r, 0, 1, m, part);
   if (DOTS) {
-    r.v[0][threadIdx.x] = (double)tt;
+    r.v[0][threadIdx.x] = tt;
     vs_columns(r, k + 1, 1, m, part);
     vs_dots(r, B, k, ld, hx, j0, n, 1, m, part);
   }
@@ -1263,9 +1262,9 @@ static int vk_multidot_t(forte_ctx *ctx, const T *V, int nv, long long ld, const
   int rc = part_buffer(ctx, (size_t)nb * nv, &part, &cnt);
   if (rc) return rc;
   FORTE_PROF(ctx, "multidot");
-  if (vs)
-    k_multidot_s<T><<<nb, VS_T, 0, ctx->stream>>>(V, nv, ld, x, n, part, out, cnt);
-  else if (pk && nv <= 4)
+  if (vs) {
+    if constexpr (sizeof(T) == 8) k_multidot_s<<<nb, VS_T, 0, ctx->stream>>>(V, nv, ld, x, n, part, out, cnt);
+  } else if (pk && nv <= 4)
     k_multidot_u<T, 4><<<nb, VK_THREADS, 0, ctx->stream>>>(V, nv, ld, x, n / Pk<T>::P, part, out, cnt);
   else if (pk && nv <= 8)
     k_multidot_u<T, 8><<<nb, VK_THREADS, 0, ctx->stream>>>(V, nv, ld, x, n / Pk<T>::P, part, out, cnt);
@@ -1326,12 +1325,14 @@ static int vk_residual_precond_t(forte_ctx *ctx, const T *B, const T *S, int k, 
       k_residual_precond_u<T, false, 2, KM><<<nb, VK_THREADS, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, \
                                                                                 npk, part, rnorm2, cnt);             \
   } while (0)
-  if (vs && dots)
-    k_residual_precond_s<T, true><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, dots, cnt);
-  else if (vs)
-    k_residual_precond_s<T, false><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, rnorm2,
-                                                                 cnt);
-  else if (pk && k <= 4)
+  if (vs) {
+    if constexpr (sizeof(T) == 8) {
+      if (dots)
+        k_residual_precond_s<true><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, dots, cnt);
+      else
+        k_residual_precond_s<false><<<nb, VS_T, 0, ctx->stream>>>(B, S, k, ld, u, theta, hd, guard, t, n, part, rnorm2, cnt);
+    }
+  } else if (pk && k <= 4)
     FORTE_RESID_U(4);
   else if (pk && k <= 8)
     FORTE_RESID_U(8);
@@ -1389,11 +1390,14 @@ static int vk_orth_update_t(forte_ctx *ctx, const T *B, int k, long long ld, con
       k_orth_update_u<T, false, KM><<<nb, VK_THREADS, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, npk,      \
                                                                         scale, part, dots_out, cnt);        \
   } while (0)
-  if (vs && dots)
-    k_orth_update_s<T, true><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
-  else if (vs)
-    k_orth_update_s<T, false><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
-  else if (pk && k <= 4)
+  if (vs) {
+    if constexpr (sizeof(T) == 8) {
+      if (dots)
+        k_orth_update_s<true><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
+      else
+        k_orth_update_s<false><<<nb, VS_T, 0, ctx->stream>>>(B, k, ld, c, t_in, t_out, n, scale, part, dots_out, cnt);
+    }
+  } else if (pk && k <= 4)
     FORTE_ORTH_U(4);
   else if (pk && k <= 8)
     FORTE_ORTH_U(8);
