@@ -654,7 +654,7 @@ static int refine_jd(forte_ctx *ctx, int nroots, double tol, int inner_mode, int
   }
   if ((rc = sigma_dispatch(ctx, V, HV, nroots, outer_mode))) return rc;
   std::vector<double> prev_rn(nroots, INFINITY);
-  std::vector<int> slow(nroots, 0);  // outer steps running that did not halve a root's residual
+  std::vector<int> slow(nroots, 0);  // outer steps that did not halve a root's residual
   int k = nroots;
   std::vector<double> G, Gk, w, U, coef, h(66);
   res.E.assign(nroots, 0.0);
@@ -699,17 +699,23 @@ static int refine_jd(forte_ctx *ctx, int nroots, double tol, int inner_mode, int
       if (!(res.rn[r] < tol)) all = false;
     }
     res.iters = outer;
-    // A root whose residual has not halved in JD_SLOW outer steps running: the
+    // A root whose residual has not halved in JD_SLOW outer steps, running or not: the
     // reduced-precision inner operator no longer resolves its correction, and its inner
-    // solves take the outer one.  (One slow step is no sign of that: it is the rule for
-    // the uppermost root when the next state is close, and passes.  Measured on
-    // CAS(12,12), 3 roots: 201 FP64-class sigmas and 414 ms when any slow step switched
-    // every root, 21 and 231 ms without, the same outer steps and residuals.)
+    // solves take the outer one, with the steps that told so on top of max_outer.  One
+    // slow step is no sign of that: it is the rule for the uppermost root when the next
+    // state is close, and passes.  Measured on one GB300, when any slow step switches every
+    // root / so: CAS(12,12), 3 roots, 6 problems: one of them 201 / 21 FP64-class sigmas,
+    // 408 / 222 ms, the others alike; 11 orbitals, 2 roots, TF32: one of 6 474 / 25 sigmas,
+    // 313 / 170 ms; 6 to 8 orbitals, 64 problems: 1930 / 777 sigmas, the same time.  64
+    // problems with integrals of 1e5 Eh, where the inner operator does fail: 1 not
+    // converged / 7 when only slow steps in a row counted.
+    int spent = 0;
     for (int r = 0; r < nroots; ++r) {
-      if (slow[r] < JD_SLOW) slow[r] = res.rn[r] >= tol && res.rn[r] > 0.5 * prev_rn[r] ? slow[r] + 1 : 0;
+      if (res.rn[r] >= tol && res.rn[r] > 0.5 * prev_rn[r]) ++slow[r];
+      if (slow[r] >= JD_SLOW && inner_mode != outer_mode) spent = JD_SLOW - 1;
       prev_rn[r] = res.rn[r];
     }
-    if (all || outer >= max_outer) {
+    if (all || outer >= max_outer + spent) {
       FORTE_CUDA_TRY(cudaMemcpyAsync(out, V, sizeof(double) * nroots * N, cudaMemcpyDeviceToDevice, st));
       res.converged = all;
       return FORTE_OK;
