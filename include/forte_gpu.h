@@ -363,7 +363,7 @@ int forte_rdm3(forte_ctx *ctx, const double *C, double *g3);
  * (threads per CTA, beta tile width) candidate and keeps the fastest; it then
  * times Davidson iterations of the class's first problem on the single-problem path
  * (those on FP32 vectors in the mixed modes).  With t_single_iteration the time per
- * problem and root, the measured one times 0.4 + 0.6 / min(P, 8) for the workers'
+ * problem and root, the measured one times 0.35 + 0.65 / min(P, 8) for the workers'
  * overlap (and 0.72 in the mixed modes, whose solves take fewer iterations), and
  * t_CTA_sigma the time of one sigma build (double-FP32 in the mixed modes), it sends the
  * class there when
