@@ -1115,16 +1115,19 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
     }
   };
   // Host wall time (ms) of one Davidson iteration of problem i, of a class of P, as
-  // single_path_ms counts it: capped at 2 and at 6 iterations (the faster of two runs each)
+  // single_path_ms counts it: capped at 2 and at 6 iterations (FP64: the faster of two runs each)
   // after a 1-iteration run that builds the lazy tables; (t6 - t2) / 4 leaves out the
   // set-up and the first sigma builds and keeps the launch and host costs of an iteration.
   auto single_iter_ms = [&](int i, int P) -> double {
+    const bool mixed = precision == FORTE_TF32 || precision == FORTE_BF16X2;
     forte_ctx *ctx = forte_cas_create(norb[i], nalpha[i], nbeta[i], h[i], eri[i]);
     if (!ctx) return INFINITY;
     bool ok = forte_set_precision(ctx, precision) == FORTE_OK &&
               forte_set_davidson_params(ctx, 12, 2, max_iter, 1e-8) == FORTE_OK;
     double t2 = INFINITY, t6 = INFINITY;
-    for (int cap : {1, 2, 6, 2, 6}) {
+    const int caps[5] = {1, 2, 6, 2, 6};
+    for (int c = 0; c < (mixed ? 3 : 5); ++c) {  // (mixed iterations take about twice as long: one run each)
+      const int cap = caps[c];
       const auto t0 = std::chrono::steady_clock::now();
       ok = ok && davidson_iterations(ctx, nroots[i], cap) == FORTE_OK;
       const double t = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -1133,7 +1136,6 @@ extern "C" int forte_batch_solve(int nprob, const int *norb, const int *nalpha, 
     }
     forte_destroy(ctx);
     clear_error();
-    const bool mixed = precision == FORTE_TF32 || precision == FORTE_BF16X2;
     return ok ? std::max(1e-3, single_path_ms((t6 - t2) / 4.0, nroots[i], mixed, P)) : INFINITY;
   };
 
