@@ -810,7 +810,7 @@ def run_configs(args):
 
 def run_extensions(args):
     """One JSON line per extension of the path: X1 the spin-free 3-RDM (FP64 Gram
-    work 2 n^6 N_det), X2 an occupation-restricted CAS(14,14) (RAS: at most two
+    work n^6 N_det / 6), X2 an occupation-restricted CAS(14,14) (RAS: at most two
     holes in the lowest four orbitals and two particles in the highest four) and
     X3 the even-S sector of CAS(14,14), each against the unrestricted solve."""
     import torch

@@ -284,7 +284,10 @@ int forte_set_davidson_params(forte_ctx *ctx, int max_subspace_per_root, int col
 
 /* Results of the last forte_davidson: energies (host [nroots], may be NULL),
  * eigenvectors (device [nroots][N_alpha][N_beta], may be NULL; normalised,
- * largest-|c| component positive), final FP64 residual norms (host
+ * largest-|c| component positive: where several components share the largest
+ * magnitude, as in high-spin states and mirror pairs I_alpha <-> I_beta, which of
+ * them is the larger one after rounding decides the sign, and that can change with
+ * the precision mode or a later version of the kernels), final FP64 residual norms (host
  * [nroots], may be NULL) and the iteration count (host, may be NULL).
  * Paper: Sec. II.A.1 (Davidson-Liu results).
  */

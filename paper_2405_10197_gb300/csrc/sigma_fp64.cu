@@ -318,10 +318,13 @@ double fp64_products(const forte_ctx *ctx) {
   return (double)ctx->Ndet * (ka * kb + (double)A.csr_ptr[1] + (double)B.csr_ptr[1]);
 }
 
-// The small-space FP64 kernels against the double-FP32 / digit-slice ones (one GB300, one
-// vector): 9.4 M products (9 orbitals, 5 + 4) 46 us against 75 / 110 us, 59 M (10, 5 + 5)
-// 184 against 140 / 187 us; four vectors 108 against 135 / 227 and 627 against 351 /
-// 486 us.  The line lies at 40 M in all.
+// The small-space FP64 kernels against the double-FP32 / digit-slice ones, us on one GB300:
+// 9.6 M products (9 orbitals, 5 + 4) 48 against 85 / 139, 38 M (four vectors of it) 100
+// against 119 / 242, 59 M (10, 5 + 5) 166 against 144 / 223, 236 M 579 against 275 / 472.
+// The line is where FP64 and double-FP32 meet, and serves the digit-slice mode too, whose
+// own crossing with FP64 lies at about 100 M.  Between 40 M and some 4 G products that mode
+// is slower than the double-FP32 one (188 M 406 against 276, 1.6 G 1257 against 1246, 5.4 G
+// 2988 against 3517): FORTE_OZ64 runs the kernels it names all the same.
 bool fp64_small(const forte_ctx *ctx, int nvec) {
   return ctx->sd[1].ell_col && fp64_products(ctx) * nvec <= 40e6;
 }
